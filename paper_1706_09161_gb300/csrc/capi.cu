@@ -513,9 +513,7 @@ static int create_problem(const lbm_params* prm, const double* C0_host, void* st
   const long long nodes = h->sp.nodes;
   const size_t E = h->elem;
   if (prm->precision == LBM_FP32 && !batched) {
-    // small FP32 problems: the SIMT operator's contraction split (F holds the partials)
-    h->sp.ksum = lbm::simt_ksplit(h);
-    h->sp.pstride = h->sp.ksum > 1 ? (long long)h->d * nodes : 0;
+    h->simt_ks = lbm::simt_ksplit(h);  // small FP32 problems: the SIMT operator's contraction split
   }
   long long ksz = 0;
   for (int mu = 0; mu < h->d; ++mu) ksz += (long long)prm->grid[mu] * prm->grid[mu];
@@ -524,8 +522,7 @@ static int create_problem(const lbm_params* prm, const double* C0_host, void* st
   if ((rc = alloc_bytes(h, &h->dev.f[1], E * h->Q * nodes))) return fail(rc);
   if ((rc = alloc_bytes(h, &h->dev.C, E * nodes))) return fail(rc);
   if ((rc = alloc_bytes(h, &h->dev.C0, E * nodes))) return fail(rc);
-  if ((rc = alloc_bytes(h, &h->dev.F, E * h->d * nodes * h->sp.ksum))) return fail(rc);
-  h->f_elems = (size_t)h->d * nodes * h->sp.ksum;
+  if ((rc = alloc_bytes(h, &h->dev.F, E * h->d * nodes))) return fail(rc);
   if ((rc = alloc_bytes(h, &h->dev.K, E * ksz))) return fail(rc);
   if ((rc = alloc_bytes(h, &h->dev.KT, E * ksz))) return fail(rc);
   if ((rc = alloc_bytes(h, (void**)&h->dev.stage, sizeof(double) * (size_t)(nodes > ksz ? nodes : ksz)))) return fail(rc);
@@ -912,27 +909,14 @@ struct TuneCfg {
 };
 
 // FP32 SIMT operator of a single problem: contraction split ks (1, 2, 4 or 8, at most
-// the contraction blocks of 32 of the shortest axis); F grows to ks partial sums and the
-// collide-stream tensor maps are re-encoded for it
+// the contraction blocks of 32 of the shortest axis)
 int simt_replan(lbm_s* h, int ks) {
   if (!(ks == 1 || ks == 2 || ks == 4 || ks == 8)) return LBM_EINVAL;
   int kbmin = 1 << 30;
   for (int mu = 0; mu < h->d; ++mu) kbmin = std::min(kbmin, (h->sp.n[mu] + 31) / 32);
   if (ks > kbmin) return LBM_EINVAL;
-  const size_t need = (size_t)ks * h->d * h->sp.nodes;
-  if (need > h->f_elems) {
-    LBM_CUDA(cudaStreamSynchronize(h->stream));
-    lbm::dev_free(h, h->dev.F);
-    h->dev.F = nullptr;
-    h->f_elems = 0;
-    const int rc = alloc_bytes(h, &h->dev.F, need * sizeof(float));
-    if (rc) return rc;
-    h->f_elems = need;
-  }
-  h->sp.ksum = ks;
-  h->sp.pstride = ks > 1 ? (long long)h->d * h->sp.nodes : 0;
-  lbm::cs_release(h);
-  return lbm::cs_prepare(h);
+  h->simt_ks = ks;
+  return LBM_OK;
 }
 
 // the handle's launch configuration set to c (operator plan for tensor-core handles, the
@@ -1020,7 +1004,7 @@ int lbm_configure(lbm_t h, int bn, int ks, int persist, int chunk, int fused) {
       c.persist = persist ? 1 : 0;
     }
   } else if (!h->is_batch() && h->elem == 4 && bn == 0 && !persist && !fused) {
-    c.ks = ks > 0 ? ks : h->sp.ksum;  // FP32 SIMT operator: its contraction split only
+    c.ks = ks > 0 ? ks : h->simt_ks;  // FP32 SIMT operator: its contraction split only
   } else if (bn > 0 || ks > 0 || persist || fused) {
     return LBM_EINVAL;  // no tensor-core operator to plan
   }
@@ -1038,7 +1022,7 @@ int lbm_autotune(lbm_t h, int nsteps, char* desc, int desc_len) {
   TuneCfg cur{0, 0, 0, h->cs_chunk > 0 ? h->cs_chunk : lbm::cs_chunk_default(h), h->fused ? 1 : 0};
   if (!h->is_batch() && h->tc) lbm::tc_config(h, &cur.bn, &cur.ks, &cur.persist);
   const bool simt32 = !h->is_batch() && !h->tc && h->elem == 4;  // FP32 SIMT operator
-  if (simt32) cur.ks = h->sp.ksum;
+  if (simt32) cur.ks = h->simt_ks;
   // candidate chunks
   std::vector<int> chunks;
   if (h->is_batch()) {

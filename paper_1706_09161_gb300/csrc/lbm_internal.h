@@ -103,7 +103,7 @@ struct lbm_s {
   cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};
   int graph_steps = 0;                 // steps per captured graph (even)
   int launches_per_step = 0;
-  size_t f_elems = 0;                  // capacity of dev.F (elements) for the SIMT operator's partials
+  int simt_ks = 1;                     // contraction split of the FP32 SIMT operator (blocks per cluster)
   // programmatic dependent launch between the operator and collide-stream: only when both
   // grids run in a single wave (measured: with multi-wave 3-D grids it costs ~30%)
   bool pdl = false;
@@ -164,8 +164,8 @@ void dev_free(const lbm_s* h, void* p);
 // ---- kernels (launchers return cudaGetLastError of the launch)
 // fractional operator, SIMT: F_mu = K_mu applied along axis mu, for all mu
 cudaError_t launch_frac_simt(const lbm_s* h, const void* C, void* F, cudaStream_t s);
-// contraction split of the FP32 SIMT operator for a single problem: F then holds that
-// many partial sums ([rank][axis][node], like the tensor-core split), 1 for FP64
+// contraction split of the FP32 SIMT operator for a single problem (a cluster of that many
+// blocks adds its partial tiles), 1 for FP64
 int simt_ksplit(const lbm_s* h);
 // the FP32 SIMT operator's grid is resident at once (programmatic dependent launch)
 bool simt_one_wave(const lbm_s* h);
