@@ -320,7 +320,7 @@ void free_all(lbm_s* h) {
 // from the collide-stream kernel itself)
 bool pdl_fits(const lbm_s* h) {
   if (h->is_batch()) return false;
-  if (!h->tc) return h->elem == 4 && lbm::cs_one_wave(h) && lbm::simt_one_wave(h);  // FP32 SIMT operator
+  if (!h->tc) return lbm::cs_one_wave(h) && lbm::simt_one_wave(h);  // SIMT operator
   const bool adjacent = lbm::bf16_parts(h->prm.precision) || lbm::cs_writes_T(h);
   // the field march's grid is not the one cs_one_wave describes: no early launch there
   return adjacent && !h->fld.on && lbm::cs_one_wave(h) && lbm::tc_one_wave(h);
@@ -529,9 +529,8 @@ static int create_problem(const lbm_params* prm, const double* C0_host, void* st
   if ((rc = alloc_bytes(h, (void**)&h->dev.partials, sizeof(double) * h->reduce_blocks))) return fail(rc);
   if ((rc = alloc_bytes(h, (void**)&h->dev.scalar, sizeof(double)))) return fail(rc);
   if ((rc = alloc_bytes(h, (void**)&h->dev.flag, sizeof(int)))) return fail(rc);
-  // kMassSlots mass partials per collide-stream block: at most one block per 32 x 16 tile and plane
-  h->cs_part_cap = (long long)((prm->grid[0] + 31) / 32) * ((prm->grid[1] + 15) / 16) * prm->grid[2];
-  if ((rc = alloc_bytes(h, (void**)&h->cs_part, sizeof(double) * lbm::kMassSlots * h->cs_part_cap))) return fail(rc);
+  h->cs_part_cap = lbm::cs_max_parts(h);
+  if ((rc = alloc_bytes(h, (void**)&h->cs_part, sizeof(double) * h->cs_part_cap))) return fail(rc);
   if (cudaMemsetAsync(h->dev.flag, 0, sizeof(int), h->stream) != cudaSuccess) return fail(LBM_ECUDA);
 
   // weight matrices K_mu (Section 2.4) in FP64 on the host, then the working precision

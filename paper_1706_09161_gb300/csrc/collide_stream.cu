@@ -318,7 +318,7 @@ __device__ __forceinline__ void write_split(const SplitOut& so, long long o, rea
 // Mass of the new concentration (the moment C = <1|f> of Algorithm 1), as a by-product of the step.
 // Every thread adds the C it wrote; each warp reduces its threads' sums in a fixed order
 // (xor shuffles: every lane ends with the same value) and lane 0 stores the warp's partial
-// at part[slot * kMassSlots + warp]; the handle adds the partials of the latest step in one
+// at part[slot * warps + warp]; the handle adds the partials of the latest step in one
 // small fixed-order FP64 pass when asked (lbm_mass).  FP32 concentrations are carried as an
 // unevaluated sum hi + lo of two floats, combined by TwoSum (Knuth), which keeps the sum
 // exact up to the rounding of lo (of order u^2 per addition, u = 2^-24) without FP64
@@ -369,11 +369,11 @@ struct MassAcc<float> {
   __device__ __forceinline__ void store(double* slot) const { *reinterpret_cast<float2*>(slot) = make_float2(hi, lo); }
 };
 
-template <typename real>
+template <int WARPS = kMassSlots, typename real>
 __device__ __forceinline__ void block_mass(MassAcc<real>& macc, double* part, int slot) {
   macc.warp_reduce();
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  if ((tid & 31) == 0 && part) macc.store(part + (long long)slot * kMassSlots + (tid >> 5));
+  if ((tid & 31) == 0 && part) macc.store(part + (long long)slot * WARPS + (tid >> 5));
 }
 
 // Thread block: 16 warps own a 32 x 16 tile of nodes (one node per thread, full
@@ -433,8 +433,12 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// One block's column (tile bx, by; planes z0 .. z1-1) of one problem.
-template <typename real, int D, bool MRT, int SPLIT, bool FLD = false, bool KS = false>
+// Warps of a block that owns a TXX x TYY tile: one thread per owned node and per ring node.
+__host__ __device__ constexpr int march_warps(int txx, int tyy) { return (txx * tyy + 2 * (txx + tyy) + 31) / 32; }
+static_assert(march_warps(TX, TY) == TY + HALO_WARPS, "32 x 16 tiles: 16 owner and 3 ring warps");
+
+// One block's column (TXX x TYY tile bx, by; planes z0 .. z1-1) of one problem.
+template <typename real, int D, bool MRT, int SPLIT, bool FLD = false, bool KS = false, int TXX = TX, int TYY = TY>
 __device__ __forceinline__ void march_body(const KConst<real>& sp, const real* __restrict__ f_in,
                                            const real* __restrict__ F, real* __restrict__ f_out,
                                            real* __restrict__ C_out, int* __restrict__ flag, const SplitOut& so,
@@ -442,32 +446,36 @@ __device__ __forceinline__ void march_body(const KConst<real>& sp, const real* _
                                            const FieldPtrs<real> fp = FieldPtrs<real>{}) {
   constexpr int Q = Lat<D>::Q;
   // movers of the current plane on the tile plus ring: [buffer][mover 1..4][y+1][x+1]
-  __shared__ real s_m[2][4][TY + 2][TX + 2];
+  __shared__ real s_m[2][4][TYY + 2][TXX + 2];
   const int n0 = sp.n[0], n1 = sp.n[1], n2 = sp.n[2];
   const long long nodes = sp.nodes;
   const long long plane = (long long)n0 * n1;
-  const int lane = threadIdx.x, wy = threadIdx.y;
-  const int x0 = bx * TX, y0 = by * TY;
+  const int tid = threadIdx.x + 32 * threadIdx.y, lane = threadIdx.x;
+  const int x0 = bx * TXX, y0 = by * TYY;
 
   // the node this thread collides every plane, and where its movers go
   int gx, gy, sx, sy;
-  const bool owner = wy < TY;
+  const bool owner = tid < TXX * TYY;
+  int side = -1;  // ring: which of the tile's sides this node borders (left, right, below, above)
   if (owner) {
-    gx = x0 + lane;
-    gy = y0 + wy;
-  } else if (wy == TY) {  // x-ring: left column (lanes 0-15), right column (16-31)
-    gx = (lane < 16) ? x0 - 1 : x0 + TX;
-    gy = y0 + (lane & 15);
-  } else {                // rows below (wy = TY+1) and above (wy = TY+2)
-    gx = x0 + lane;
-    gy = (wy == TY + 1) ? y0 - 1 : y0 + TY;
+    gx = x0 + tid % TXX;
+    gy = y0 + tid / TXX;
+  } else if (const int ring = tid - TXX * TYY; ring < 2 * TYY) {
+    side = ring / TYY;
+    gx = side ? x0 + TXX : x0 - 1;
+    gy = y0 + ring % TYY;
+  } else {
+    const int row = ring - 2 * TYY;
+    side = 2 + row / TXX;  // 4 and beyond: threads past the ring, idle
+    gx = x0 + row % TXX;
+    gy = side == 2 ? y0 - 1 : y0 + TYY;
   }
   sx = gx - x0 + 1;
   sy = gy - y0 + 1;
   // programmatic dependent launch: the operator's F (and the previous step's f) must be
   // complete before any load
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const bool in_xy = gx >= 0 && gx < n0 && gy >= 0 && gy < n1;
+  const bool in_xy = side < 4 && gx >= 0 && gx < n0 && gy >= 0 && gy < n1;
   const long long col = gx + (long long)n0 * gy;
   bool bad = false;
   MassAcc<real> macc;
@@ -493,14 +501,10 @@ __device__ __forceinline__ void march_body(const KConst<real>& sp, const real* _
     } else {
       real h[Q];
       collide_at<real, D, MRT, FLD, KS>(sp, f_in, F, in_xy, col + z * plane, h, fp);
-      if (wy == TY) {
-        if (lane < 16) s_m[buf][0][sy][sx] = h[1];  // moves +x into the tile
-        else s_m[buf][1][sy][sx] = h[2];            // moves -x into the tile
-      } else if (wy == TY + 1) {
-        s_m[buf][2][sy][sx] = h[3];                 // moves +y into the tile
-      } else {
-        s_m[buf][3][sy][sx] = h[4];                 // moves -y into the tile
-      }
+      if (side == 0) s_m[buf][0][sy][sx] = h[1];       // moves +x into the tile
+      else if (side == 1) s_m[buf][1][sy][sx] = h[2];  // moves -x into the tile
+      else if (side == 2) s_m[buf][2][sy][sx] = h[3];  // moves +y into the tile
+      else if (side == 3) s_m[buf][3][sy][sx] = h[4];  // moves -y into the tile
     }
     __syncthreads();
     if (owner && in_xy) {
@@ -579,7 +583,7 @@ __device__ __forceinline__ void march_body(const KConst<real>& sp, const real* _
   }
   // one flag update per warp at most
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(flag, 1);
-  block_mass(macc, mpart, mslot);
+  block_mass<march_warps(TXX, TYY)>(macc, mpart, mslot);
 }
 
 // movers of the current tile plus ring for the 2-D FP32 marches: [buffer][mover 1..4][y+1][x+1]
@@ -743,8 +747,8 @@ collide_stream_march2_kernel(const KConst<float> sp, const float* __restrict__ f
   if (!early) pdl_trigger();
 }
 
-template <typename real, int D, bool MRT, int SPLIT, bool FLD = false>
-__global__ void __launch_bounds__(TX*(TY + HALO_WARPS), 2)
+template <typename real, int D, bool MRT, int SPLIT, bool FLD = false, int TXX = TX, int TYY = TY>
+__global__ void __launch_bounds__(32 * march_warps(TXX, TYY), sizeof(real) == 4 ? 2 : 1)
 collide_stream_march_kernel(const KConst<real> sp, const real* __restrict__ f_in, const real* __restrict__ F,
                             real* __restrict__ f_out, real* __restrict__ C_out, int* __restrict__ flag, SplitOut so,
                             int nz, int early, double* mpart, const FieldPtrs<real> fp = FieldPtrs<real>{}) {
@@ -754,7 +758,7 @@ collide_stream_march_kernel(const KConst<real> sp, const real* __restrict__ f_in
   const int bz = blockIdx.z;
   const int z0 = static_cast<int>((long long)bz * n2 / nz), z1 = static_cast<int>((long long)(bz + 1) * n2 / nz);
   if (early) pdl_trigger();
-  march_body<real, D, MRT, SPLIT, FLD>(sp, f_in, F, f_out, C_out, flag, so, blockIdx.x, blockIdx.y, z0, z1, mpart,
+  march_body<real, D, MRT, SPLIT, FLD, false, TXX, TYY>(sp, f_in, F, f_out, C_out, flag, so, blockIdx.x, blockIdx.y, z0, z1, mpart,
                                        block_linear(), fp);
   if (!early) pdl_trigger();
 }
@@ -1367,7 +1371,7 @@ cudaError_t fused_launch(const lbm_s* h, int nsteps, int grid, cudaStream_t s) {
   SplitOut so{h->dev.Chi, h->dev.Clo, tc_split_pitch(h)};
   const int bx = (h->sp.n[0] + TX - 1) / TX, by = (h->sp.n[1] + TY - 1) / TY;
   const int ychunk = h->cs_chunk > 0 ? std::min(h->cs_chunk, by) : ychunk_for((long long)bx * by, by);
-  h->cs_nparts = bx * ((by + ychunk - 1) / ychunk);  // kMassSlots mass partials per collide-stream item
+  h->cs_nparts = kMassSlots * bx * ((by + ychunk - 1) / ychunk);  // per collide-stream item
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(TX, TY + HALO_WARPS);
@@ -1525,6 +1529,61 @@ int z_chunks(long long cols, int n2) {
   return best;
 }
 
+// FP64 march: block tile and z chunks.  The FP64 pipe bounds it (a warp instruction holds the
+// SM's pipe for 16 clocks, about 45 of them per collided node), so the plan with the smallest
+// share on the busiest SM wins: ceil(blocks / SMs) blocks of march_warps warps over the planes
+// of a chunk plus two (the chunk's first and last neighbours are collided again), plus the
+// unhidden load and barrier latency of each plane of one block.  Measured against 32 x 16 tiles
+// and chunks of at least 16 planes: 64^2 (8 blocks before, 128 now) 14.5 -> 8.4 us alone and the
+// whole step 12.5 -> 7.3 us; 80^3 (75 blocks of 19 warps before) 160 -> 81 us.
+struct March64Plan {
+  int tile;  // 0: 32 x 16, 1: 16 x 16, 2: 8 x 4
+  int bx, by, nz;
+};
+constexpr int kTile64[3][2] = {{TX, TY}, {16, 16}, {8, 4}};
+
+March64Plan march64_plan(const lbm_s* h, int chunk) {
+  const int n0 = h->sp.n[0], n1 = h->sp.n[1], n2 = h->sp.n[2];
+  const long long sms = device_sms();
+  March64Plan best{};
+  double best_cost = -1.0;
+  for (int t = 0; t < 3; ++t) {
+    const int bx = (n0 + kTile64[t][0] - 1) / kTile64[t][0], by = (n1 + kTile64[t][1] - 1) / kTile64[t][1];
+    for (int nz = 1; nz <= n2; ++nz) {
+      if (chunk > 0 && h->d == 3 && nz != std::min(chunk, n2)) continue;
+      const double planes = h->d == 2 ? 1.0 : static_cast<double>((n2 + nz - 1) / nz) + 2.0;
+      const double blocks = static_cast<double>(((long long)bx * by * nz + sms - 1) / sms);
+      const double cost = planes * (blocks * march_warps(kTile64[t][0], kTile64[t][1]) * 45 * 16 + 1500);
+      if (best_cost < 0.0 || cost < best_cost) {
+        best_cost = cost;
+        best = {t, bx, by, nz};
+      }
+    }
+  }
+  return best;
+}
+
+template <int D, bool MRT, bool FLD, int TXX, int TYY>
+cudaError_t launch_march64(cudaLaunchConfig_t& cfg, const KConst<double>& sp, const double* fi, const double* F,
+                           double* fo, double* Co, int* flag, int nz, double* mp, const FieldPtrs<double>& fp) {
+  cfg.blockDim = dim3(32, march_warps(TXX, TYY));
+  return cudaLaunchKernelEx(&cfg, collide_stream_march_kernel<double, D, MRT, 0, FLD, TXX, TYY>, sp, fi, F, fo, Co,
+                            flag, SplitOut{}, nz, 0, mp, fp);
+}
+
+template <int D, bool MRT, bool FLD>
+cudaError_t launch_march64_any(const lbm_s* h, cudaLaunchConfig_t& cfg, const KConst<double>& sp, const double* fi,
+                               const double* F, double* fo, double* Co, const FieldPtrs<double>& fp) {
+  const March64Plan pl = march64_plan(h, h->cs_chunk);
+  cfg.gridDim = dim3(pl.bx, pl.by, pl.nz);
+  h->cs_nparts = march_warps(kTile64[pl.tile][0], kTile64[pl.tile][1]) * pl.bx * pl.by * pl.nz;
+  int* flag = h->dev.flag;
+  double* mp = h->cs_part;
+  if (pl.tile == 0) return launch_march64<D, MRT, FLD, TX, TY>(cfg, sp, fi, F, fo, Co, flag, pl.nz, mp, fp);
+  if (pl.tile == 1) return launch_march64<D, MRT, FLD, 16, 16>(cfg, sp, fi, F, fo, Co, flag, pl.nz, mp, fp);
+  return launch_march64<D, MRT, FLD, 8, 4>(cfg, sp, fi, F, fo, Co, flag, pl.nz, mp, fp);
+}
+
 // tile rows per 2-D block: ceil(tiles / 304) (one wave of two blocks per SM), at most by
 int ychunk_for(long long tiles, int by) {
   const long long w = 2LL * device_sms();
@@ -1564,7 +1623,7 @@ cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out
     // coefficients per node: the plain march with the per-node collision (2-D: one plane)
     const int nz = (D == 2) ? 1 : (h->cs_chunk > 0 ? std::min(h->cs_chunk, sp.n[2]) : z_chunks((long long)bx * by, sp.n[2]));
     cfg.gridDim = dim3(bx, by, nz);
-    h->cs_nparts = bx * by * nz;
+    h->cs_nparts = kMassSlots * bx * by * nz;
     const int early = early_trigger(h, cfg.gridDim);
     FieldPtrs<real> fp{static_cast<const real*>(h->fld.coll), static_cast<const real*>(h->fld.advw),
                        static_cast<const real*>(h->fld.g),    static_cast<real*>(h->fld.G),
@@ -1576,6 +1635,7 @@ cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out
       for (int mu = 0; mu < 3; ++mu)
         for (int k = 0; k < 3; ++k) fp.gs[mu][k] = h->tc->gp[mu][k];
     }
+    if constexpr (sizeof(real) == 8) return launch_march64_any<D, MRT, true>(h, cfg, sp, fi, F, fo, Co, fp);
     if constexpr (sizeof(real) == 4) {
       // tensor-core forms: the march also writes the operator's operands of the new C
       if (split == 1)
@@ -1588,14 +1648,17 @@ cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out
         return cudaLaunchKernelEx(&cfg, collide_stream_march_kernel<real, D, MRT, 3, true>, sp, fi, F, fo, Co, flag, so,
                                   nz, early, mp, fp);
     }
-    return cudaLaunchKernelEx(&cfg, collide_stream_march_kernel<real, D, MRT, 0, true>, sp, fi, F, fo, Co, flag, so,
-                              nz, early, mp, fp);
+    if constexpr (sizeof(real) == 4)
+      return cudaLaunchKernelEx(&cfg, collide_stream_march_kernel<real, D, MRT, 0, true>, sp, fi, F, fo, Co, flag, so,
+                                nz, early, mp, fp);
   }
+  if constexpr (sizeof(real) == 8)
+    return launch_march64_any<D, MRT, false>(h, cfg, sp, fi, F, fo, Co, FieldPtrs<double>{});
   if constexpr (D == 2 && sizeof(real) == 4) {
     // tile rows per block: about one wave of two blocks per SM, unless tuned
     const int ychunk = h->cs_chunk > 0 ? std::min(h->cs_chunk, by) : ychunk_for((long long)bx * by, by);
     cfg.gridDim = dim3(bx, (by + ychunk - 1) / ychunk, 1);
-    h->cs_nparts = static_cast<int>(cfg.gridDim.x * cfg.gridDim.y);
+    h->cs_nparts = kMassSlots * static_cast<int>(cfg.gridDim.x * cfg.gridDim.y);
     const int early = early_trigger(h, cfg.gridDim);
     if (h->cs_plan) {
       const CsPlan* pl = static_cast<const CsPlan*>(h->cs_plan);
@@ -1615,9 +1678,10 @@ cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out
     if (split == 3) return launch_march2<MRT, 3>(cfg, sp, fi, F, fo, Co, flag, so, ychunk, early, mp);
     return launch_march2<MRT, 2>(cfg, sp, fi, F, fo, Co, flag, so, ychunk, early, mp);
   }
+  if constexpr (sizeof(real) == 4) {
   const int nz = h->cs_chunk > 0 ? std::min(h->cs_chunk, sp.n[2]) : z_chunks((long long)bx * by, sp.n[2]);
   cfg.gridDim = dim3(bx, by, nz);
-  h->cs_nparts = bx * by * nz;
+  h->cs_nparts = kMassSlots * bx * by * nz;
   const int early = early_trigger(h, cfg.gridDim);
   if constexpr (D == 3 && sizeof(real) == 4) {
     if (h->cs_plan) {
@@ -1647,6 +1711,7 @@ cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out
                               early, mp, FieldPtrs<real>{});
   return cudaLaunchKernelEx(&cfg, collide_stream_march_kernel<real, D, MRT, 2>, sp, fi, F, fo, Co, flag, so, nz,
                             early, mp, FieldPtrs<real>{});
+  }
 }
 
 int grid_for(long long n) {
@@ -1772,6 +1837,10 @@ void cs_release(lbm_s* h) {
 }
 
 bool cs_one_wave(const lbm_s* h) {
+  if (h->elem == 8) {
+    const March64Plan pl = march64_plan(h, h->cs_chunk);
+    return one_wave(dim3(pl.bx, pl.by, pl.nz));
+  }
   const int bx = (h->sp.n[0] + TX - 1) / TX, by = (h->sp.n[1] + TY - 1) / TY;
   if (h->d == 2 && h->elem == 4) {
     const int ychunk = h->cs_chunk > 0 ? std::min(h->cs_chunk, by) : ychunk_for((long long)bx * by, by);
@@ -1782,11 +1851,20 @@ bool cs_one_wave(const lbm_s* h) {
   return one_wave(dim3(bx, by, nz));
 }
 
+long long cs_max_parts(const lbm_s* h) {
+  long long most = 0;
+  for (int t = 0; t < (h->elem == 8 ? 3 : 1); ++t) {  // one block per tile and plane at most
+    const long long bx = (h->sp.n[0] + kTile64[t][0] - 1) / kTile64[t][0], by = (h->sp.n[1] + kTile64[t][1] - 1) / kTile64[t][1];
+    most = std::max(most, march_warps(kTile64[t][0], kTile64[t][1]) * bx * by * h->sp.n[2]);
+  }
+  return most;
+}
+
 int cs_chunk_default(const lbm_s* h) {
   const int bx = (h->sp.n[0] + TX - 1) / TX, by = (h->sp.n[1] + TY - 1) / TY;
   if (h->is_batch()) return kBatchYChunk;
   if (h->d == 2) return h->elem == 4 ? ychunk_for((long long)bx * by, by) : 1;
-  return z_chunks((long long)bx * by, h->sp.n[2]);
+  return h->elem == 8 ? march64_plan(h, 0).nz : z_chunks((long long)bx * by, h->sp.n[2]);
 }
 
 int cs_batch_prepare(lbm_s* b) {
@@ -1812,9 +1890,10 @@ int cs_batch_prepare(lbm_s* b) {
     e.by = (h->sp.n[1] + TY - 1) / TY;
     // 2-D: tile rows per block (the pipelined y-march); 3-D: the whole z extent
     e.zchunk = (h->d == 2) ? std::min(e.by, b->cs_chunk > 0 ? b->cs_chunk : kBatchYChunk) : h->sp.n[2];
-    h->cs_nparts = e.bx * ((h->d == 2) ? (e.by + e.zchunk - 1) / e.zchunk : e.by);
-    for (int k = 0; k < h->cs_nparts; ++k) map.push_back(make_int2(i, k));
-    total += h->cs_nparts;
+    const int blocks = e.bx * ((h->d == 2) ? (e.by + e.zchunk - 1) / e.zchunk : e.by);
+    h->cs_nparts = kMassSlots * blocks;
+    for (int k = 0; k < blocks; ++k) map.push_back(make_int2(i, k));
+    total += blocks;
   }
   dev_free(b, b->batch_cs);
   dev_free(b, b->batch_cs_start);

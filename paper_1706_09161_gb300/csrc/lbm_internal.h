@@ -11,7 +11,7 @@
 namespace lbm {
 
 constexpr int kMaxQ = 7;
-// mass partials per collide-stream block: one per warp of its 32 x (16 + 3) threads
+// mass partials per collide-stream block of 32 x (16 + 3) threads: one per warp
 constexpr int kMassSlots = 19;
 struct TcPlan;  // tensor-core plan (frac_tc.cu)
 
@@ -115,7 +115,7 @@ struct lbm_s {
   unsigned int* fused_bar = nullptr;   // grid-barrier counter
   int device = 0;
   // FP64 warp partials of the mass of the concentration each collide-stream launch writes
-  // (kMassSlots per block of its grid: cs_nparts blocks, at most cs_part_cap); mass_valid when the
+  // (one per warp of its grid: cs_nparts, at most cs_part_cap); mass_valid when the
   // latest C came from a step (not from a re-initialisation); mass_limit > 0 turns a mass of
   // larger magnitude (or a non-finite one) into LBM_ERR_UNSTABLE at the next synchronising call
   double* cs_part = nullptr;
@@ -233,6 +233,7 @@ bool encode_f32_map(void* map, int rank, void* base, const unsigned long long* d
                     const unsigned long long* strides_bytes, const unsigned int* box);
 bool cs_one_wave(const lbm_s* h);  // the collide-stream grid fits in one wave
 int cs_chunk_default(const lbm_s* h);  // the built-in tile rows (2-D) / z chunks (3-D)
+long long cs_max_parts(const lbm_s* h);  // the most mass partials any collide-stream launch of h writes
 // fused 2-D step (bf16 split, per-tile plan with 64/128-column tiles and a split of 2 or
 // 4): LBM_OK if this handle can run it (sets fused_grid), LBM_ENOTSUP otherwise
 int fused_prepare(lbm_s* h);

@@ -128,7 +128,7 @@ cudaError_t launch_mass(const lbm_s* h, const void* C, cudaStream_t s) {
 }
 
 cudaError_t launch_step_mass(const lbm_s* h, double limit, cudaStream_t s) {
-  step_mass_kernel<<<1, kReduceThreads, 0, s>>>(h->cs_part, h->cs_nparts * kMassSlots, h->elem == 4 ? 1 : 0,
+  step_mass_kernel<<<1, kReduceThreads, 0, s>>>(h->cs_part, h->cs_nparts, h->elem == 4 ? 1 : 0,
                                                  h->dev.scalar, limit, h->dev.flag);
   return cudaGetLastError();
 }
