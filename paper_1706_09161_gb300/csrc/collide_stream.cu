@@ -20,6 +20,7 @@
 
 #include "lbm_internal.h"
 #include "tc_dev.cuh"
+#include "two_float.cuh"
 
 namespace lbm {
 namespace {
@@ -328,49 +329,8 @@ __device__ __forceinline__ void write_split(const SplitOut& so, long long o, rea
 // collide-stream kernels, and even the three FP64 operations per warp of a double partial
 // kept that pipe 11% busy at the tail of the 512^2 kernel.  FP64 concentrations are summed
 // and stored in FP64.  No block-wide barrier.  part may be null (no partial wanted).
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bp = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bp)), __fsub_rn(b, bp));
-}
-
-template <typename real>
-struct MassAcc;
-template <>
-struct MassAcc<double> {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double x) { s += x; }
-  __device__ __forceinline__ void warp_reduce() {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  }
-  __device__ __forceinline__ void store(double* slot) const { *slot = s; }
-};
-template <>
-struct MassAcc<float> {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float x) {
-    float t, e;
-    two_sum(hi, x, t, e);
-    hi = t;
-    lo = __fadd_rn(lo, e);
-  }
-  __device__ __forceinline__ void warp_reduce() {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float oh = __shfl_xor_sync(0xffffffffu, hi, o), ol = __shfl_xor_sync(0xffffffffu, lo, o);
-      float t, e;
-      two_sum(hi, oh, t, e);
-      hi = t;
-      lo = __fadd_rn(__fadd_rn(lo, ol), e);
-    }
-  }
-  // the pair (hi, lo) in the slot's 8 bytes; the final pass adds hi + lo in FP64
-  __device__ __forceinline__ void store(double* slot) const { *reinterpret_cast<float2*>(slot) = make_float2(hi, lo); }
-};
-
 template <int WARPS = kMassSlots, typename real>
-__device__ __forceinline__ void block_mass(MassAcc<real>& macc, double* part, int slot) {
+__device__ __forceinline__ void block_mass(SumAcc<real>& macc, double* part, int slot) {
   macc.warp_reduce();
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
   if ((tid & 31) == 0 && part) macc.store(part + (long long)slot * WARPS + (tid >> 5));
@@ -478,7 +438,7 @@ __device__ __forceinline__ void march_body(const KConst<real>& sp, const real* _
   const bool in_xy = side < 4 && gx >= 0 && gx < n0 && gy >= 0 && gy < n1;
   const long long col = gx + (long long)n0 * gy;
   bool bad = false;
-  MassAcc<real> macc;
+  SumAcc<real> macc;
 
   real cur[Q], nxt[Q];
   real prev5 = static_cast<real>(0);
@@ -641,7 +601,7 @@ __device__ __forceinline__ void march2_pipe(const KConst<float>& sp, const float
   issue(tr0, 0);
   if (tr0 + 1 < tr1) issue(tr0 + 1, 1); else cp_async_commit();
   bool bad = false;
-  MassAcc<float> macc;
+  SumAcc<float> macc;
   int buf = 0;
   for (int tr = tr0; tr < tr1; ++tr) {
     const int slot = (tr - tr0) % PIPE_STAGES;
@@ -929,7 +889,7 @@ collide_stream_tma3_kernel(const KConst<float> sp, const __grid_constant__ CUten
     issue(z0 + 1);  // z0 + 1 <= z1: needed by the owners' first iteration
   }
   bool bad = false;
-  MassAcc<float> macc;
+  SumAcc<float> macc;
   float cur[Q], nxt[Q];
   float prev5 = 0.f;
   if (owner) {
@@ -1144,7 +1104,7 @@ __device__ __forceinline__ void march2_tma(const KConst<float>& sp, const CUtens
   if (tid == 0)
     for (int t = tr0; t < tr1 && t < tr0 + nst; ++t) issue(t);
   bool bad = false;
-  MassAcc<float> macc;
+  SumAcc<float> macc;
   int buf = 0;
   for (int tr = tr0; tr < tr1; ++tr) {
     cs_mbar_wait(&full[stage_of(tr)], parity_of(tr), flag);
@@ -1599,13 +1559,14 @@ int cs_split_code(const lbm_s* h) {
 }
 
 template <typename real, int D, bool MRT>
-cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out, cudaStream_t s, int tk) {
+cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out, cudaStream_t s, int tk,
+                      const CsSlot* slot) {
   const KConst<real> sp = make_const<real>(h->sp);
   SplitOut so{h->dev.Chi, h->dev.Clo, tc_split_pitch(h)};
   so.lo2 = h->dev.Cl2;
   const int split = cs_split_code(h);
   const real* fi = static_cast<const real*>(f_in);
-  const real* F = static_cast<const real*>(h->dev.F);
+  const real* F = static_cast<const real*>(slot ? slot->F : h->dev.F);
   real* fo = static_cast<real*>(f_out);
   real* Co = static_cast<real*>(C_out);
   int* flag = h->dev.flag;
@@ -1662,15 +1623,16 @@ cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out
     const int early = early_trigger(h, cfg.gridDim);
     if (h->cs_plan) {
       const CsPlan* pl = static_cast<const CsPlan*>(h->cs_plan);
-      const CUtensorMap& mf = pl->f[f_in == h->dev.f[0] ? 0 : 1];
+      const CUtensorMap& mf = slot ? *static_cast<const CUtensorMap*>(slot->map_f) : pl->f[f_in == h->dev.f[0] ? 0 : 1];
+      const CUtensorMap& mF = slot ? *static_cast<const CUtensorMap*>(slot->map_F) : pl->F;
       cfg.dynamicSmemBytes = tma2_smem(h->sp.ksum);
-      if (split == 0) return launch_tma2<MRT, 0>(cfg, sp, mf, pl->F, fo, Co, flag, so, ychunk, early, mp);
-      if (split == 1) return launch_tma2<MRT, 1>(cfg, sp, mf, pl->F, fo, Co, flag, so, ychunk, early, mp);
-      if (split == 3) return launch_tma2<MRT, 3>(cfg, sp, mf, pl->F, fo, Co, flag, so, ychunk, early, mp);
+      if (split == 0) return launch_tma2<MRT, 0>(cfg, sp, mf, mF, fo, Co, flag, so, ychunk, early, mp);
+      if (split == 1) return launch_tma2<MRT, 1>(cfg, sp, mf, mF, fo, Co, flag, so, ychunk, early, mp);
+      if (split == 3) return launch_tma2<MRT, 3>(cfg, sp, mf, mF, fo, Co, flag, so, ychunk, early, mp);
       so.thi[0] = static_cast<float*>(h->tc->ct_hi[1]);  // the y operand of the tf32 operator
       so.tg1 = h->tc->tg[1];
       so.tpx = h->tc->tpx;
-      return launch_tma2<MRT, 2>(cfg, sp, mf, pl->F, fo, Co, flag, so, ychunk, early, mp);
+      return launch_tma2<MRT, 2>(cfg, sp, mf, mF, fo, Co, flag, so, ychunk, early, mp);
     }
     cfg.dynamicSmemBytes = PIPE_SMEM;
     if (split == 0) return launch_march2<MRT, 0>(cfg, sp, fi, F, fo, Co, flag, so, ychunk, early, mp);
@@ -1687,17 +1649,18 @@ cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out
     if (h->cs_plan) {
       // TMA-fed march: the map of whichever population buffer is the input
       const CsPlan* pl = static_cast<const CsPlan*>(h->cs_plan);
-      const CUtensorMap& mf = pl->f[f_in == h->dev.f[0] ? 0 : 1];
+      const CUtensorMap& mf = slot ? *static_cast<const CUtensorMap*>(slot->map_f) : pl->f[f_in == h->dev.f[0] ? 0 : 1];
+      const CUtensorMap& mF = slot ? *static_cast<const CUtensorMap*>(slot->map_F) : pl->F;
       cfg.dynamicSmemBytes = TMA_SMEM;
-      if (split == 0) return launch_tma3<MRT, 0>(cfg, sp, mf, pl->F, fo, Co, flag, so, nz, early, mp);
-      if (split == 1) return launch_tma3<MRT, 1>(cfg, sp, mf, pl->F, fo, Co, flag, so, nz, early, mp);
-      if (split == 3) return launch_tma3<MRT, 3>(cfg, sp, mf, pl->F, fo, Co, flag, so, nz, early, mp);
+      if (split == 0) return launch_tma3<MRT, 0>(cfg, sp, mf, mF, fo, Co, flag, so, nz, early, mp);
+      if (split == 1) return launch_tma3<MRT, 1>(cfg, sp, mf, mF, fo, Co, flag, so, nz, early, mp);
+      if (split == 3) return launch_tma3<MRT, 3>(cfg, sp, mf, mF, fo, Co, flag, so, nz, early, mp);
       for (int a = 0; a < 2; ++a) {  // the y and z operands of the tf32 operator
         so.thi[a] = static_cast<float*>(h->tc->ct_hi[a + 1]);
       }
       so.tg1 = h->tc->tg[1];
       so.tpx = h->tc->tpx;
-      return launch_tma3<MRT, 2>(cfg, sp, mf, pl->F, fo, Co, flag, so, nz, early, mp);
+      return launch_tma3<MRT, 2>(cfg, sp, mf, mF, fo, Co, flag, so, nz, early, mp);
     }
   }
   if (split == 0)
@@ -1729,36 +1692,46 @@ bool cs_writes_T(const lbm_s* h) {
          h->prm.precision == LBM_FP32_TF32SPLIT && !h->fld.on;  // the field march writes x-major operands only
 }
 
-cudaError_t launch_collide_stream(const lbm_s* h, const void* f_in, void* f_out, void* C_out, cudaStream_t s,
-                                  int tk) {
+cudaError_t launch_collide_stream(const lbm_s* h, const void* f_in, void* f_out, void* C_out, cudaStream_t s, int tk,
+                                  const CsSlot* slot) {
   const bool mrt = h->prm.collision == LBM_MRT;
   if (h->elem == 8) {
-    if (h->d == 2) return mrt ? launch_cs<double, 2, true>(h, f_in, f_out, C_out, s, tk)
-                              : launch_cs<double, 2, false>(h, f_in, f_out, C_out, s, tk);
-    return mrt ? launch_cs<double, 3, true>(h, f_in, f_out, C_out, s, tk)
-               : launch_cs<double, 3, false>(h, f_in, f_out, C_out, s, tk);
+    if (h->d == 2) return mrt ? launch_cs<double, 2, true>(h, f_in, f_out, C_out, s, tk, slot)
+                              : launch_cs<double, 2, false>(h, f_in, f_out, C_out, s, tk, slot);
+    return mrt ? launch_cs<double, 3, true>(h, f_in, f_out, C_out, s, tk, slot)
+               : launch_cs<double, 3, false>(h, f_in, f_out, C_out, s, tk, slot);
   }
-  if (h->d == 2) return mrt ? launch_cs<float, 2, true>(h, f_in, f_out, C_out, s, tk)
-                            : launch_cs<float, 2, false>(h, f_in, f_out, C_out, s, tk);
-  return mrt ? launch_cs<float, 3, true>(h, f_in, f_out, C_out, s, tk)
-             : launch_cs<float, 3, false>(h, f_in, f_out, C_out, s, tk);
+  if (h->d == 2) return mrt ? launch_cs<float, 2, true>(h, f_in, f_out, C_out, s, tk, slot)
+                            : launch_cs<float, 2, false>(h, f_in, f_out, C_out, s, tk, slot);
+  return mrt ? launch_cs<float, 3, true>(h, f_in, f_out, C_out, s, tk, slot)
+             : launch_cs<float, 3, false>(h, f_in, f_out, C_out, s, tk, slot);
 }
 
 constexpr int kBatchYChunk = 16;  // tile rows per block (the autotuner's usual choice on mixed batches)
 
-// window maps of a 2-D handle: populations (n0, n1, 5) and fractional terms (n0, n1, 2)
-bool encode_2d_maps(const lbm_s* h, CUtensorMap* mf, CUtensorMap* mF) {
-  const unsigned long long n0 = h->sp.n[0], n1 = h->sp.n[1];
-  const unsigned long long nodes = h->sp.nodes;
-  const unsigned long long strides[2] = {n0 * 4, nodes * 4};
-  const unsigned long long ks = (unsigned long long)h->sp.ksum;  // F: [partial][axis][node]
-  const unsigned long long df[3] = {n0, n1, 5};
-  const unsigned long long dF[3] = {n0, n1, 2 * ks};
-  const unsigned int bf[3] = {TW, TH, 5};
-  const unsigned int bF[3] = {TW, TH, (unsigned int)(2 * ks)};
-  return encode_f32_map(&mf[0], 3, h->dev.f[0], df, strides, bf) &&
-         encode_f32_map(&mf[1], 3, h->dev.f[1], df, strides, bf) &&
-         encode_f32_map(mF, 3, h->dev.F, dF, strides, bF);
+// window map of `planes` fields (x fastest, `base` their first) for the TMA-fed marches:
+// (n0, n1, planes) in 2-D, (n0, n1, n2, planes) in 3-D
+bool encode_window(const lbm_s* h, CUtensorMap* m, const void* base, unsigned long long planes) {
+  const unsigned long long n0 = h->sp.n[0], n1 = h->sp.n[1], n2 = h->sp.n[2], nodes = h->sp.nodes;
+  if (h->d == 2) {
+    const unsigned long long dims[3] = {n0, n1, planes}, strides[2] = {n0 * 4, nodes * 4};
+    const unsigned int box[3] = {TW, TH, (unsigned int)planes};
+    return encode_f32_map(m, 3, const_cast<void*>(base), dims, strides, box);
+  }
+  const unsigned long long dims[4] = {n0, n1, n2, planes}, strides[3] = {n0 * 4, n0 * n1 * 4, nodes * 4};
+  const unsigned int box[4] = {TW, TH, 1, (unsigned int)planes};
+  return encode_f32_map(m, 4, const_cast<void*>(base), dims, strides, box);
+}
+
+// window maps of a handle: its population buffers and its fractional terms ([partial][axis][node])
+bool encode_maps(const lbm_s* h, CUtensorMap* mf, CUtensorMap* mF) {
+  return encode_window(h, &mf[0], h->dev.f[0], h->Q) && encode_window(h, &mf[1], h->dev.f[1], h->Q) &&
+         encode_window(h, mF, h->dev.F, (unsigned long long)h->d * h->sp.ksum);
+}
+
+bool cs_encode_slot(const lbm_s* h, const void* f, const void* F, void* map_f, void* map_F) {
+  return encode_window(h, static_cast<CUtensorMap*>(map_f), f, h->Q) &&
+         encode_window(h, static_cast<CUtensorMap*>(map_F), F, h->d);
 }
 
 // the fused step for this handle's plan: 0 (not covered) or the blocks per SM it gets
@@ -1808,26 +1781,8 @@ int cs_prepare(lbm_s* h) {
   if (h->d == 3 && h->sp.ksum != 1) return LBM_OK;  // the plain 3-D march sums the partials
   CsPlan* pl = new (std::nothrow) CsPlan();
   if (!pl) return LBM_ENOMEM;
-  if (h->d == 2) {
-    if (encode_2d_maps(h, pl->f, &pl->F)) h->cs_plan = pl;
-    else delete pl;  // the cp.async march serves the handle
-    return LBM_OK;
-  }
-  const unsigned long long n0 = h->sp.n[0], n1 = h->sp.n[1], n2 = h->sp.n[2];
-  const unsigned long long nodes = h->sp.nodes;
-  const unsigned long long strides[3] = {n0 * 4, n0 * n1 * 4, nodes * 4};
-  const unsigned long long df[4] = {n0, n1, n2, 7};
-  const unsigned long long dF[4] = {n0, n1, n2, 3};
-  const unsigned int bf[4] = {TW, TH, 1, 7};
-  const unsigned int bF[4] = {TW, TH, 1, 3};
-  bool ok = encode_f32_map(&pl->f[0], 4, h->dev.f[0], df, strides, bf) &&
-            encode_f32_map(&pl->f[1], 4, h->dev.f[1], df, strides, bf) &&
-            encode_f32_map(&pl->F, 4, h->dev.F, dF, strides, bF);
-  if (!ok) {
-    delete pl;
-    return LBM_OK;  // the plain march serves the handle
-  }
-  h->cs_plan = pl;
+  if (encode_maps(h, pl->f, &pl->F)) h->cs_plan = pl;
+  else delete pl;  // the cp.async (2-D) or plain (3-D) march serves the handle
   return LBM_OK;
 }
 
@@ -1885,7 +1840,7 @@ int cs_batch_prepare(lbm_s* b) {
     e.so.lo2 = h->dev.Cl2;
     e.flag = h->dev.flag;
     e.mpart = h->cs_part;
-    e.tma = (h->d == 2 && h->sp.n[0] % 4 == 0 && encode_2d_maps(h, e.mf, &e.mF)) ? 1 : 0;
+    e.tma = (h->d == 2 && h->sp.n[0] % 4 == 0 && encode_maps(h, e.mf, &e.mF)) ? 1 : 0;
     e.bx = (h->sp.n[0] + TX - 1) / TX;
     e.by = (h->sp.n[1] + TY - 1) / TY;
     // 2-D: tile rows per block (the pipelined y-march); 3-D: the whole z extent

@@ -15,6 +15,7 @@
 #include <algorithm>
 
 #include "lbm_internal.h"
+#include "simt_dev.cuh"
 
 namespace lbm {
 namespace {
@@ -73,18 +74,6 @@ __device__ __forceinline__ BlockAt locate_block(const GemmPlan& P, long long b, 
 constexpr int SBK = 16;
 constexpr int kSlice = 32;  // contraction slices of a split start at multiples of this
 
-__device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-  unsigned long long d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-
-__device__ __forceinline__ unsigned long long twice(float a) {
-  unsigned long long d;
-  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(a));
-  return d;
-}
-
 __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr, uint32_t rank) {
   uint32_t r;
   float4 v;
@@ -99,17 +88,6 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// four consecutive values p[0..3] of which `left` exist (zeros past them)
-__device__ __forceinline__ float4 load4(const float* p, int left, bool vec) {
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (left >= 4 && vec) return *reinterpret_cast<const float4*>(p);
-  if (left > 0) v.x = p[0];
-  if (left > 1) v.y = p[1];
-  if (left > 2) v.z = p[2];
-  if (left > 3) v.w = p[3];
-  return v;
 }
 
 __device__ __forceinline__ void store4(float* p, float4 v, int left, bool vec) {
@@ -489,9 +467,9 @@ bool blocks_fit(Kernel k, int threads, long long blocks) {
 template <typename real>
 cudaError_t frac_all_axes(const lbm_s* h, const real* C, real* F, cudaStream_t s, bool transpose = false,
                           long long cstride = 0) {
-  // the forward operator of a handle with programmatic dependent launch overlaps the
-  // previous collide-stream kernel's tail
-  const bool pdl = !transpose && h->pdl;
+  // programmatic dependent launch: the forward operator overlaps the previous collide-stream
+  // kernel's tail where the handle has it on, the transpose that of the adjoint's step
+  const bool pdl = transpose || h->pdl;
   cudaLaunchConfig_t cfg = {};
   cfg.stream = s;
   cudaLaunchAttribute at[2];
@@ -517,7 +495,7 @@ cudaError_t frac_all_axes(const lbm_s* h, const real* C, real* F, cudaStream_t s
       GemmPlan P = make_plan<real>(h, C, F, transpose, cstride, G.BM, G.BN, ks);
       // 2-D only: the 3-D marches' long blocks, launched early, would pile up two to an SM on
       // the SMs this grid leaves first (measured: 48^3 step 24 -> 37 us)
-      P.early = pdl && h->d == 2 && blocks_fit(kernel, G.THREADS, P.total);
+      P.early = !transpose && pdl && h->d == 2 && blocks_fit(kernel, G.THREADS, P.total);
       cfg.gridDim = dim3(static_cast<unsigned>(P.total), 1, 1);
       cfg.blockDim = dim3(G.THREADS, 1, 1);
       return cudaLaunchKernelEx(&cfg, kernel, P);

@@ -174,8 +174,16 @@ bool simt_one_wave(const lbm_s* h);
 cudaError_t launch_frac_tc(const lbm_s* h, cudaStream_t s);
 // fused equilibrium + collision + streaming + Dirichlet + new concentration; on the
 // tensor-core path it also writes the hi/lo split of the new concentration
+// other arrays than the handle's own for one launch: F, and with a TMA-fed march the window
+// maps (CUtensorMap) of f_in and F (cs_encode_slot)
+struct CsSlot {
+  const void* F;
+  const void* map_f;
+  const void* map_F;
+};
 cudaError_t launch_collide_stream(const lbm_s* h, const void* f_in, void* f_out, void* C_out,
-                                  cudaStream_t s, int tk = 0);
+                                  cudaStream_t s, int tk = 0, const CsSlot* slot = nullptr);
+bool cs_encode_slot(const lbm_s* h, const void* f, const void* F, void* map_f, void* map_F);
 // f = feq(C, F) (with u(x) when the coefficients vary)
 cudaError_t launch_init_equilibrium(const lbm_s* h, void* f, cudaStream_t s);
 // G_mu = g_mu(x) C (spatially varying coefficients only)
@@ -188,9 +196,6 @@ cudaError_t launch_convert_out(const void* src, int elem, double* dst_f64, long 
 // dst_f64[i] = sum_{s < k} src[s * stride + i], FP32 partials added in order of s
 cudaError_t launch_sum_partials_out(const float* src, int k, long long stride, double* dst_f64, long long n,
                                     cudaStream_t s);
-// dst[i] = sum_{s < k} src[s * stride + i] in FP32, in order of s (as the collide-stream
-// kernels add the operator's partial sums)
-cudaError_t launch_sum_partials(const float* src, int k, long long stride, float* dst, long long n, cudaStream_t s);
 // mass reduction: partials then final
 cudaError_t launch_mass(const lbm_s* h, const void* C, cudaStream_t s);
 // mass of the latest step from the collide-stream kernel's warp partials (one small pass,
