@@ -154,8 +154,6 @@ int derive(const lbm_params* p, Derived* out) {
   sp.wi = (d == 2) ? 1.0 / 6.0 : 1.0 / 8.0;
   for (int mu = 0; mu < 3; ++mu) sp.adv[mu] = (mu < d) ? (p->dt / p->dx) * p->u[mu] / e2 : 0.0;
   sp.C_wall = p->C_wall;
-  sp.ksum = 1;
-  sp.pstride = 0;
   const double ratio = p->dt / (p->dx * p->dx);
   double Dm[9];
   for (int i = 0; i < d; ++i)
@@ -523,6 +521,7 @@ static int create_problem(const lbm_params* prm, const double* C0_host, void* st
   if ((rc = alloc_bytes(h, &h->dev.C, E * nodes))) return fail(rc);
   if ((rc = alloc_bytes(h, &h->dev.C0, E * nodes))) return fail(rc);
   if ((rc = alloc_bytes(h, &h->dev.F, E * h->d * nodes))) return fail(rc);
+  h->f_elems = (size_t)h->d * nodes;
   if ((rc = alloc_bytes(h, &h->dev.K, E * ksz))) return fail(rc);
   if ((rc = alloc_bytes(h, &h->dev.KT, E * ksz))) return fail(rc);
   if ((rc = alloc_bytes(h, (void**)&h->dev.stage, sizeof(double) * (size_t)(nodes > ksz ? nodes : ksz)))) return fail(rc);
@@ -770,9 +769,9 @@ int lbm_read_F(lbm_t h, int mu, double* F_host) {
   const long long nodes = h->sp.nodes;
   int rc = run_frac(h, h->stream);
   if (rc) return rc;
-  if (h->sp.ksum > 1)  // split-K partial sums of the tensor-core operator (FP32 forms)
+  if (h->sp.ksum > 1)
     LBM_CUDA(lbm::launch_sum_partials_out(static_cast<const float*>(h->dev.F) + (size_t)mu * nodes, h->sp.ksum,
-                                          h->sp.pstride, h->dev.stage, nodes, h->stream));
+                                          (long long)h->d * nodes, h->dev.stage, nodes, h->stream));
   else
     LBM_CUDA(lbm::launch_convert_out((char*)h->dev.F + (size_t)mu * nodes * h->elem, h->elem, h->dev.stage, nodes,
                                      h->stream));
@@ -1326,10 +1325,8 @@ int lbm_set_params(lbm_t h, const lbm_params* prm) {
   const lbm_params keep = h->prm;
   const lbm::StepParams keep_sp = h->sp;
   h->prm = *prm;
-  lbm::StepParams sp = dv.sp;
-  sp.ksum = keep_sp.ksum;  // the launch plan stays: its partial sums of F
-  sp.pstride = keep_sp.pstride;
-  h->sp = sp;
+  h->sp = dv.sp;
+  h->sp.ksum = keep_sp.ksum;  // the launch plan stays
   if (h->fld.on) {
     rc = rebuild_fields(h);  // per-node rates, g and the weights from the new constants
   } else {

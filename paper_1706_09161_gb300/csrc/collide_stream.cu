@@ -81,7 +81,7 @@ KConst<real> make_const(const StepParams& sp) {
   for (int i = 0; i < 3; ++i) k.advw[i] = static_cast<real>(sp.adv[i] * sp.wi);
   k.C_wall = static_cast<real>(sp.C_wall);
   k.ksum = sp.ksum;
-  k.pstride = sp.pstride;
+  k.pstride = (sp.n[2] > 1 ? 3 : 2) * sp.nodes;
   for (int i = 0; i < 3; ++i) k.sfree[i] = static_cast<real>(sp.sfree[i]);
   return k;
 }
@@ -1780,7 +1780,6 @@ cudaError_t launch_fused(lbm_s* h, int nsteps, cudaStream_t s) {
 
 int cs_prepare(lbm_s* h) {
   if (h->elem != 4 || h->sp.n[0] % 4 != 0) return LBM_OK;
-  if (h->d == 3 && h->sp.ksum != 1) return LBM_OK;  // the plain 3-D march sums the partials
   CsPlan* pl = new (std::nothrow) CsPlan();
   if (!pl) return LBM_ENOMEM;
   if (encode_maps(h, pl->f, &pl->F)) h->cs_plan = pl;

@@ -21,10 +21,14 @@
 // accumulator is allocated), warp 1 / lane 0 issues the MMAs and releases ring slots
 // with tcgen05.commit, then all four warps drain the accumulator (tcgen05.ld, one
 // lane quarter per warp) into a shared [BN][128] tile that one TMA store writes to F.
-// Small problems split the contraction over ksplit independent CTAs per tile: CTA
-// `rank` contracts its k-range and stores its partial tile to slot `rank` of F, laid out
-// [rank][axis][node]; the kernels that read F add the ksplit partials in rank order, so
-// the result does not depend on timing (and no CTA waits for another).  Problems with many tiles use the persistent kernel further
+// Small problems split the contraction over ksplit CTAs, CTA `rank` contracting its k-range.
+// Where F is stored with TMA and read by the 2-D march, the partial tiles stay in slots of F,
+// [rank][axis][node], which the march adds in rank order.  Else (ragged rows, 3-D) the CTAs of a
+// tile form a cluster that adds the partial tiles in rank order through distributed shared
+// memory, each CTA summing and storing its share of the rows.  Either way the result does not
+// depend on timing.  (Measured: 301 x 203 bf16x6 step 13.5 us with slots, 10.6 with clusters,
+// whose plain stores and reads of F are a quarter; 512^2 12.4 and 13.2: a cluster's four CTAs
+// cannot start on the SMs that the previous kernel leaves one by one.)  Problems with many tiles use the persistent kernel further
 // down (two TMEM accumulators, epilogue overlapping the next tile).  Every mbarrier wait is
 // bounded by a 2 s %globaltimer budget; a wait that gives up sets bit 2 of the
 // handle's error flag and the CTA skips the rest of its work and releases TMEM.
@@ -45,10 +49,26 @@ namespace {
 
 // One output tile (or one k-slice of it when KS > 1) of one problem; `block` is the
 // CTA's index among that problem's CTAs.  `maps` may live in parameter or global memory.
-// per-tile operator: 4 warps (producer, MMA issuer, all four drain TMEM); tf32 adds warps 4-7,
-// which with warps 2-3 split each stage's C into hi + lo and leave before the epilogue
+// per-tile operator: 8 warps (producer, MMA issuer; all drain TMEM, two warps per lane
+// quarter, which take alternate 32-column chunks); tf32: warps 2-7 also split each stage's C
+// into hi + lo
 constexpr int kTileSplitWarps = 6;
-__host__ __device__ constexpr int tile_threads(int E) { return E == 4 ? 256 : 128; }
+constexpr int kTileThreads = 256;
+
+// four floats of the shared memory of cluster rank `rank` at this block's address `addr`
+__device__ __forceinline__ float4 ld_peer_f4(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  float4 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(r)
+               : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void peers_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void peers_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 template <int E, int BN, int KS, int KP = 2>
 __device__ __forceinline__ void frac_tc_tile(const TcMaps& maps, const TcParams& P, int block, uint8_t* smem_raw) {
@@ -147,26 +167,37 @@ __device__ __forceinline__ void frac_tc_tile(const TcMaps& maps, const TcParams&
     }
   }
   __syncwarp();
-  if (warp >= 4) return;  // tf32's extra splitting warps: the epilogue is warps 0-3
 
   // ---------------- epilogue
-  bool have = mbar_wait(done, 0, P.flag);
+  const bool have = mbar_wait(done, 0, P.flag);
   tc_fence_after();
   float* tile = reinterpret_cast<float*>(smem);  // the operand ring is idle once `done` fired
-  const int row = threadIdx.x;                   // accumulator lane = x offset in the tile
-  const uint32_t lane_addr = tmem + (static_cast<uint32_t>(warp * 32) << 16);
-  int r0 = 0, r1 = BN;  // tile rows (output nodes n) this CTA writes
-  // KS > 1: this CTA's partial sum over its k-range goes to partial slot `rank` of F
-  // (F is [rank][axis][node]); the consumers add the KS partials in rank order
+  const int row = (warp & 3) * 32 + (threadIdx.x & 31);  // accumulator lane = x offset in the tile
+  const uint32_t lane_addr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
   const long long nodes = P.nodes;
-  float* F = P.F + (long long)rank * P.naxes * nodes + (long long)mu * nodes;
+  float* F = P.F + (long long)mu * nodes;
   const int n0 = P.n0, n1 = P.n1;
   const int lim = (mu == 0) ? n1 : ax.side;  // output rows that exist
-  // TMEM -> shared tile [BN][128] (lane = x), 32 rows at a time; with TMA stores each
-  // 32-row chunk leaves by its own store as soon as it is in shared memory, so the stores
-  // overlap the drain of the next chunk (each chunk has its own 16 KB of the tile)
+  const bool slots = KS > 1 && P.slots;      // partial tiles stay in slots of F
+  auto store_rows = [&](int c0) {            // the box of the F map: 32 rows, or BN / KS if fewer
+    const int c1 = mu == 2 ? m_out : ncol0 + c0, c2 = mu == 2 ? ncol0 + c0 : m_out;
+    if (slots)
+      asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
+                       reinterpret_cast<uint64_t>(&maps.f[mu])),
+                   "r"(m_in), "r"(c1), "r"(c2), "r"(rank), "r"(smem_u32(tile + c0 * BM))
+                   : "memory");
+    else
+      asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+                     reinterpret_cast<uint64_t>(&maps.f[mu])),
+                 "r"(m_in), "r"(c1), "r"(c2), "r"(smem_u32(tile + c0 * BM))
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+  };
+  // TMEM -> shared tile [BN][128] (lane = x), 32 rows at a time, two chunks in flight (warps
+  // 0-3 and 4-7); unsplit tiles leave by one TMA store per chunk as soon as it is in shared
+  // memory, so the stores overlap the drain of the next chunk
 #pragma unroll 1
-  for (int c0 = 0; c0 < BN; c0 += 32) {
+  for (int c0 = 32 * (warp >> 2); c0 < BN; c0 += 64) {
     float v[32], w[32];
     tmem_ld32(lane_addr + c0, v);
     for (int r = 1; r < nreg; ++r) {  // the regions, added in k order
@@ -176,51 +207,66 @@ __device__ __forceinline__ void frac_tc_tile(const TcMaps& maps, const TcParams&
     }
 #pragma unroll
     for (int j = 0; j < 32; ++j) tile[(c0 + j) * BM + row] = have ? v[j] : 0.0f;
+    if ((KS == 1 || slots) && P.tma_store) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + (warp >> 2)) : "memory");  // the four warps of this chunk
+      if ((threadIdx.x & 127) == 0 && have && ncol0 + c0 < lim) store_rows(c0);
+    }
+  }
+  int r0 = 0, r1 = BN;  // tile rows (output nodes n) this CTA stores
+  if (KS > 1 && !slots) {
+    // split contraction: the KS partial tiles of the cluster, added in rank order; CTA `rank`
+    // sums and stores its share of the rows.  (Every thread of every CTA reaches both cluster
+    // barriers, also after a wait that gave up.)
+    constexpr int RP = BN / KS;
+    r0 = rank * RP;
+    r1 = r0 + RP;
+    peers_arrive();
+    peers_wait();
+    const uint32_t base = smem_u32(tile);
+#pragma unroll
+    for (int e = threadIdx.x; e < RP * (BM / 4); e += kTileThreads) {
+      const uint32_t off = 4u * (r0 * BM + 4 * e);
+      float4 v[KS];
+#pragma unroll
+      for (int q = 0; q < KS; ++q) v[q] = ld_peer_f4(base + off, q);
+#pragma unroll
+      for (int q = 1; q < KS; ++q) {
+        v[0].x += v[q].x;
+        v[0].y += v[q].y;
+        v[0].z += v[q].z;
+        v[0].w += v[q].w;
+      }
+      *reinterpret_cast<float4*>(reinterpret_cast<uint8_t*>(tile) + off) = v[0];  // only this CTA reads its own rows
+    }
+    peers_arrive();  // this thread is done with the peers' tiles
     if (P.tma_store) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      named_sync128();  // warps 0-3 (tf32's extra warps have left)
-      if (threadIdx.x == 0 && have && ncol0 + c0 < lim) {
-        int c1, c2;
-        if (mu == 2) {
-          c1 = m_out;
-          c2 = ncol0 + c0;
-        } else {
-          c1 = ncol0 + c0;
-          c2 = m_out;
-        }
-        if (KS == 1)
-          asm volatile(
-              "cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
-                  reinterpret_cast<uint64_t>(&maps.f[mu])),
-              "r"(m_in), "r"(c1), "r"(c2), "r"(smem_u32(tile + c0 * BM))
-              : "memory");
-        else
-          asm volatile(
-              "cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
-                  reinterpret_cast<uint64_t>(&maps.f[mu])),
-              "r"(m_in), "r"(c1), "r"(c2), "r"(rank), "r"(smem_u32(tile + c0 * BM))
-              : "memory");
-        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-      }
+      __syncthreads();
+      constexpr int BOX = RP < 32 ? RP : 32;
+      if (threadIdx.x == 0 && have)
+        for (int c0 = r0; c0 < r1 && ncol0 + c0 < lim; c0 += BOX) store_rows(c0);
     }
   }
   if (P.tma_store) {
-    if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    // the stores have read the tile (the grid's end makes them visible)
+    if ((threadIdx.x & 127) == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   } else {
     // rows of F that are not 16-byte aligned: plain stores, coalesced along x
-    named_sync128();  // warps 0-3 (tf32's extra warps have left)
-    const int x = m_in + row;
+    __syncthreads();
+    const int xo = threadIdx.x & 127, x = m_in + xo;
     if (have && x < n0) {
-      for (int rr = r0; rr < r1; ++rr) {
+      for (int rr = r0 + (threadIdx.x >> 7); rr < r1; rr += 2) {
         const int n = ncol0 + rr;  // x axis: row y at z = m_out; y/z axes: node along mu
         if (n >= lim) break;
         const long long idx = (mu == 2) ? ((long long)n * n1 + m_out) * n0 + x : ((long long)m_out * n1 + n) * n0 + x;
-        F[idx] = tile[(rr - r0) * BM + row];
+        F[idx] = tile[rr * BM + xo];
       }
     }
   }
+  if (KS > 1 && !slots) peers_wait();  // the peers have read this CTA's tile
   tc_fence_before();
-  named_sync128();  // warps 0-3 (tf32's extra warps have left)
+  __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(nreg * BN) : "memory");
@@ -229,7 +275,7 @@ __device__ __forceinline__ void frac_tc_tile(const TcMaps& maps, const TcParams&
 }
 
 template <int E, int BN, int KS, int KP>
-__global__ void __launch_bounds__(tile_threads(E), 1)
+__global__ void __launch_bounds__(kTileThreads, 1)
 frac_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams P) {
   extern __shared__ uint8_t smem_raw[];
   frac_tc_tile<E, BN, KS, KP>(maps, P, blockIdx.x, smem_raw);
@@ -676,14 +722,17 @@ cudaError_t launch_kernel(const TcPlan* p, cudaStream_t s) {
   if (const cudaError_t e = smem_attr_once(attr, frac_tc_kernel<E, BN, KS, KP>, (int)Cfg<E, BN, KS, KP>::SMEM); e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p->prm.total_tiles * KS, 1, 1);
-  cfg.blockDim = dim3(tile_threads(E), 1, 1);
+  cfg.blockDim = dim3(kTileThreads, 1, 1);
   cfg.dynamicSmemBytes = Cfg<E, BN, KS, KP>::SMEM;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = p->pdl ? 1 : 0;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = KS;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = KS > 1 && !p->prm.slots ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, frac_tc_kernel<E, BN, KS, KP>, p->maps, p->prm);
 }
 
@@ -824,7 +873,6 @@ int tc_prepare(lbm_s* h, const std::vector<std::vector<double>>& K, int force_bn
     p->koff[mu] = koff[mu];
   }
   if (int rc = tc_set_weights(h, K)) return rc;
-  p->f_elems = (size_t)h->d * h->sp.nodes;
 
   // default plan: column tiles of 128 (an M = 128 MMA costs the same for any N <= 128)
   // or 256 when that still fills the GPU; small problems split the contraction over up
@@ -833,9 +881,19 @@ int tc_prepare(lbm_s* h, const std::vector<std::vector<double>>& K, int force_bn
   const int kSMs = device_sms();
   int bn = (p->kparts == 2 && tc_count_tiles(h, 256) >= kSMs) ? 256 : 128;
   const int kbmin = tc_kbmin(h);
-  int ks = 1;
-  const long long nt = tc_count_tiles(h, bn);
-  while (ks * 2 <= 8 && ks * 2 <= kbmin && nt * ks * 2 <= kSMs) ks *= 2;
+  auto split = [&](long long tiles) {
+    int k = 1;
+    while (k * 2 <= 8 && k * 2 <= kbmin && tiles * k * 2 <= kSMs) k *= 2;
+    return k;
+  };
+  int ks = split(tc_count_tiles(h, bn));
+  // 64-column tiles where they put more CTAs to work (small and ragged grids; measured:
+  // 256^2 bf16x6 step 8.7 us with 128 columns, 8.1 with 64, 301 x 203 10.6 and 9.9)
+  const long long t64 = tc_count_tiles(h, 64);
+  if (bn == 128 && t64 * split(t64) <= kSMs && t64 * split(t64) > tc_count_tiles(h, 128) * ks) {
+    bn = 64;
+    ks = split(t64);
+  }
   bool persist = false;
   if (force_bn > 0) {
     bn = force_bn;
@@ -868,8 +926,26 @@ int tc_kbmin(const lbm_s* h) {
   return kbmin;
 }
 
+// tensor maps of the fractional terms F_mu, boxes of 128 x and `rows` output rows; slots > 1:
+// [slot][axis][node] with the slot as a fourth coordinate
+static bool encode_F(const lbm_s* h, float* F, int slots, int rows, TcMaps* maps) {
+  const int* n = h->sp.n;
+  EncodeTiled enc = get_encoder();
+  for (int mu = 0; enc && mu < h->d; ++mu) {
+    const cuuint64_t fd[4] = {(cuuint64_t)n[0], (cuuint64_t)n[1], (cuuint64_t)n[2], (cuuint64_t)slots};
+    const cuuint64_t fs[3] = {(cuuint64_t)n[0] * 4, (cuuint64_t)n[0] * n[1] * 4, (cuuint64_t)h->d * h->sp.nodes * 4};
+    const cuuint32_t fb[4] = {BM, mu == 2 ? 1u : (cuuint32_t)rows, mu == 2 ? (cuuint32_t)rows : 1u, 1u};
+    const cuuint32_t es[4] = {1, 1, 1, 1};
+    if (enc(&maps->f[mu], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, slots > 1 ? 4 : 3, F + (size_t)mu * h->sp.nodes, fd, fs, fb,
+            es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return false;
+  }
+  return enc != nullptr;
+}
+
 // (Re)plan the operator: column tile width bn, contraction split ks, persistent or per
-// tile; re-encodes every tensor map and grows the F buffer when the split needs it.
+// tile; re-encodes every tensor map.
 int tc_replan(lbm_s* h, int bn, int ks, int persist) {
   TcPlan* p = h->tc;
   if (!p) return LBM_EINVAL;
@@ -956,37 +1032,21 @@ int tc_replan(lbm_s* h, int bn, int ks, int persist) {
         !encode(&p->maps.k_l2[mu], E, 2, static_cast<uint8_t*>(h->dev.Kl2) + koff[mu] * E, kdims, kstr, kbox))
       return LBM_ECUDA;
   }
-  // split contraction: F holds one partial sum per rank, [rank][axis][node]; the
-  // kernels that read F add them in rank order
-  const size_t need = (size_t)ks * h->d * h->sp.nodes;
-  if (need > p->f_elems) {
+  P.F = static_cast<float*>(h->dev.F);
+  // row chunks of an output tile: what one CTA of a cluster stores, at most 32 rows
+  P.slots = ks > 1 && h->d == 2 && P.tma_store ? 1 : 0;
+  const size_t need = (size_t)(P.slots ? ks : 1) * h->d * h->sp.nodes;
+  if (need > h->f_elems) {
+    cudaStreamSynchronize(h->stream);
     dev_free(h, h->dev.F);
     h->dev.F = nullptr;
-    p->f_elems = 0;
+    h->f_elems = 0;
     if (dev_alloc(h, (void**)&h->dev.F, need * 4) != cudaSuccess) return LBM_ENOMEM;
-    p->f_elems = need;
+    h->f_elems = need;
+    P.F = static_cast<float*>(h->dev.F);
   }
-  P.F = static_cast<float*>(h->dev.F);
-  h->sp.ksum = ks;
-  h->sp.pstride = (ks > 1) ? (long long)h->d * h->sp.nodes : 0;
-  if (P.tma_store) {
-    for (int mu = 0; mu < h->d; ++mu) {
-      // 32-row chunks of an output tile (per tile: of one rank's partial when ks > 1)
-      const cuuint32_t rows = 32u;
-      const cuuint64_t fd[4] = {(cuuint64_t)n[0], (cuuint64_t)n[1], (cuuint64_t)n[2], (cuuint64_t)ks};
-      const cuuint64_t fs[3] = {(cuuint64_t)n[0] * 4, (cuuint64_t)n[0] * n[1] * 4,
-                                (cuuint64_t)h->d * h->sp.nodes * 4};
-      const cuuint32_t fb[4] = {BM, mu == 2 ? 1u : rows, mu == 2 ? rows : 1u, 1u};
-      const cuuint32_t es[4] = {1, 1, 1, 1};
-      EncodeTiled enc = get_encoder();
-      if (!enc) return LBM_ECUDA;
-      CUresult r = enc(&p->maps.f[mu], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, ks > 1 ? 4 : 3,
-                       static_cast<float*>(h->dev.F) + (size_t)mu * h->sp.nodes, fd, fs, fb, es,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-      if (r != CUDA_SUCCESS) return LBM_ECUDA;
-    }
-  }
+  h->sp.ksum = P.slots ? ks : 1;
+  if (P.tma_store && !encode_F(h, P.F, h->sp.ksum, P.slots ? 32 : std::min(32, bn / ks), &p->maps)) return LBM_ECUDA;
   P.total_tiles = tiles;
   P.early_trigger = (tiles * ks <= kSMs) ? 1 : 0;
   return LBM_OK;

@@ -25,10 +25,7 @@ struct StepParams {
   double w0, wi;             // lattice weights: rest and moving (Fig. 1 caption)
   double adv[3];             // (dt/dx) u_mu / e^2: advective factor of Eq. (Feq)
   double C_wall;             // Dirichlet value (Eq. Dirichlet_BC)
-  // fractional terms held as ksum partial sums over the contraction (split-K operator):
-  // F_mu(node) = sum_{s < ksum} F[s * pstride + mu * nodes + node], added in order of s
-  int ksum;
-  long long pstride;
+  int ksum = 1;              // F holds ksum partial sums, [rank][axis][node], added in order (2-D, tensor cores)
   double sfree[3];           // MRT rates of the free moments (Eq. MatrixS)
 };
 
@@ -103,6 +100,7 @@ struct lbm_s {
   cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};
   int graph_steps = 0;                 // steps per captured graph (even)
   int launches_per_step = 0;
+  size_t f_elems = 0;                  // capacity of dev.F (elements)
   int simt_ks = 1;                     // contraction split of the FP32 SIMT operator (blocks per cluster)
   // programmatic dependent launch between the operator and collide-stream: only when both
   // grids run in a single wave (measured: with multi-wave 3-D grids it costs ~30%)

@@ -28,8 +28,9 @@ struct TcParams {
   int n0, n1, n2;
   int naxes;
   int total_tiles;
-  int ksplit;     // CTAs per output tile, each contracting a k-range into its own partial
+  int ksplit;     // CTAs per output tile (one cluster), each contracting a k-range
   int tma_store;  // F rows are 16-byte aligned (n0 % 4 == 0): store tiles with TMA
+  int slots;      // ksplit > 1 without a cluster: the partial tiles go to F as [rank][axis][node]
   int early_trigger;  // the per-tile grid fits in one wave: release dependents after the prologue
   long long nodes;
   TcAxis ax[3];
@@ -42,7 +43,7 @@ struct TcMaps {
   CUtensorMap c_l2[3];           // third part of C (six-product bf16 form only)
   CUtensorMap k_hi[3], k_lo[3];  // K_mu split; box BK x 128 for the x axis (A), BK x BN else (B)
   CUtensorMap k_l2[3];           // third part of K_mu (five- and six-product bf16 forms)
-  CUtensorMap f[3];              // F_mu (FP32), box 128 x (BN / ksplit) output rows
+  CUtensorMap f[3];              // F_mu (FP32), box 128 x min(32, BN / ksplit) output rows
 };
 
 struct TcPlan {
@@ -56,7 +57,6 @@ struct TcPlan {
   bool pdl = false;      // launch with programmatic stream serialization (the handle's choice)
   int ldk[3] = {0, 0, 0};     // padded row pitch of K_mu's split parts (elements)
   size_t koff[3] = {0, 0, 0}; // offset of K_mu's split parts (elements)
-  size_t f_elems = 0;         // capacity of the F buffer (floats)
   size_t smem = 0;
   int ldp = 0;       // padded x pitch of the C split arrays (elements)
   // tf32 only: C (FP32, split into tf32 hi + lo by the operator in shared memory) regrouped
