@@ -1024,7 +1024,7 @@ int lbm_autotune(lbm_t h, int nsteps, char* desc, int desc_len) {
   // candidate chunks
   std::vector<int> chunks;
   if (h->is_batch()) {
-    chunks = {2, 4, 8, 16};
+    chunks = {2, 4, 8, 16, 32};
   } else if (h->d == 2) {
     const int by = (h->sp.n[1] + 15) / 16;
     for (int c : {1, 2, 3, 4, 8}) if (c <= by) chunks.push_back(c);

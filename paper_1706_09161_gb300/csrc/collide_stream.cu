@@ -285,17 +285,15 @@ struct SplitOut {
 
 // Per-problem entry of a grouped (batched) collide-stream launch.
 struct BatchCS {
-  CUtensorMap mf[2];  // 2-D members with n0 % 4 == 0: population windows (see march2_tma)
-  CUtensorMap mF;     //   and fractional-term windows
   KConst<float> k;
   const float* f[2];  // population buffers; the launch's parity picks input and output
   const float* F;
   float* C;
   SplitOut so;
   int* flag;
-  double* mpart;       // the problem's mass partials, one per block of it
-  int bx, by, zchunk;  // blocks in x, y and the z chunk length (2-D: tile rows per block)
-  int tma;             // the maps above are valid
+  double* mpart;              // the problem's mass partials, one per warp
+  int v, strips, rows, items; // 2-D: strip march (StripGrid)
+  int bx;                     // 3-D: tile columns in x
 };
 
 // SPLIT: 1 = bf16 hi + lo, 3 = bf16 in three parts (each the rounding of what the previous
@@ -688,6 +686,222 @@ __device__ __forceinline__ void march2_pipe(const KConst<float>& sp, const float
   }
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(flag, 1);
   block_mass(macc, mpart, mslot);
+}
+
+// ---------------------------------------------------------------------------- 2-D FP32 strip march
+// One warp owns a strip of 32 V nodes along x (V = 2 adjacent nodes per lane where rows are
+// whole 8-byte pairs, else 1) and marches up a chunk of rows, colliding every row once: the y
+// movers (e_3, e_4) stay in registers (previous row's f*_3, next row's f*_4), the x movers
+// (e_1, e_2) go to the neighbouring lane by shuffle, and the strip's two ring columns are
+// collided 16 rows at a time, one node per lane.  No shared memory, no barrier and no block:
+// warps are independent, each with the next two rows' loads in flight.  A chunk of R rows
+// collides (R + 2) / R + 1 / (32 V) of its nodes.  Serves the batches, where there are rows
+// enough to keep every SM's warps busy (16 problems of 128^2 to 1024^2: 69 us with the TMA-fed
+// blocks of 19 warps, 335 instructions per node; 59 us and 165 here); a single 512^2 lattice is a chain of
+// latencies in which the TMA-fed blocks are the faster form (512^2 bf16x6 step 12.4 us against
+// 13.4 us with strips of two rows).
+template <int V>
+struct StripRow {
+  float f[5][V], F[2][V];
+};
+
+template <int V>
+__device__ __forceinline__ void load_v(float (&d)[V], const float* __restrict__ p) {
+  if constexpr (V == 2) {
+    const float2 t = *reinterpret_cast<const float2*>(p);
+    d[0] = t.x;
+    d[1] = t.y;
+  } else {
+    d[0] = *p;
+  }
+}
+
+template <int V>
+__device__ __forceinline__ void store_v(float* __restrict__ p, const float (&d)[V]) {
+  if constexpr (V == 2) *reinterpret_cast<float2*>(p) = make_float2(d[0], d[1]);
+  else *p = d[0];
+}
+
+// the values of V neighbouring nodes from offset `o` on, zeros where !ok
+template <int V>
+__device__ __forceinline__ void strip_load(long long nodes, const float* __restrict__ f, const float* __restrict__ F,
+                                           long long o, bool ok, StripRow<V>& r) {
+  if (ok) {
+#pragma unroll
+    for (int q = 0; q < 5; ++q) load_v<V>(r.f[q], f + q * nodes + o);
+#pragma unroll
+    for (int mu = 0; mu < 2; ++mu) load_v<V>(r.F[mu], F + mu * nodes + o);
+  } else {
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+#pragma unroll
+      for (int q = 0; q < 5; ++q) r.f[q][v] = 0.f;
+      r.F[0][v] = r.F[1][v] = 0.f;
+    }
+  }
+}
+
+// equilibrium and collision of the V nodes of a loaded row
+template <int V, bool MRT, bool KS>
+__device__ __forceinline__ void strip_collide(const KConst<float>& sp, const StripRow<V>& r, float (&fs)[5][V]) {
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    float f[5], o[5];
+    const float F[2] = {r.F[0][v], r.F[1][v]};
+#pragma unroll
+    for (int q = 0; q < 5; ++q) f[q] = r.f[q][v];
+    collide_node<float, 2, MRT, KS>(sp, f, F, o);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) fs[q][v] = o[q];
+  }
+}
+
+// bf16 operand parts of V neighbouring values at element o (write_split of each, packed stores)
+template <int SPLIT, int V>
+__device__ __forceinline__ void write_split_v(const SplitOut& so, long long o, const float (&c)[V]) {
+  static_assert(SPLIT == 1 || SPLIT == 3, "bf16 forms");
+  if constexpr (V == 1) {
+    write_split<SPLIT>(so, o, c[0]);
+  } else {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(c[0], c[1]);
+    const float r0 = c[0] - __low2float(h), r1 = c[1] - __high2float(h);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(r0, r1);
+    *reinterpret_cast<__nv_bfloat162*>(static_cast<__nv_bfloat16*>(so.hi) + o) = h;
+    *reinterpret_cast<__nv_bfloat162*>(static_cast<__nv_bfloat16*>(so.lo) + o) = l;
+    if constexpr (SPLIT == 3)
+      *reinterpret_cast<__nv_bfloat162*>(static_cast<__nv_bfloat16*>(so.lo2) + o) =
+          __floats2bfloat162_rn(r0 - __low2float(l), r1 - __high2float(l));
+  }
+}
+
+// the warp's strip (nodes x0 .. x0 + 32 V - 1), rows y0 .. y1 - 1; its mass partial to mpart[slot]
+template <int V, bool MRT, int SPLIT, bool KS>
+__device__ __forceinline__ void strip_march(const KConst<float>& sp, const float* __restrict__ f_in,
+                                            const float* __restrict__ F, float* __restrict__ f_out,
+                                            float* __restrict__ C_out, int* __restrict__ flag, const SplitOut& so,
+                                            int x0, int y0, int y1, double* mpart, int slot) {
+  const int n0 = sp.n[0], n1 = sp.n[1], lane = threadIdx.x & 31;
+  const long long nodes = sp.nodes;
+  const int gx = x0 + V * lane;
+  const bool in_x = gx < n0;  // (n0 is a multiple of V)
+  const bool side = x0 == 0 || x0 + 32 * V >= n0;
+  StripRow<V> row[2];
+  auto load = [&](int y, StripRow<V>& r) {
+    strip_load<V>(nodes, f_in, F, (long long)y * n0 + gx, in_x && y >= 0 && y < n1, r);
+  };
+  load(y0 - 1, row[0]);
+  load(y0, row[1]);
+  // ring columns of rows yb .. yb + 15: lane r the left column's f*_1 of row yb + r, lane 16 + r
+  // the right column's f*_2
+  float h = 0.f;
+  auto ring = [&](int yb) {
+    const int hx = lane < 16 ? x0 - 1 : x0 + 32 * V, hy = yb + (lane & 15);
+    StripRow<1> r;
+    float o[5][1];
+    strip_load<1>(nodes, f_in, F, (long long)hy * n0 + hx, hx >= 0 && hx < n0 && hy < y1, r);
+    strip_collide<1, MRT, KS>(sp, r, o);
+    h = lane < 16 ? o[1][0] : o[2][0];
+  };
+  ring(y0);
+  SumAcc<float> macc;
+  float bad = 0.f;
+  float c[4][V], p3[V];  // f*_0..3 of the last collided row, f*_3 of the one before
+#pragma unroll
+  for (int v = 0; v < V; ++v) c[0][v] = c[1][v] = c[2][v] = c[3][v] = p3[v] = 0.f;
+  auto advance = [&](int y, StripRow<V>& r) {
+    float n[5][V];
+    strip_collide<V, MRT, KS>(sp, r, n);
+    if (y + 2 <= y1) load(y + 2, r);
+    const int yo = y - 1;  // the row that is complete now
+    if (yo >= y0) {
+      const int k = (yo - y0) & 15;
+      if (yo > y0 && k == 0) ring(yo);
+      const float hl = __shfl_sync(0xffffffffu, h, k), hr = __shfl_sync(0xffffffffu, h, 16 + k);
+      const float up = __shfl_up_sync(0xffffffffu, c[1][V - 1], 1), dn = __shfl_down_sync(0xffffffffu, c[2][0], 1);
+      float o[5][V], C[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        o[0][v] = c[0][v];
+        o[1][v] = v == 0 ? (lane == 0 ? hl : up) : c[1][v > 0 ? v - 1 : 0];
+        o[2][v] = v == V - 1 ? (lane == 31 ? hr : dn) : c[2][v < V - 1 ? v + 1 : 0];
+        o[3][v] = p3[v];
+        o[4][v] = n[4][v];
+        C[v] = 0.f;
+      }
+      if (!side && yo > 0 && yo + 1 < n1) {  // no wall within reach (warp-uniform)
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+#pragma unroll
+          for (int q = 0; q < 5; ++q) C[v] += o[q][v];
+      } else {
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          const bool known[5] = {true, gx + v > 0, gx + v + 1 < n0, yo > 0, yo + 1 < n1};
+          int n_unknown = 0;
+#pragma unroll
+          for (int q = 0; q < 5; ++q) {
+            if (known[q]) {
+              C[v] += o[q][v];
+            } else {
+              o[q][v] = 0.f;
+              ++n_unknown;
+            }
+          }
+          if (n_unknown > 0) {
+            // Eq. (Dirichlet_BC); with k unknown populations each takes 1/k of the deficit
+            const float fill = (sp.C_wall - C[v]) / static_cast<float>(n_unknown);
+#pragma unroll
+            for (int q = 0; q < 5; ++q)
+              if (!known[q]) o[q][v] = fill;
+            C[v] = o[0][v];
+#pragma unroll
+            for (int q = 1; q < 5; ++q) C[v] += o[q][v];
+          }
+        }
+      }
+      if (in_x) {
+        const long long node = (long long)yo * n0 + gx;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) store_v<V>(f_out + q * nodes + node, o[q]);
+        store_v<V>(C_out + node, C);
+        if constexpr (SPLIT != 0) write_split_v<SPLIT, V>(so, (long long)yo * so.ldp + gx, C);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          bad = __fmaf_rn(C[v], 0.f, bad);  // NaN once a C is not finite
+          macc.add(C[v]);
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      p3[v] = c[3][v];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) c[q][v] = n[q][v];
+    }
+  };
+  for (int y = y0 - 1; y <= y1; y += 2) {
+    advance(y, row[0]);
+    if (y + 1 <= y1) advance(y + 1, row[1]);
+  }
+  if (__any_sync(0xffffffffu, bad != 0.f) && lane == 0) atomicOr(flag, 1);
+  macc.warp_reduce();
+  if (lane == 0 && mpart) macc.store(mpart + slot);
+}
+
+// rows of a chunk: kStripRows per unit of the tunable chunk
+constexpr int kStripRows = 2, kStripWarps = 4;
+
+// how a 2-D problem's nodes are dealt to warps: item = chunk * strips + strip
+struct StripGrid {
+  int v, strips, rows, items;
+};
+StripGrid strip_grid(const int* n, int chunk) {
+  StripGrid g;
+  g.v = n[0] % 2 == 0 ? 2 : 1;
+  g.strips = (n[0] + 32 * g.v - 1) / (32 * g.v);
+  g.rows = std::min(kStripRows * chunk, n[1]);
+  g.items = g.strips * ((n[1] + g.rows - 1) / g.rows);
+  return g;
 }
 
 // linear index of this block in its grid (the slot of its mass partial)
@@ -1348,40 +1562,37 @@ cudaError_t fused_launch(const lbm_s* h, int nsteps, int grid, cudaStream_t s) {
                             h->cs_part);
 }
 
-// 2-D batch blocks run either march (per problem): room for the larger ring
-constexpr int BATCH2_SMEM = (int)(TMA2_SMEM > (size_t)PIPE_SMEM ? TMA2_SMEM : (size_t)PIPE_SMEM);
-
 // Grouped form for a batch of independent problems: one launch covers every block of
 // every problem; block_map[b] = (problem, block within it), one load per block.  The
 // problem's constants are staged in shared memory.
+__host__ __device__ constexpr int batch_threads(int d) { return d == 2 ? 32 * kStripWarps : NT; }
+
 template <int D, bool MRT, int SPLIT>
-__global__ void __launch_bounds__(TX*(TY + HALO_WARPS), 2)
+__global__ void __launch_bounds__(batch_threads(D), D == 2 ? 4 : 2)
 collide_stream_batch_kernel(const BatchCS* __restrict__ tab, const int2* __restrict__ block_map, int parity) {
   __shared__ KConst<float> s_k;
   const int2 pb = __ldg(&block_map[blockIdx.x]);
   const BatchCS& e = tab[pb.x];
   const int tid = threadIdx.y * TX + threadIdx.x;
   constexpr int words = sizeof(KConst<float>) / sizeof(int);
-  for (int i = tid; i < words; i += TX * (TY + HALO_WARPS))
+  for (int i = tid; i < words; i += batch_threads(D))
     reinterpret_cast<int*>(&s_k)[i] = reinterpret_cast<const int*>(&e.k)[i];
   if (D == 2 && MRT && tid < kMaxQ * 8) {
     const int r = tid >> 3, c = tid & 7;
     reinterpret_cast<float*>(&s_om_rows[r][0])[c] = c < kMaxQ ? e.k.omega[r][c] : 0.0f;
   }
   __syncthreads();
-  const int lb = pb.y;
-  const int bx = lb % e.bx, rest = lb / e.bx;
+  float* fo = const_cast<float*>(e.f[parity ^ 1]);
   if constexpr (D == 2) {
-    extern __shared__ __align__(128) uint8_t batch_raw[];
-    if (e.tma)
-      march2_tma<MRT, SPLIT, true>(s_k, &e.mf[parity], &e.mF, const_cast<float*>(e.f[parity ^ 1]), e.C, e.flag, e.so,
-                             e.zchunk, bx, rest, batch_raw, e.mpart, lb);
-    else
-      march2_pipe<MRT, SPLIT, true>(s_k, e.f[parity], e.F, const_cast<float*>(e.f[parity ^ 1]), e.C, e.flag, e.so,
-                              e.zchunk, bx, rest, reinterpret_cast<float*>(batch_raw), e.mpart, lb);
+    const int item = pb.y * kStripWarps + (tid >> 5);
+    if (item < e.items) {
+      const int x = item % e.strips * 32 * e.v, y0 = item / e.strips * e.rows, y1 = min(y0 + e.rows, s_k.n[1]);
+      if (e.v == 2) strip_march<2, MRT, SPLIT, true>(s_k, e.f[parity], e.F, fo, e.C, e.flag, e.so, x, y0, y1, e.mpart, item);
+      else strip_march<1, MRT, SPLIT, true>(s_k, e.f[parity], e.F, fo, e.C, e.flag, e.so, x, y0, y1, e.mpart, item);
+    }
   } else {
-    march_body<float, D, MRT, SPLIT>(s_k, e.f[parity], e.F, const_cast<float*>(e.f[parity ^ 1]), e.C, e.flag, e.so,
-                                     bx, rest, 0, e.k.n[2], e.mpart, lb);
+    march_body<float, D, MRT, SPLIT>(s_k, e.f[parity], e.F, fo, e.C, e.flag, e.so, pb.y % e.bx, pb.y / e.bx, 0,
+                                     e.k.n[2], e.mpart, pb.y);
   }
 }
 
@@ -1709,7 +1920,7 @@ cudaError_t launch_collide_stream(const lbm_s* h, const void* f_in, void* f_out,
              : launch_cs<float, 3, false>(h, f_in, f_out, C_out, s, tk, slot);
 }
 
-constexpr int kBatchYChunk = 16;  // tile rows per block (the autotuner's usual choice on mixed batches)
+constexpr int kBatchChunk = 4;  // units of kStripRows per warp
 
 // window map of `planes` fields (x fastest, `base` their first) for the TMA-fed marches:
 // (n0, n1, planes) in 2-D, (n0, n1, n2, planes) in 3-D
@@ -1808,7 +2019,7 @@ bool cs_one_wave(const lbm_s* h) {
 }
 
 long long cs_max_parts(const lbm_s* h) {
-  long long most = 0;
+  long long most = h->d == 2 && h->elem == 4 ? strip_grid(h->sp.n, 1).items : 0;
   for (int t = 0; t < (h->elem == 8 ? 3 : 1); ++t) {  // one block per tile and plane at most
     const long long bx = (h->sp.n[0] + kTile64[t][0] - 1) / kTile64[t][0], by = (h->sp.n[1] + kTile64[t][1] - 1) / kTile64[t][1];
     most = std::max(most, march_warps(kTile64[t][0], kTile64[t][1]) * bx * by * h->sp.n[2]);
@@ -1818,7 +2029,7 @@ long long cs_max_parts(const lbm_s* h) {
 
 int cs_chunk_default(const lbm_s* h) {
   const int bx = (h->sp.n[0] + TX - 1) / TX, by = (h->sp.n[1] + TY - 1) / TY;
-  if (h->is_batch()) return kBatchYChunk;
+  if (h->is_batch()) return kBatchChunk;
   if (h->d == 2) return h->elem == 4 ? ychunk_for((long long)bx * by, by) : 1;
   return h->elem == 8 ? march64_plan(h, 0).nz : z_chunks((long long)bx * by, h->sp.n[2]);
 }
@@ -1841,13 +2052,17 @@ int cs_batch_prepare(lbm_s* b) {
     e.so.lo2 = h->dev.Cl2;
     e.flag = h->dev.flag;
     e.mpart = h->cs_part;
-    e.tma = (h->d == 2 && h->sp.n[0] % 4 == 0 && encode_maps(h, e.mf, &e.mF)) ? 1 : 0;
     e.bx = (h->sp.n[0] + TX - 1) / TX;
-    e.by = (h->sp.n[1] + TY - 1) / TY;
-    // 2-D: tile rows per block (the pipelined y-march); 3-D: the whole z extent
-    e.zchunk = (h->d == 2) ? std::min(e.by, b->cs_chunk > 0 ? b->cs_chunk : kBatchYChunk) : h->sp.n[2];
-    const int blocks = e.bx * ((h->d == 2) ? (e.by + e.zchunk - 1) / e.zchunk : e.by);
+    int blocks = e.bx * ((h->sp.n[1] + TY - 1) / TY);  // 3-D: one column each, the whole z extent
     h->cs_nparts = kMassSlots * blocks;
+    if (h->d == 2) {
+      const StripGrid g = strip_grid(h->sp.n, b->cs_chunk > 0 ? b->cs_chunk : kBatchChunk);
+      e.v = g.v;
+      e.strips = g.strips;
+      e.rows = g.rows;
+      e.items = h->cs_nparts = g.items;
+      blocks = (g.items + kStripWarps - 1) / kStripWarps;
+    }
     for (int k = 0; k < blocks; ++k) map.push_back(make_int2(i, k));
     total += blocks;
   }
@@ -1870,22 +2085,10 @@ cudaError_t launch_collide_stream_batch(const lbm_s* b, int parity, cudaStream_t
   const int split = cs_split_code(h0);  // 0, 1 or 3 (batches have no tf32 form)
   const BatchCS* tab = static_cast<const BatchCS*>(b->batch_cs);
   const int P = static_cast<int>(b->subs.size());
-  dim3 block(TX, TY + HALO_WARPS);
+  const dim3 block(TX, batch_threads(h0->d) / TX);
   const int g = b->batch_cs_blocks;
-  const int smem = (h0->d == 2) ? BATCH2_SMEM : 0;
-  if (h0->d == 2) {
-    static std::atomic<unsigned long long> attr[2][4] = {{{0}, {0}, {0}, {0}}, {{0}, {0}, {0}, {0}}};
-    cudaError_t e;
-    if (mrt) e = split == 3 ? smem_attr_once(attr[1][3], collide_stream_batch_kernel<2, true, 3>, BATCH2_SMEM)
-                 : split    ? smem_attr_once(attr[1][1], collide_stream_batch_kernel<2, true, 1>, BATCH2_SMEM)
-                            : smem_attr_once(attr[1][0], collide_stream_batch_kernel<2, true, 0>, BATCH2_SMEM);
-    else e = split == 3 ? smem_attr_once(attr[0][3], collide_stream_batch_kernel<2, false, 3>, BATCH2_SMEM)
-             : split    ? smem_attr_once(attr[0][1], collide_stream_batch_kernel<2, false, 1>, BATCH2_SMEM)
-                        : smem_attr_once(attr[0][0], collide_stream_batch_kernel<2, false, 0>, BATCH2_SMEM);
-    if (e != cudaSuccess) return e;
-  }
 #define LBM_CSB(D_, M_, S_) \
-  collide_stream_batch_kernel<D_, M_, S_><<<g, block, smem, s>>>(tab, reinterpret_cast<const int2*>(b->batch_cs_start), parity)
+  collide_stream_batch_kernel<D_, M_, S_><<<g, block, 0, s>>>(tab, reinterpret_cast<const int2*>(b->batch_cs_start), parity)
   if (h0->d == 2) {
     if (mrt) { if (split == 3) LBM_CSB(2, true, 3); else if (split) LBM_CSB(2, true, 1); else LBM_CSB(2, true, 0); }
     else { if (split == 3) LBM_CSB(2, false, 3); else if (split) LBM_CSB(2, false, 1); else LBM_CSB(2, false, 0); }
