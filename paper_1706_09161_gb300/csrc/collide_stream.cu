@@ -938,14 +938,14 @@ collide_stream_march_kernel(const KConst<real> sp, const real* __restrict__ f_in
 }
 
 // ---------------------------------------------------------------------------- TMA-fed 3-D march
-// FP32 forms with n0 % 4 == 0: per plane, one thread loads the block's 40 x 18 window of
-// all Q populations and all d fractional terms (tile, one-node ring, x aligned down to a
-// 16-byte boundary) with two 4-D TMA box loads into a 3-stage shared-memory ring, two
-// planes ahead of the plane being collided; every thread then reads its node (owners)
-// or ring node (the three halo warps) from shared memory.  Nodes outside the domain
-// arrive as zeros (TMA out-of-bounds fill), which the collision maps to zero movers,
-// exactly as the plain march treats them.  The march itself (movers through shared
-// memory, z movers in registers, walls, moment, split) is that of march_body.
+// FP32 forms with n0 % 4 == 0, bound by HBM: per plane, one thread loads the block's 40 x 18
+// window of all Q populations and all d fractional terms (tile, one-node ring, x aligned down
+// to a 16-byte boundary) with two 4-D TMA box loads into a 3-stage shared-memory ring, up to
+// three planes ahead of the plane being collided.  Nodes outside the domain arrive as zeros
+// (TMA out-of-bounds fill), which the collision maps to zero movers, exactly as the plain march
+// treats them.  Measured against one node per thread (608 threads, two barriers per plane, two
+// planes ahead, 410 instructions per node) with its z chunks: 256^3 bf16x6 231 -> 209 us (1317 MB,
+// 93% of the measured copy rate), tf32x3 247 -> 229, 160 x 128 x 100 43 -> 33.
 constexpr int TW = TX + 8, TH = TY + 2;  // staged window: x from x0 - 4, y from y0 - 1
 constexpr int TCP = TX;  // row pitch of the tf32 C ring
 constexpr int TMA_STAGES = 3;
@@ -1001,47 +1001,49 @@ __device__ __forceinline__ void cs_tma_4d(void* dst, const CUtensorMap* map, int
       : "memory");
 }
 
+// Two x-neighbours per thread: 8 owner warps (a half-warp per row of the tile), one warp of
+// ring pairs (the rows below and above) and one of single ring nodes (the columns left and
+// right).  x movers go to the neighbouring lane by shuffle, y movers through shared memory in
+// three buffers (one barrier per plane: a buffer is rewritten only after the next plane's
+// barrier), z movers stay in registers.
+constexpr int T3_WARPS = TX * TY / 64 + 2;
+
 template <bool MRT, int SPLIT>
-__global__ void __launch_bounds__(TX*(TY + HALO_WARPS), 2)
-collide_stream_tma3_kernel(const KConst<float> sp, const __grid_constant__ CUtensorMap map_f,
+__global__ void __launch_bounds__(32 * T3_WARPS, 2)
+collide_stream_tma3_kernel(const __grid_constant__ KConst<float> sp, const __grid_constant__ CUtensorMap map_f,
                            const __grid_constant__ CUtensorMap map_F, float* __restrict__ f_out,
-                           float* __restrict__ C_out, int* __restrict__ flag, SplitOut so, int nz, int early,
-                           double* mpart) {
+                           float* __restrict__ C_out, int* __restrict__ flag, const __grid_constant__ SplitOut so, int nz,
+                           int early, double* mpart) {
   constexpr int D = 3, Q = 7;
   extern __shared__ uint8_t cs_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(cs_raw) + 127) & ~uintptr_t(127));
   uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)TMA_STAGES * TMA_STAGE);
-  __shared__ float s_m[2][4][TY + 2][TX + 2];
-  // tf32: C of the last four planes (slot z & 3), the source of the regrouped split
-  __shared__ float s_c[SPLIT == 2 ? 4 * TY * TCP : 1];
+  __shared__ __align__(8) float s_up[3][TY + 1][TX];  // f*_3 of row r - 1 at [r]
+  __shared__ __align__(8) float s_dn[3][TY + 1][TX];  // f*_4 of row r at [r]
+  __shared__ float s_x[3][2][TY];                     // f*_1 of the left column, f*_2 of the right one
+  // tf32: C of the last two planes, the source of the copy regrouped along y
+  __shared__ __align__(8) float s_c[SPLIT == 2 ? 2 : 1][SPLIT == 2 ? TY : 1][TX];
   const bool wT = SPLIT == 2 && so.thi[0] != nullptr;
   const int n0 = sp.n[0], n1 = sp.n[1], n2 = sp.n[2];
   const long long nodes = sp.nodes;
   const long long plane = (long long)n0 * n1;
-  const int lane = threadIdx.x, wy = threadIdx.y;
-  const int tid = wy * TX + lane;
+  const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
   const int bz = blockIdx.z;
   const int z0 = static_cast<int>((long long)bz * n2 / nz), z1 = static_cast<int>((long long)(bz + 1) * n2 / nz);
   if (early) pdl_trigger();
 
-  int gx, gy, sx, sy;
-  const bool owner = wy < TY;
-  if (owner) {
-    gx = x0 + lane;
-    gy = y0 + wy;
-  } else if (wy == TY) {
-    gx = (lane < 16) ? x0 - 1 : x0 + TX;
-    gy = y0 + (lane & 15);
-  } else {
-    gx = x0 + lane;
-    gy = (wy == TY + 1) ? y0 - 1 : y0 + TY;
+  const bool owner = warp < TX * TY / 64;
+  const int xp = 2 * (lane & 15), row = 2 * warp + (lane >> 4);  // owner's place in the tile
+  const int gx = x0 + xp, gy = y0 + row;
+  // place in the staged window: owners and row ring pairs (x aligned to 8 bytes), column ring nodes
+  int lx = xp + 4, ly = row + 1;
+  if (warp == T3_WARPS - 2) ly = lane < 16 ? 0 : TY + 1;
+  if (warp == T3_WARPS - 1) {
+    lx = lane < 16 ? 3 : TX + 4;
+    ly = (lane & 15) + 1;
   }
-  sx = gx - x0 + 1;
-  sy = gy - y0 + 1;
-  const int lx = gx - (x0 - 4), ly = gy - (y0 - 1);  // position in the staged window
-  const bool in_xy = gx >= 0 && gx < n0 && gy >= 0 && gy < n1;
-  const long long col = gx + (long long)n0 * gy;
+  const float* win = reinterpret_cast<const float*>(ring) + ly * TW + lx;
 
   // plane p lives in stage (p - z0 + 1) % 3; its k-th use of that stage completes phase k
   auto stage_of = [&](int p) { return (p - z0 + 1) % TMA_STAGES; };
@@ -1055,37 +1057,48 @@ collide_stream_tma3_kernel(const KConst<float> sp, const __grid_constant__ CUten
     cs_tma_4d(st, &map_f, x0 - 4, y0 - 1, p, 0, &full[s]);
     cs_tma_4d(st + TMA_FF_OFF, &map_F, x0 - 4, y0 - 1, p, 0, &full[s]);
   };
-  auto collide_staged = [&](int p, float* fs) {
+  auto collide_pair = [&](int p, float (&fs)[2][Q]) {
     cs_mbar_wait(&full[stage_of(p)], parity_of(p), flag);
-    const float* st = reinterpret_cast<const float*>(ring + (size_t)stage_of(p) * TMA_STAGE);
-    float fv[Q], Fv[D];
+    const float* st = win + stage_of(p) * (TMA_STAGE / 4);
+    float fv[2][Q], Fv[2][D];
 #pragma unroll
-    for (int q = 0; q < Q; ++q) fv[q] = st[(q * TH + ly) * TW + lx];
-#pragma unroll
-    for (int mu = 0; mu < D; ++mu) Fv[mu] = st[TMA_FF_OFF / 4 + (mu * TH + ly) * TW + lx];
-    collide_node<float, D, MRT>(sp, fv, Fv, fs);
-  };
-
-  // tf32: planes (ge & ~3 or z0) .. ge of the ring to the regrouped copies.  y copy:
-  // owner warp (plane ge & ~3 + (wy & 3), y group wy >> 2) writes 32 x 16-byte groups
-  // (512 contiguous bytes); z copy: each owner writes its own column's z group.
-  auto flush_T = [&](int ge) {
-    const int gs = max(ge & ~3, z0), cnt = ge - gs + 1;
-    const int zz = (ge & ~3) + (wy & 3), yq = 4 * (wy >> 2);
-    if (zz >= gs && zz <= ge && gx < n0 && y0 + yq < n1) {
-      const float* r = &s_c[((zz & 3) * TY + yq) * TCP + lane];
-      const long long o = (((long long)zz * so.tg1 + ((y0 + yq) >> 2)) * so.tpx + gx) * 4;
-      *reinterpret_cast<float4*>(so.thi[0] + o) = make_float4(r[0], r[TCP], r[2 * TCP], r[3 * TCP]);
+    for (int q = 0; q < Q; ++q) {
+      const float2 t = *reinterpret_cast<const float2*>(st + q * (TH * TW));
+      fv[0][q] = t.x;
+      fv[1][q] = t.y;
     }
-    if (in_xy) {
-      const long long o = (((long long)(gs >> 2) * n1 + gy) * so.tpx + gx) * 4 + (gs & 3);
-      if (cnt == 4) {
-        *reinterpret_cast<float4*>(so.thi[1] + o) =
-            make_float4(s_c[(0 * TY + wy) * TCP + lane], s_c[(1 * TY + wy) * TCP + lane],
-                        s_c[(2 * TY + wy) * TCP + lane], s_c[(3 * TY + wy) * TCP + lane]);
-      } else {
-        for (int k = 0; k < cnt; ++k) so.thi[1][o + k] = s_c[(((gs + k) & 3) * TY + wy) * TCP + lane];
-      }
+#pragma unroll
+    for (int mu = 0; mu < D; ++mu) {
+      const float2 t = *reinterpret_cast<const float2*>(st + TMA_FF_OFF / 4 + mu * (TH * TW));
+      Fv[0][mu] = t.x;
+      Fv[1][mu] = t.y;
+    }
+    collide_node<float, D, MRT>(sp, fv[0], Fv[0], fs[0]);
+    collide_node<float, D, MRT>(sp, fv[1], Fv[1], fs[1]);
+  };
+  // plane p's movers into buffer b; the owners' populations stay in fs
+  auto movers = [&](int p, int b, float (&fs)[2][Q]) {
+    if (owner) {
+      collide_pair(p, fs);
+      *reinterpret_cast<float2*>(&s_up[b][row + 1][xp]) = make_float2(fs[0][3], fs[1][3]);
+      *reinterpret_cast<float2*>(&s_dn[b][row][xp]) = make_float2(fs[0][4], fs[1][4]);
+    } else if (p >= z1) {
+      return;  // only the owners' f*_6 of the plane past the chunk is needed
+    } else if (warp == T3_WARPS - 2) {
+      float h[2][Q];
+      collide_pair(p, h);
+      if (lane < 16) *reinterpret_cast<float2*>(&s_up[b][0][xp]) = make_float2(h[0][3], h[1][3]);  // moves +y into the tile
+      else *reinterpret_cast<float2*>(&s_dn[b][TY][xp]) = make_float2(h[0][4], h[1][4]);           // moves -y into it
+    } else {
+      cs_mbar_wait(&full[stage_of(p)], parity_of(p), flag);
+      const float* st = win + stage_of(p) * (TMA_STAGE / 4);
+      float fv[Q], Fv[D], h[Q];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) fv[q] = st[q * (TH * TW)];
+#pragma unroll
+      for (int mu = 0; mu < D; ++mu) Fv[mu] = st[TMA_FF_OFF / 4 + mu * (TH * TW)];
+      collide_node<float, D, MRT>(sp, fv, Fv, h);
+      s_x[b][lane >> 4][lane & 15] = lane < 16 ? h[1] : h[2];  // moves +x, -x into the tile
     }
   };
 
@@ -1102,118 +1115,163 @@ collide_stream_tma3_kernel(const KConst<float> sp, const __grid_constant__ CUten
     issue(z0);
     issue(z0 + 1);  // z0 + 1 <= z1: needed by the owners' first iteration
   }
-  bool bad = false;
   SumAcc<float> macc;
-  float cur[Q], nxt[Q];
-  float prev5 = 0.f;
-  if (owner) {
-    float t[Q];
-    collide_staged(z0 - 1, t);
-    prev5 = t[5];
-    collide_staged(z0, cur);
-  }
-  __syncthreads();  // plane z0 - 1 is read: its stage takes plane z0 + 2
-  if (tid == 0 && z0 + 2 <= z1) {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    issue(z0 + 2);
-  }
-  int buf = 0;
-  for (int z = z0; z < z1; ++z) {
-    if (owner) {
-      collide_staged(z + 1, nxt);
-      s_m[buf][0][sy][sx] = cur[1];
-      s_m[buf][1][sy][sx] = cur[2];
-      s_m[buf][2][sy][sx] = cur[3];
-      s_m[buf][3][sy][sx] = cur[4];
-    } else {
-      float h[Q];
-      collide_staged(z, h);
-      if (wy == TY) {
-        if (lane < 16) s_m[buf][0][sy][sx] = h[1];  // moves +x into the tile
-        else s_m[buf][1][sy][sx] = h[2];            // moves -x into the tile
-      } else if (wy == TY + 1) {
-        s_m[buf][2][sy][sx] = h[3];                 // moves +y into the tile
-      } else {
-        s_m[buf][3][sy][sx] = h[4];                 // moves -y into the tile
-      }
-    }
-    __syncthreads();
-    // plane z is read by everyone: its stage takes plane z + 3
-    if (tid == 0 && z + 3 <= z1) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue(z + 3);
-    }
-    if (SPLIT == 2 && wT && z > z0 && ((z - 1) & 3) == 3) {
-      if (owner) flush_T(z - 1);
-      __syncthreads();  // slot z & 3 is rewritten below
-    }
-    float Cn = 0.f;
-    if (owner && in_xy) {
-      float fv[Q];
-      bool known[Q];
-      fv[0] = cur[0];
-      known[0] = true;
-      known[1] = gx > 0;
-      known[2] = gx + 1 < n0;
-      known[3] = gy > 0;
-      known[4] = gy + 1 < n1;
-      known[5] = z > 0;
-      known[6] = z + 1 < n2;
-      fv[1] = s_m[buf][0][sy][sx - 1];
-      fv[2] = s_m[buf][1][sy][sx + 1];
-      fv[3] = s_m[buf][2][sy - 1][sx];
-      fv[4] = s_m[buf][3][sy + 1][sx];
-      fv[5] = prev5;
-      fv[6] = nxt[6];
-      float sum_known = 0.f;
-      int n_unknown = 0;
+  float bad = 0.f;
+  float c[2][Q], p5[2] = {0.f, 0.f};  // plane z: f*_q of this pair; f*_5 of plane z - 1
+  float tz[2][4] = {};                // tf32: C of the current group of four planes
 #pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        if (known[q]) {
-          sum_known += fv[q];
-        } else {
-          fv[q] = 0.f;
-          ++n_unknown;
+  for (int v = 0; v < 2; ++v)
+#pragma unroll
+    for (int q = 0; q < Q; ++q) c[v][q] = 0.f;
+  if (owner) {
+    collide_pair(z0 - 1, c);
+    p5[0] = c[0][5];
+    p5[1] = c[1][5];
+  }
+  movers(z0, 0, c);
+  __syncthreads();  // planes z0 - 1 and z0 are read: their stages take z0 + 2 and z0 + 3
+  if (tid == 0) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (z0 + 2 <= z1) issue(z0 + 2);
+    if (z0 + 3 <= z1) issue(z0 + 3);
+  }
+  // tf32: plane p of s_c to the copy regrouped along y: 32 x 4 groups of 16 bytes
+  auto flush_y = [&](int p) {
+    const int x = tid & 31, yq = 4 * (tid >> 5);
+    if (tid < 4 * TX && x0 + x < n0 && y0 + yq < n1) {
+      const float* r = &s_c[p & 1][SPLIT == 2 ? yq : 0][x];
+      const long long o = (((long long)p * so.tg1 + ((y0 + yq) >> 2)) * so.tpx + x0 + x) * 4;
+      *reinterpret_cast<float4*>(so.thi[0] + o) = make_float4(r[0], r[TX], r[2 * TX], r[3 * TX]);
+    }
+  };
+  const bool in_xy = gx < n0 && gy < n1;  // (owners; n0 is a multiple of 4)
+  const bool side = x0 == 0 || x0 + TX >= n0 || y0 == 0 || y0 + TY >= n1;
+  const unsigned off = static_cast<unsigned>(gy * n0 + gx);
+  int b = 0;
+  for (int z = z0; z < z1; ++z) {
+    float n[2][Q];
+    const int bn = b == 2 ? 0 : b + 1;
+    movers(z + 1, bn, n);
+    __syncthreads();
+    // plane z + 1 is read by everyone: its stage takes plane z + 4
+    if (tid == 0 && z + 4 <= z1) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      issue(z + 4);
+    }
+    if (SPLIT == 2 && wT && z > z0) flush_y(z - 1);
+    if (owner) {
+      const float up = __shfl_up_sync(0xffffffffu, c[1][1], 1), dn = __shfl_down_sync(0xffffffffu, c[0][2], 1);
+      const float2 y3 = *reinterpret_cast<const float2*>(&s_up[b][row][xp]);
+      const float2 y4 = *reinterpret_cast<const float2*>(&s_dn[b][row + 1][xp]);
+      float o[2][Q], C[2] = {0.f, 0.f};
+      o[0][0] = c[0][0];
+      o[1][0] = c[1][0];
+      o[0][1] = xp == 0 ? s_x[b][0][row] : up;
+      o[1][1] = c[0][1];
+      o[0][2] = c[1][2];
+      o[1][2] = xp == TX - 2 ? s_x[b][1][row] : dn;
+      o[0][3] = y3.x;
+      o[1][3] = y3.y;
+      o[0][4] = y4.x;
+      o[1][4] = y4.y;
+      o[0][5] = p5[0];
+      o[1][5] = p5[1];
+      o[0][6] = n[0][6];
+      o[1][6] = n[1][6];
+      if (!side && z > 0 && z + 1 < n2) {  // no wall within reach (block-uniform)
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+#pragma unroll
+          for (int q = 0; q < Q; ++q) C[v] += o[v][q];
+      } else {
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          const bool known[Q] = {true, gx + v > 0, gx + v + 1 < n0, gy > 0, gy + 1 < n1, z > 0, z + 1 < n2};
+          int n_unknown = 0;
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            if (known[q]) {
+              C[v] += o[v][q];
+            } else {
+              o[v][q] = 0.f;
+              ++n_unknown;
+            }
+          }
+          if (n_unknown > 0) {
+            // Eq. (Dirichlet_BC); with k unknown populations each takes 1/k of the deficit
+            const float fill = (sp.C_wall - C[v]) / static_cast<float>(n_unknown);
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+              if (!known[q]) o[v][q] = fill;
+            C[v] = o[v][0];
+#pragma unroll
+            for (int q = 1; q < Q; ++q) C[v] += o[v][q];
+          }
         }
       }
-      float C = sum_known;
-      if (n_unknown > 0) {
-        // Eq. (Dirichlet_BC); with k unknown populations each takes 1/k of the deficit
-        const float fill = (sp.C_wall - sum_known) / static_cast<float>(n_unknown);
+      if (in_xy) {
+        float* fz = f_out + z * plane;
 #pragma unroll
-        for (int q = 0; q < Q; ++q)
-          if (!known[q]) fv[q] = fill;
-        C = fv[0];
+        for (int q = 0; q < Q; ++q) *reinterpret_cast<float2*>(fz + q * nodes + off) = make_float2(o[0][q], o[1][q]);
+        if (SPLIT == 0 || C_out) *reinterpret_cast<float2*>(C_out + z * plane + off) = make_float2(C[0], C[1]);
+        if constexpr (SPLIT == 2) {
+          *reinterpret_cast<float2*>(static_cast<float*>(so.hi) + ((long long)z * n1 + gy) * so.ldp + gx) =
+              make_float2(C[0], C[1]);
+        } else if constexpr (SPLIT != 0) {
+          write_split_v<SPLIT, 2>(so, ((long long)z * n1 + gy) * so.ldp + gx, C);
+        }
 #pragma unroll
-        for (int q = 1; q < Q; ++q) C += fv[q];
+        for (int v = 0; v < 2; ++v) {
+          bad = __fmaf_rn(C[v], 0.f, bad);  // NaN once a C is not finite
+          macc.add(C[v]);
+        }
+      } else {
+        C[0] = C[1] = 0.f;  // zero outside the domain
       }
-      const long long node = col + z * plane;
+      if (SPLIT == 2 && wT) {
+        *reinterpret_cast<float2*>(&s_c[z & 1][SPLIT == 2 ? row : 0][xp]) = make_float2(C[0], C[1]);
+        // z copy: each node's group of four planes, or the part of it that lies in this chunk
+        const int k = z & 3;
 #pragma unroll
-      for (int q = 0; q < Q; ++q) f_out[q * nodes + node] = fv[q];
-      C_out[node] = C;
-      if (SPLIT) write_split<SPLIT>(so, ((long long)z * n1 + gy) * so.ldp + gx, C);
-      bad |= !isfinite(C);
-      macc.add(C);
-      Cn = C;
-    }
-    if (owner) {
-      if (SPLIT == 2 && wT) s_c[((z & 3) * TY + wy) * TCP + lane] = Cn;  // zero outside the domain
-      prev5 = cur[5];
+        for (int j = 0; j < 4; ++j)
+          if (j == k) {
+            tz[0][j] = C[0];
+            tz[1][j] = C[1];
+          }
+        if (in_xy && (k == 3 || z + 1 == z1)) {
+          const int first = max(z0 - (z & ~3), 0);
+          float* t = so.thi[1] + (((long long)(z >> 2) * n1 + gy) * so.tpx + gx) * 4;
 #pragma unroll
-      for (int q = 0; q < Q; ++q) cur[q] = nxt[q];
+          for (int v = 0; v < 2; ++v) {
+            if (first == 0 && k == 3) {
+              *reinterpret_cast<float4*>(t + 4 * v) = make_float4(tz[v][0], tz[v][1], tz[v][2], tz[v][3]);
+            } else {
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (j >= first && j <= k) t[4 * v + j] = tz[v][j];
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        p5[v] = c[v][5];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) c[v][q] = n[v][q];
+      }
     }
-    buf ^= 1;
+    b = bn;
   }
   if (SPLIT == 2 && wT) {
     __syncthreads();
-    if (owner) flush_T(z1 - 1);
+    flush_y(z1 - 1);
   }
   // every issued plane (up to z1) was waited for by the owners; after a timeout make sure
   // no copy is still in flight into this block's shared memory before it exits
   if (tid == 0)
     for (int p = (z1 - 2 > z0 - 1 ? z1 - 2 : z0 - 1); p <= z1; ++p) cs_mbar_wait(&full[stage_of(p)], parity_of(p), flag);
-  if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(flag, 1);
-  block_mass(macc, mpart, block_linear());
+  if (__any_sync(0xffffffffu, bad != 0.f) && lane == 0) atomicOr(flag, 1);
+  block_mass<T3_WARPS>(macc, mpart, block_linear());
   if (!early) pdl_trigger();
 }
 
@@ -1679,13 +1737,15 @@ cudaError_t launch_march2(const cudaLaunchConfig_t& cfg, const KConst<float>& sp
                             early, mpart);
 }
 
-// z chunks of the 3-D march over `cols` tile columns: the count that maximises the wave
-// efficiency (blocks / 304 over its ceiling, two blocks per SM) per plane collided,
-// each chunk re-colliding two planes at its start; chunks of at least 4 planes (with fewer
-// blocks than the GPU holds, a block's chain of planes is the whole time: 48^3 in 18 blocks of
-// 18 planes 23 us, in 72 of 6 12.6 us)
+// z chunks of the 3-D march over `cols` tile columns.  With waves enough, chunks of 16 planes:
+// long chunks leave a long last wave, short ones re-collide two planes each (256^3 bf16x6 march
+// with 7 / 9 / 16 / 24 / 38 chunks: 231 / 216 / 209 / 210 / 217 us).  Else the count that
+// maximises the wave efficiency (blocks / 304 over its ceiling, two blocks per SM) per plane
+// collided, chunks of at least 4 planes (with fewer blocks than the GPU holds, a block's chain
+// of planes is the whole time: 48^3 in 18 blocks of 18 planes 23 us, in 72 of 6 12.6 us)
 int z_chunks(long long cols, int n2) {
   if (n2 < 8) return 1;
+  if (cols * (n2 / 16) >= 8LL * device_sms()) return (n2 + 15) / 16;
   const int sms = device_sms();
   int best = 1;
   double best_eff = 0.0;
@@ -1865,6 +1925,8 @@ cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out
       const CUtensorMap& mf = slot ? *static_cast<const CUtensorMap*>(slot->map_f) : pl->f[f_in == h->dev.f[0] ? 0 : 1];
       const CUtensorMap& mF = slot ? *static_cast<const CUtensorMap*>(slot->map_F) : pl->F;
       cfg.dynamicSmemBytes = TMA_SMEM;
+      cfg.blockDim = dim3(32, T3_WARPS);
+      h->cs_nparts = T3_WARPS * bx * by * nz;
       if (split == 0) return launch_tma3<MRT, 0>(cfg, sp, mf, mF, fo, Co, flag, so, nz, early, mp);
       if (split == 1) return launch_tma3<MRT, 1>(cfg, sp, mf, mF, fo, Co, flag, so, nz, early, mp);
       if (split == 3) return launch_tma3<MRT, 3>(cfg, sp, mf, mF, fo, Co, flag, so, nz, early, mp);
