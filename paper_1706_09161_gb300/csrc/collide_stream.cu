@@ -512,7 +512,7 @@ __device__ __forceinline__ void march_body(const KConst<real>& sp, const real* _
       const long long node = col + z * plane;
 #pragma unroll
       for (int q = 0; q < Q; ++q) f_out[q * nodes + node] = fv[q];
-      C_out[node] = C;
+      if (SPLIT == 0 || C_out) C_out[node] = C;
       if (SPLIT && FLD && fp.gsplit) {
 #pragma unroll
         for (int mu = 0; mu < D; ++mu) {
@@ -677,7 +677,7 @@ __device__ __forceinline__ void march2_pipe(const KConst<float>& sp, const float
       const long long node = gx + (long long)n0 * gy;
 #pragma unroll
       for (int q = 0; q < Q; ++q) f_out[q * nodes + node] = fv[q];
-      C_out[node] = C;
+      if (SPLIT == 0 || C_out) C_out[node] = C;
       if (SPLIT) write_split<SPLIT>(so, (long long)gy * so.ldp + gx, C);
       bad |= !isfinite(C);
       macc.add(C);
@@ -863,7 +863,7 @@ __device__ __forceinline__ void strip_march(const KConst<float>& sp, const float
         const long long node = (long long)yo * n0 + gx;
 #pragma unroll
         for (int q = 0; q < 5; ++q) store_v<V>(f_out + q * nodes + node, o[q]);
-        store_v<V>(C_out + node, C);
+        if (SPLIT == 0 || C_out) store_v<V>(C_out + node, C);
         if constexpr (SPLIT != 0) write_split_v<SPLIT, V>(so, (long long)yo * so.ldp + gx, C);
 #pragma unroll
         for (int v = 0; v < V; ++v) {
@@ -1459,7 +1459,7 @@ __device__ __forceinline__ void march2_tma(const KConst<float>& sp, const CUtens
       const long long node = gx + (long long)n0 * gy;
 #pragma unroll
       for (int q = 0; q < Q; ++q) f_out[q * nodes + node] = fv[q];
-      C_out[node] = C;
+      if (SPLIT == 0 || C_out) C_out[node] = C;
       if (SPLIT) write_split<SPLIT>(so, (long long)gy * so.ldp + gx, C);
       if (SPLIT == 2 && wT) s_c[((tr & 1) * TY + dy) * TCP + dx] = C;
       bad |= !isfinite(C);
@@ -1627,7 +1627,7 @@ __host__ __device__ constexpr int batch_threads(int d) { return d == 2 ? 32 * kS
 
 template <int D, bool MRT, int SPLIT>
 __global__ void __launch_bounds__(batch_threads(D), D == 2 ? 4 : 2)
-collide_stream_batch_kernel(const BatchCS* __restrict__ tab, const int2* __restrict__ block_map, int parity) {
+collide_stream_batch_kernel(const BatchCS* __restrict__ tab, const int2* __restrict__ block_map, int parity, int keep_C) {
   __shared__ KConst<float> s_k;
   const int2 pb = __ldg(&block_map[blockIdx.x]);
   const BatchCS& e = tab[pb.x];
@@ -1641,15 +1641,16 @@ collide_stream_batch_kernel(const BatchCS* __restrict__ tab, const int2* __restr
   }
   __syncthreads();
   float* fo = const_cast<float*>(e.f[parity ^ 1]);
+  float* Co = keep_C ? e.C : nullptr;
   if constexpr (D == 2) {
     const int item = pb.y * kStripWarps + (tid >> 5);
     if (item < e.items) {
       const int x = item % e.strips * 32 * e.v, y0 = item / e.strips * e.rows, y1 = min(y0 + e.rows, s_k.n[1]);
-      if (e.v == 2) strip_march<2, MRT, SPLIT, true>(s_k, e.f[parity], e.F, fo, e.C, e.flag, e.so, x, y0, y1, e.mpart, item);
-      else strip_march<1, MRT, SPLIT, true>(s_k, e.f[parity], e.F, fo, e.C, e.flag, e.so, x, y0, y1, e.mpart, item);
+      if (e.v == 2) strip_march<2, MRT, SPLIT, true>(s_k, e.f[parity], e.F, fo, Co, e.flag, e.so, x, y0, y1, e.mpart, item);
+      else strip_march<1, MRT, SPLIT, true>(s_k, e.f[parity], e.F, fo, Co, e.flag, e.so, x, y0, y1, e.mpart, item);
     }
   } else {
-    march_body<float, D, MRT, SPLIT>(s_k, e.f[parity], e.F, fo, e.C, e.flag, e.so, pb.y % e.bx, pb.y / e.bx, 0,
+    march_body<float, D, MRT, SPLIT>(s_k, e.f[parity], e.F, fo, Co, e.flag, e.so, pb.y % e.bx, pb.y / e.bx, 0,
                                      e.k.n[2], e.mpart, pb.y);
   }
 }
@@ -2141,7 +2142,7 @@ int cs_batch_prepare(lbm_s* b) {
   return LBM_OK;
 }
 
-cudaError_t launch_collide_stream_batch(const lbm_s* b, int parity, cudaStream_t s) {
+cudaError_t launch_collide_stream_batch(const lbm_s* b, int parity, cudaStream_t s, bool keep_C) {
   const lbm_s* h0 = b->subs[0];
   const bool mrt = h0->prm.collision == LBM_MRT;
   const int split = cs_split_code(h0);  // 0, 1 or 3 (batches have no tf32 form)
@@ -2150,7 +2151,7 @@ cudaError_t launch_collide_stream_batch(const lbm_s* b, int parity, cudaStream_t
   const dim3 block(TX, batch_threads(h0->d) / TX);
   const int g = b->batch_cs_blocks;
 #define LBM_CSB(D_, M_, S_) \
-  collide_stream_batch_kernel<D_, M_, S_><<<g, block, 0, s>>>(tab, reinterpret_cast<const int2*>(b->batch_cs_start), parity)
+  collide_stream_batch_kernel<D_, M_, S_><<<g, block, 0, s>>>(tab, reinterpret_cast<const int2*>(b->batch_cs_start), parity, keep_C || split == 0)
   if (h0->d == 2) {
     if (mrt) { if (split == 3) LBM_CSB(2, true, 3); else if (split) LBM_CSB(2, true, 1); else LBM_CSB(2, true, 0); }
     else { if (split == 3) LBM_CSB(2, false, 3); else if (split) LBM_CSB(2, false, 1); else LBM_CSB(2, false, 0); }

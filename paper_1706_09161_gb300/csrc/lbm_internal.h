@@ -179,6 +179,7 @@ struct CsSlot {
   const void* map_f;
   const void* map_F;
 };
+// C_out may be null where the next operator reads the split operands only (C_is_spare)
 cudaError_t launch_collide_stream(const lbm_s* h, const void* f_in, void* f_out, void* C_out,
                                   cudaStream_t s, int tk = 0, const CsSlot* slot = nullptr);
 bool cs_encode_slot(const lbm_s* h, const void* f, const void* F, void* map_f, void* map_F);
@@ -244,7 +245,7 @@ cudaError_t launch_fused(lbm_s* h, int nsteps, cudaStream_t s);
 bool tc_tma_store(const lbm_s* h);  // the operator stores F tiles with TMA
 bool tc_one_wave(const lbm_s* h);  // the tensor-core operator grid fits in one wave
 void tc_set_pdl(lbm_s* h, bool on);
-cudaError_t launch_collide_stream_batch(const lbm_s* b, int parity, cudaStream_t s);
+cudaError_t launch_collide_stream_batch(const lbm_s* b, int parity, cudaStream_t s, bool keep_C = true);
 void tc_release(lbm_s* h);
 int tc_set_weights(lbm_s* h, const std::vector<std::vector<double>>& K);  // re-split K_mu (plan kept)
 int tc_set_gfield(lbm_s* h, bool on);  // bf16 forms: operands g_mu(x) C per axis (or C)
