@@ -1,0 +1,119 @@
+"""Collide-stream kernels and the per-tile operator at the edges of their tiles, and the stores
+that a call of several steps leaves out, against the FP64 oracle.
+
+Concentrations: 6x the error that the form's own arithmetic makes when re-run on the CPU
+(``arith_bounds.bounds``, never below 1e-5), in relative L2 and node by node.  The mass is the
+sum of the C that the kernel stores: rel 1e-6 of sum |C|, FP32 rounding of each term counted.
+Operator: the split's rounding plus 2 sqrt(N) roundings of 2^-23 of FP32 accumulation, as a
+relative L2 (all terms are non-negative).  Where only the schedule differs, results are equal bit
+for bit.
+"""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import arith_bounds
+from oracle import lbm_oracle as O
+from paper_1706_09161_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA GPU required for -m gpu tests")
+    from paper_1706_09161_gb300 import lbm
+    return lbm
+
+
+def _case(grid, seed, collision="mrt"):
+    rng = np.random.default_rng(seed)
+    pb = W.random_problem(rng, len(grid), collision, grid, spherical=collision == "bgk")
+    pb = dataclasses.replace(pb, alpha=tuple(1.5 + 0.5 * (a - 1.2) / 0.8 for a in pb.alpha))
+    return pb, W.random_field(rng, grid)
+
+
+# strips of 64 (even rows) or 32 nodes (odd rows): below, at and above one strip; rows below, at
+# and above a ring block (16) and a chunk (8), the last chunk of one row
+@pytest.mark.parametrize("precision", ["fp32", "bf16split", "bf16x6split"])
+@pytest.mark.parametrize("collision", ["bgk", "mrt"])
+def test_batch_strips(L, precision, collision):
+    sizes = [(3, 3), (31, 9), (33, 16), (63, 17), (64, 8), (65, 33), (66, 25), (128, 7), (130, 70), (191, 41)]
+    cases = [_case(g, 211 + sum(g), collision) for g in sizes]
+    n = 6
+    with L.Batch([p for p, _ in cases], [c for _, c in cases], precision) as b:
+        b.step(n)
+        for i, (pb, C0) in enumerate(cases):
+            C = b.C(i)
+            arith_bounds.check_form(C, pb, C0, n, precision, f"{sizes[i]}")
+            assert abs(b.mass(i) - C.sum()) <= 1e-6 * np.abs(C).sum(), sizes[i]
+
+
+# tiles of 32 x 16 nodes with and without remainders, one to several z chunks, the shortest box
+@pytest.mark.parametrize("precision", ["fp32", "bf16split", "bf16x6split", "tf32split"])
+@pytest.mark.parametrize("grid", [(4, 3, 3), (32, 16, 17), (36, 17, 33), (64, 15, 16), (28, 33, 50)])
+def test_3d_march_chunks(L, precision, grid):
+    pb, C0 = _case(grid, 307 + sum(grid))
+    n = 5
+    f = []
+    for chunk in (0, 1, 2, grid[2]):
+        with L.Lattice(pb, C0, precision) as lat:
+            lat.configure(0 if precision == "fp32" else 128, 1, 0, chunk, 0)
+            lat.reset()
+            lat.step(n)
+            f.append(lat.f())
+            C, mass = lat.C(), lat.mass()
+        assert np.array_equal(f[0], f[-1]), chunk
+        assert abs(mass - C.sum()) <= 1e-6 * np.abs(C).sum(), chunk
+    arith_bounds.check_form(C, pb, C0, n, precision, f"{grid}")
+
+
+# rows that TMA cannot store, where the CTAs of a tile add their partial tiles themselves, and
+# grids small enough for 64-column tiles; sides below, at and above a tile
+@pytest.mark.parametrize("kind", ["bf16split", "bf16x5split", "bf16x6split", "tf32split"])
+@pytest.mark.parametrize("grid", [(301, 203), (129, 257), (63, 300), (256, 255), (67, 65, 30), (48, 48, 48)])
+def test_operator_built_in_plan(L, kind, grid):
+    split = {"bf16split": 4e-5, "bf16x5split": 2e-5, "bf16x6split": 2e-6, "tf32split": 2e-6}[kind]
+    pb, C0 = _case(grid, 401 + sum(grid))
+    with L.Lattice(pb, C0, kind) as lat:
+        F = O.fractional_terms(O.Operators(pb), torch.tensor(lat.C()))
+        for mu, N in enumerate(grid):
+            tol = max(split, 2.0 * np.sqrt(N) * 2.0 ** -23)
+            assert arith_bounds.rel_l2(lat.F(mu), F[mu].numpy()) < tol, mu
+
+
+# C is stored by the last step of a call only (133 steps: a captured graph and single steps)
+@pytest.mark.parametrize("kind", ["fp32", "bf16split", "bf16x5split", "bf16x6split", "tf32split"])
+@pytest.mark.parametrize("grid,fields", [((68, 50), False), ((67, 50), False), ((36, 20, 18), False),
+                                         ((35, 20, 18), False), ((68, 50), True), ((36, 20, 18), True)])
+def test_one_call_equals_single_steps(L, kind, grid, fields):
+    pb, C0 = _case(grid, 503 + sum(grid))
+    n = 133
+    with L.Lattice(pb, C0, kind) as a, L.Lattice(pb, C0, kind) as b:
+        for lat in (a, b):
+            if fields:
+                x = np.linspace(0.0, 1.0, grid[0]) * np.ones(pb.shape)
+                d = pb.d
+                lat.set_fields(D=np.array(pb.D).reshape((d, d) + (1,) * d) * (1.0 + 0.3 * x),
+                               g=np.stack([1.0 + 0.2 * x] * d), u=np.stack([0.02 * x] * d))
+        a.step(n)
+        for _ in range(n):
+            b.step(1)
+        assert np.array_equal(a.f(), b.f())
+        assert np.array_equal(a.C(), b.C())
+
+
+@pytest.mark.parametrize("kind", ["fp32", "bf16split", "bf16x6split"])
+def test_one_batch_call_equals_single_steps(L, kind):
+    cases = [_case(g, 601 + sum(g)) for g in [(37, 20), (64, 64), (130, 33)]]
+    n = 133
+    args = ([p for p, _ in cases], [c for _, c in cases], kind)
+    with L.Batch(*args) as a, L.Batch(*args) as b:
+        a.step(n)
+        for _ in range(n):
+            b.step(1)
+        for i in range(len(cases)):
+            assert np.array_equal(a.C(i), b.C(i)), i
