@@ -320,8 +320,7 @@ bool pdl_fits(const lbm_s* h) {
   if (h->is_batch()) return false;
   if (!h->tc) return lbm::cs_one_wave(h) && lbm::simt_one_wave(h);  // SIMT operator
   const bool adjacent = lbm::bf16_parts(h->prm.precision) || lbm::cs_writes_T(h);
-  // the field march's grid is not the one cs_one_wave describes: no early launch there
-  return adjacent && !h->fld.on && lbm::cs_one_wave(h) && lbm::tc_one_wave(h);
+  return adjacent && !(h->fld.on && h->d == 3) && lbm::cs_one_wave(h) && lbm::tc_one_wave(h);
 }
 
 int alloc_bytes(const lbm_s* h, void** p, size_t bytes) {
@@ -1235,8 +1234,6 @@ static int rebuild_fields(lbm_s* h) {
     h->fld.on = true;
     h->fused = false;  // the fused step runs the constant-coefficient march only
   }
-  h->pdl = pdl_fits(h);  // the march, and with tf32 whether the operands need a launch of their own
-  if (h->tc) lbm::tc_set_pdl(h, h->pdl);
   h->fld.gvar = h->fld.on && g_field != nullptr;
   {  // g inside the integrals (K without g), or folded into K
     Derived dv;
@@ -1245,6 +1242,15 @@ static int rebuild_fields(lbm_s* h) {
     if ((rc = upload_weights(h, dv.h, h->tc ? &Kall : nullptr))) return rc;
     if (h->tc && ((rc = lbm::tc_set_weights(h, Kall)) || (rc = lbm::tc_set_gfield(h, h->fld.gvar)))) return rc;
   }
+  if (h->tc) {  // where the partial sums of a split contraction are added depends on the march
+    int bn, ks, persist;
+    lbm::tc_config(h, &bn, &ks, &persist);
+    if ((rc = lbm::tc_replan(h, bn, ks, persist))) return rc;
+    lbm::cs_release(h);
+    if ((rc = lbm::cs_prepare(h))) return rc;
+  }
+  h->pdl = pdl_fits(h);  // the march, and with tf32 whether the operands need a launch of their own
+  if (h->tc) lbm::tc_set_pdl(h, h->pdl);
   return lbm_reset(h);
 }
 

@@ -29,6 +29,24 @@ template <int D> struct Lat;
 template <> struct Lat<2> { static constexpr int Q = 5; };
 template <> struct Lat<3> { static constexpr int Q = 7; };
 
+// MRT change of basis, Eq. (MatrixD2): entry (i, q) of M for D2Q5 (D = 2) or D3Q7 (D = 3),
+// and the squared norm of row i (the rows are orthogonal: M^-1 = M^T diag(1 / norm))
+__host__ __device__ constexpr int mom(int D, int i, int q) {
+  if (i == 0) return 1;
+  if (i <= D) return q == 2 * i - 1 ? 1 : (q == 2 * i ? -1 : 0);  // flux moments
+  if (D == 2) return i == 3 ? (q == 0 ? 4 : -1) : (q == 0 ? 0 : (q <= 2 ? 1 : -1));
+  if (i == 4) return q == 0 ? 6 : -1;
+  if (i == 5) return q == 0 ? 0 : (q <= 2 ? 2 : -1);
+  return (q == 0 || q <= 2) ? 0 : (q <= 4 ? 1 : -1);
+}
+__host__ __device__ constexpr int mom_norm(int D, int i) {
+  int n = 0;
+  for (int q = 0; q < 2 * D + 1; ++q) n += mom(D, i, q) * mom(D, i, q);
+  return n;
+}
+static_assert(mom_norm(2, 3) == 20 && mom_norm(3, 4) == 42 && mom_norm(3, 5) == 12 && mom_norm(3, 6) == 4,
+              "moment rows of Eq. (MatrixD2)");
+
 // Per-step constants in the working precision (no FP64 arithmetic per node on the
 // FP32 forms; GB300's FP64 rate is a small fraction of its FP32 rate).
 template <typename real>
@@ -41,7 +59,8 @@ struct KConst {
   real C_wall;
   int ksum;           // F holds ksum partial sums (split-K operator), added in order
   long long pstride;  // elements between partial sums
-  real sfree[3];      // MRT rates of the free moments d+1..Q-1 (spatially varying coefficients)
+  real sfree[3];      // MRT rates of the free moments d+1..Q-1 over the squared norms of their rows of M
+                      // (spatially varying coefficients)
 };
 
 // Coefficients that vary from node to node (lbm_set_fields), working precision, [k][node]:
@@ -82,7 +101,8 @@ KConst<real> make_const(const StepParams& sp) {
   k.C_wall = static_cast<real>(sp.C_wall);
   k.ksum = sp.ksum;
   k.pstride = (sp.n[2] > 1 ? 3 : 2) * sp.nodes;
-  for (int i = 0; i < 3; ++i) k.sfree[i] = static_cast<real>(sp.sfree[i]);
+  const int d = sp.n[2] > 1 ? 3 : 2;
+  for (int i = 0; i < d; ++i) k.sfree[i] = static_cast<real>(sp.sfree[i] / mom_norm(d, d + 1 + i));
   return k;
 }
 
@@ -155,37 +175,63 @@ __device__ __forceinline__ void collide_node(const KConst<real>& sp, const real*
   }
 }
 
-// MRT change of basis, Eq. (MatrixD2): entry (i, q) of M for D2Q5 (D = 2) or D3Q7 (D = 3),
-// and the squared norm of row i (the rows are orthogonal: M^-1 = M^T diag(1 / norm))
-__host__ __device__ constexpr int mom(int D, int i, int q) {
-  if (i == 0) return 1;
-  if (i <= D) return q == 2 * i - 1 ? 1 : (q == 2 * i ? -1 : 0);  // flux moments
-  if (D == 2) return i == 3 ? (q == 0 ? 4 : -1) : (q == 0 ? 0 : (q <= 2 ? 1 : -1));
-  if (i == 4) return q == 0 ? 6 : -1;
-  if (i == 5) return q == 0 ? 0 : (q <= 2 ? 2 : -1);
-  return (q == 0 || q <= 2) ? 0 : (q <= 4 ? 1 : -1);
-}
-__host__ __device__ constexpr int mom_norm(int D, int i) {
-  int n = 0;
-  for (int q = 0; q < 2 * D + 1; ++q) n += mom(D, i, q) * mom(D, i, q);
-  return n;
-}
-static_assert(mom_norm(2, 3) == 20 && mom_norm(3, 4) == 42 && mom_norm(3, 5) == 12 && mom_norm(3, 6) == 4,
-              "moment rows of Eq. (MatrixD2)");
-
-template <typename real, int D>
-__device__ __forceinline__ void collide_moments(const KConst<real>& sp, const FieldPtrs<real>& fp, long long node,
-                                                const real* f, const real* dl, real* fs);
-
-// Equilibrium and collision of one node with coefficients of that node (FieldPtrs):
-// Eq. (Feq) with u(x); BGK f* = f - (f - feq)/lambda(x); MRT in moment space
-// f* = f - M^-1 Lambda(x) M (f - feq), Lambda(x) = diag(1, R(x), s_free) (Eqs. MRT-Coll,
-// MatrixS, D_ab with lambda_{mu nu}(x)).
+// One node's coefficients (FieldPtrs): relaxation rate or rate block R, advective factors, source.
 template <typename real, int D, bool MRT>
-__device__ __forceinline__ void collide_node_field(const KConst<real>& sp, const FieldPtrs<real>& fp, long long node,
-                                                   const real* f, const real* F, real* fs) {
+struct NodeCoef {
+  static constexpr int NR = MRT ? D * (D + 1) / 2 : 1;
+  real coll[NR], adv[D], src;
+};
+
+// MRT collision in moment space with the rates of the node: f* = f - M^-1 Lambda(x) M dl,
+// dl = f - feq, Lambda(x) = diag(1, R(x), s_free) (Eqs. MRT-Coll, MatrixS, D_ab).  The squared
+// norms of M's rows are in the rates (sfree) or powers of two; the conserved moment, dm[0], is
+// rounding only.  No division: an FP32 one by 5 or 20 is a dozen instructions, an FP64 one a
+// chain on the narrow FP64 pipe.
+template <typename real, int D>
+__device__ __forceinline__ void collide_moments(const KConst<real>& sp, const real* coll, const real* f, const real* dl,
+                                                real* fs) {
   constexpr int Q = Lat<D>::Q;
-  const long long nodes = sp.nodes;
+  real dm[Q];
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    real acc = static_cast<real>(mom(D, i, 0)) * dl[0];
+#pragma unroll
+    for (int q = 1; q < Q; ++q)
+      if (mom(D, i, q) != 0) acc += static_cast<real>(mom(D, i, q)) * dl[q];
+    dm[i] = acc;
+  }
+  real dmp[Q];  // Lambda dm over the rows' norms
+  dmp[0] = dm[0] * (static_cast<real>(1) / static_cast<real>(mom_norm(D, 0)));
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    real acc = static_cast<real>(0);
+#pragma unroll
+    for (int b = 0; b < D; ++b) {
+      const int lo = a < b ? a : b, hi = a < b ? b : a;  // packed upper triangle, row by row
+      const real t = coll[lo * D - lo * (lo - 1) / 2 + hi - lo];
+      acc = b == 0 ? t * dm[1] : acc + t * dm[1 + b];
+    }
+    dmp[1 + a] = acc * static_cast<real>(0.5);
+  }
+#pragma unroll
+  for (int k = D + 1; k < Q; ++k) dmp[k] = sp.sfree[k - D - 1] * dm[k];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    real acc = static_cast<real>(0);
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+      if (mom(D, i, q) != 0) acc += static_cast<real>(mom(D, i, q)) * dmp[i];
+    fs[q] = f[q] - acc;
+  }
+}
+
+// Equilibrium and collision of one node with coefficients of that node:
+// Eq. (Feq) with u(x); BGK f* = f - (f - feq)/lambda(x); MRT in moment space.
+template <typename real, int D, bool MRT>
+__device__ __forceinline__ void collide_node_field(const KConst<real>& sp, const FieldPtrs<real>& fp,
+                                                   const NodeCoef<real, D, MRT>& c, const real* f, const real* F,
+                                                   real* fs) {
+  constexpr int Q = Lat<D>::Q;
   real C = f[0];
 #pragma unroll
   for (int q = 1; q < Q; ++q) C += f[q];
@@ -197,74 +243,22 @@ __device__ __forceinline__ void collide_node_field(const KConst<real>& sp, const
 #pragma unroll
   for (int mu = 0; mu < D; ++mu) {
     const real a = sp.wi * F[mu];
-    const real b = fp.advw[mu * nodes + node] * C;
+    const real b = c.adv[mu] * C;
     dl[2 * mu + 1] = f[2 * mu + 1] - (a + b);
     dl[2 * mu + 2] = f[2 * mu + 2] - (a - b);
   }
   if (!MRT) {
-    const real om = fp.coll[node];
+    const real om = c.coll[0];
 #pragma unroll
     for (int q = 0; q < Q; ++q) fs[q] = f[q] - om * dl[q];
   } else {
-    collide_moments<real, D>(sp, fp, node, f, dl, fs);
+    collide_moments<real, D>(sp, c.coll, f, dl, fs);
   }
   if (fp.src) {  // |w> S_c(x, t) dt, Eq. (LBE_Ket)
-    const real sv = fp.src[node] * static_cast<real>(fp.tf[0]);
+    const real sv = c.src * static_cast<real>(fp.tf[0]);
     fs[0] += sp.w0 * sv;
 #pragma unroll
     for (int q = 1; q < Q; ++q) fs[q] += sp.wi * sv;
-  }
-}
-
-// MRT collision in moment space with the rates of the node: f* = f - M^-1 Lambda(x) M dl,
-// dl = f - feq, Lambda(x) = diag(1, R(x), s_free) (Eqs. MRT-Coll, MatrixS, D_ab)
-template <typename real, int D>
-__device__ __forceinline__ void collide_moments(const KConst<real>& sp, const FieldPtrs<real>& fp, long long node,
-                                                const real* f, const real* dl, real* fs) {
-  constexpr int Q = Lat<D>::Q;
-  const long long nodes = sp.nodes;
-  real dm[Q];
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    real acc = static_cast<real>(mom(D, i, 0)) * dl[0];
-#pragma unroll
-    for (int q = 1; q < Q; ++q)
-      if (mom(D, i, q) != 0) acc += static_cast<real>(mom(D, i, q)) * dl[q];
-    dm[i] = acc;
-  }
-  real R[D][D];
-  if (D == 2) {
-    R[0][0] = fp.coll[node];
-    R[0][1] = R[1][0] = fp.coll[nodes + node];
-    R[1][1] = fp.coll[2 * nodes + node];
-  } else {
-    int k = 0;
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-#pragma unroll
-      for (int b = a; b < D; ++b) {
-        R[a][b] = R[b][a] = fp.coll[k * nodes + node];
-        ++k;
-      }
-  }
-  real dmp[Q];
-  dmp[0] = dm[0];  // conserved moment: rate 1, no effect (dm[0] = 0 up to rounding)
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    real acc = R[a][0] * dm[1];
-#pragma unroll
-    for (int b = 1; b < D; ++b) acc += R[a][b] * dm[1 + b];
-    dmp[1 + a] = acc;
-  }
-#pragma unroll
-  for (int k = D + 1; k < Q; ++k) dmp[k] = sp.sfree[k - D - 1] * dm[k];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    real acc = static_cast<real>(0);
-#pragma unroll
-    for (int i = 0; i < Q; ++i)
-      if (mom(D, i, q) != 0) acc += static_cast<real>(mom(D, i, q)) * dmp[i] / static_cast<real>(mom_norm(D, i));
-    fs[q] = f[q] - acc;
   }
 }
 
@@ -360,8 +354,15 @@ __device__ __forceinline__ void collide_at(const KConst<real>& sp, const real* _
   for (int q = 0; q < Q; ++q) f[q] = f_in[q * nodes + node];
 #pragma unroll
   for (int mu = 0; mu < D; ++mu) Fv[mu] = frac_term(sp, F, mu, node);
-  if (FLD) collide_node_field<real, D, MRT>(sp, fp, node, f, Fv, fs);
-  else collide_node<real, D, MRT, KS>(sp, f, Fv, fs);
+  if constexpr (FLD) {
+    NodeCoef<real, D, MRT> c;
+#pragma unroll
+    for (int k = 0; k < NodeCoef<real, D, MRT>::NR; ++k) c.coll[k] = fp.coll[k * nodes + node];
+#pragma unroll
+    for (int mu = 0; mu < D; ++mu) c.adv[mu] = fp.advw[mu * nodes + node];
+    c.src = fp.src ? fp.src[node] : static_cast<real>(0);
+    collide_node_field<real, D, MRT>(sp, fp, c, f, Fv, fs);
+  } else collide_node<real, D, MRT, KS>(sp, f, Fv, fs);
 }
 
 // Asynchronous prefetch of the 2-D march (FP32): every thread copies the populations and
@@ -700,9 +701,10 @@ __device__ __forceinline__ void march2_pipe(const KConst<float>& sp, const float
 // blocks of 19 warps, 335 instructions per node; 59 us and 165 here); a single 512^2 lattice is a chain of
 // latencies in which the TMA-fed blocks are the faster form (512^2 bf16x6 step 12.4 us against
 // 13.4 us with strips of two rows).
-template <int V>
+template <int V, bool MRT, bool FLD>
 struct StripRow {
   float f[5][V], F[2][V];
+  float coll[MRT ? 3 : 1][V], adv[2][V], src[V];  // FLD
 };
 
 template <int V>
@@ -723,44 +725,70 @@ __device__ __forceinline__ void store_v(float* __restrict__ p, const float (&d)[
 }
 
 // the values of V neighbouring nodes from offset `o` on, zeros where !ok
-template <int V>
+template <int V, bool MRT, bool FLD>
 __device__ __forceinline__ void strip_load(long long nodes, const float* __restrict__ f, const float* __restrict__ F,
-                                           long long o, bool ok, StripRow<V>& r) {
+                                           const FieldPtrs<float>& fp, long long o, bool ok,
+                                           StripRow<V, MRT, FLD>& r) {
+  constexpr int NR = MRT ? 3 : 1;
   if (ok) {
 #pragma unroll
     for (int q = 0; q < 5; ++q) load_v<V>(r.f[q], f + q * nodes + o);
 #pragma unroll
     for (int mu = 0; mu < 2; ++mu) load_v<V>(r.F[mu], F + mu * nodes + o);
+    if constexpr (FLD) {
+#pragma unroll
+      for (int k = 0; k < NR; ++k) load_v<V>(r.coll[k], fp.coll + k * nodes + o);
+#pragma unroll
+      for (int mu = 0; mu < 2; ++mu) load_v<V>(r.adv[mu], fp.advw + mu * nodes + o);
+      if (fp.src) load_v<V>(r.src, fp.src + o);
+    }
   } else {
 #pragma unroll
     for (int v = 0; v < V; ++v) {
 #pragma unroll
       for (int q = 0; q < 5; ++q) r.f[q][v] = 0.f;
       r.F[0][v] = r.F[1][v] = 0.f;
+      if constexpr (FLD) {
+#pragma unroll
+        for (int k = 0; k < NR; ++k) r.coll[k][v] = 0.f;
+        r.adv[0][v] = r.adv[1][v] = r.src[v] = 0.f;
+      }
     }
   }
 }
 
 // equilibrium and collision of the V nodes of a loaded row
-template <int V, bool MRT, bool KS>
-__device__ __forceinline__ void strip_collide(const KConst<float>& sp, const StripRow<V>& r, float (&fs)[5][V]) {
+template <int V, bool MRT, bool KS, bool FLD>
+__device__ __forceinline__ void strip_collide(const KConst<float>& sp, const FieldPtrs<float>& fp,
+                                              const StripRow<V, MRT, FLD>& r, float (&fs)[5][V]) {
 #pragma unroll
   for (int v = 0; v < V; ++v) {
     float f[5], o[5];
     const float F[2] = {r.F[0][v], r.F[1][v]};
 #pragma unroll
     for (int q = 0; q < 5; ++q) f[q] = r.f[q][v];
-    collide_node<float, 2, MRT, KS>(sp, f, F, o);
+    if constexpr (FLD) {
+      NodeCoef<float, 2, MRT> c;
+#pragma unroll
+      for (int k = 0; k < NodeCoef<float, 2, MRT>::NR; ++k) c.coll[k] = r.coll[k][v];
+      c.adv[0] = r.adv[0][v];
+      c.adv[1] = r.adv[1][v];
+      c.src = r.src[v];
+      collide_node_field<float, 2, MRT>(sp, fp, c, f, F, o);
+    } else {
+      collide_node<float, 2, MRT, KS>(sp, f, F, o);
+    }
 #pragma unroll
     for (int q = 0; q < 5; ++q) fs[q][v] = o[q];
   }
 }
 
-// bf16 operand parts of V neighbouring values at element o (write_split of each, packed stores)
+// operands of V neighbouring values at element o (write_split of each, packed stores)
 template <int SPLIT, int V>
 __device__ __forceinline__ void write_split_v(const SplitOut& so, long long o, const float (&c)[V]) {
-  static_assert(SPLIT == 1 || SPLIT == 3, "bf16 forms");
-  if constexpr (V == 1) {
+  if constexpr (SPLIT == 2) {
+    store_v<V>(static_cast<float*>(so.hi) + o, c);
+  } else if constexpr (V == 1) {
     write_split<SPLIT>(so, o, c[0]);
   } else {
     const __nv_bfloat162 h = __floats2bfloat162_rn(c[0], c[1]);
@@ -775,19 +803,20 @@ __device__ __forceinline__ void write_split_v(const SplitOut& so, long long o, c
 }
 
 // the warp's strip (nodes x0 .. x0 + 32 V - 1), rows y0 .. y1 - 1; its mass partial to mpart[slot]
-template <int V, bool MRT, int SPLIT, bool KS>
+template <int V, bool MRT, int SPLIT, bool KS, bool FLD = false>
 __device__ __forceinline__ void strip_march(const KConst<float>& sp, const float* __restrict__ f_in,
                                             const float* __restrict__ F, float* __restrict__ f_out,
                                             float* __restrict__ C_out, int* __restrict__ flag, const SplitOut& so,
-                                            int x0, int y0, int y1, double* mpart, int slot) {
+                                            int x0, int y0, int y1, double* mpart, int slot,
+                                            const FieldPtrs<float>& fp = FieldPtrs<float>{}) {
   const int n0 = sp.n[0], n1 = sp.n[1], lane = threadIdx.x & 31;
   const long long nodes = sp.nodes;
   const int gx = x0 + V * lane;
   const bool in_x = gx < n0;  // (n0 is a multiple of V)
   const bool side = x0 == 0 || x0 + 32 * V >= n0;
-  StripRow<V> row[2];
-  auto load = [&](int y, StripRow<V>& r) {
-    strip_load<V>(nodes, f_in, F, (long long)y * n0 + gx, in_x && y >= 0 && y < n1, r);
+  StripRow<V, MRT, FLD> row[2];
+  auto load = [&](int y, StripRow<V, MRT, FLD>& r) {
+    strip_load(nodes, f_in, F, fp, (long long)y * n0 + gx, in_x && y >= 0 && y < n1, r);
   };
   load(y0 - 1, row[0]);
   load(y0, row[1]);
@@ -796,10 +825,10 @@ __device__ __forceinline__ void strip_march(const KConst<float>& sp, const float
   float h = 0.f;
   auto ring = [&](int yb) {
     const int hx = lane < 16 ? x0 - 1 : x0 + 32 * V, hy = yb + (lane & 15);
-    StripRow<1> r;
+    StripRow<1, MRT, FLD> r;
     float o[5][1];
-    strip_load<1>(nodes, f_in, F, (long long)hy * n0 + hx, hx >= 0 && hx < n0 && hy < y1, r);
-    strip_collide<1, MRT, KS>(sp, r, o);
+    strip_load(nodes, f_in, F, fp, (long long)hy * n0 + hx, hx >= 0 && hx < n0 && hy < y1, r);
+    strip_collide<1, MRT, KS, FLD>(sp, fp, r, o);
     h = lane < 16 ? o[1][0] : o[2][0];
   };
   ring(y0);
@@ -808,11 +837,18 @@ __device__ __forceinline__ void strip_march(const KConst<float>& sp, const float
   float c[4][V], p3[V];  // f*_0..3 of the last collided row, f*_3 of the one before
 #pragma unroll
   for (int v = 0; v < V; ++v) c[0][v] = c[1][v] = c[2][v] = c[3][v] = p3[v] = 0.f;
-  auto advance = [&](int y, StripRow<V>& r) {
-    float n[5][V];
-    strip_collide<V, MRT, KS>(sp, r, n);
-    if (y + 2 <= y1) load(y + 2, r);
+  auto advance = [&](int y, StripRow<V, MRT, FLD>& r) {
     const int yo = y - 1;  // the row that is complete now
+    float g[2][V];         // g_mu of that row
+    if constexpr (FLD) {
+      if (in_x && yo >= y0 && (fp.gsplit || fp.G)) {
+#pragma unroll
+        for (int mu = 0; mu < 2; ++mu) load_v<V>(g[mu], fp.g + mu * nodes + (long long)yo * n0 + gx);
+      }
+    }
+    float n[5][V];
+    strip_collide<V, MRT, KS, FLD>(sp, fp, r, n);
+    if (y + 2 <= y1) load(y + 2, r);
     if (yo >= y0) {
       const int k = (yo - y0) & 15;
       if (yo > y0 && k == 0) ring(yo);
@@ -848,8 +884,11 @@ __device__ __forceinline__ void strip_march(const KConst<float>& sp, const float
             }
           }
           if (n_unknown > 0) {
-            // Eq. (Dirichlet_BC); with k unknown populations each takes 1/k of the deficit
-            const float fill = (sp.C_wall - C[v]) / static_cast<float>(n_unknown);
+            // Eq. (Dirichlet_BC); with k unknown populations each takes 1/k of the deficit; the
+            // wall value varies with position and time when given (Section 2.5)
+            float cwall = sp.C_wall;
+            if (FLD && fp.cw && in_x) cwall = fp.cw[(long long)yo * n0 + gx + v] * static_cast<float>(fp.tf[1]);
+            const float fill = (cwall - C[v]) / static_cast<float>(n_unknown);
 #pragma unroll
             for (int q = 0; q < 5; ++q)
               if (!known[q]) o[q][v] = fill;
@@ -864,7 +903,28 @@ __device__ __forceinline__ void strip_march(const KConst<float>& sp, const float
 #pragma unroll
         for (int q = 0; q < 5; ++q) store_v<V>(f_out + q * nodes + node, o[q]);
         if (SPLIT == 0 || C_out) store_v<V>(C_out + node, C);
-        if constexpr (SPLIT != 0) write_split_v<SPLIT, V>(so, (long long)yo * so.ldp + gx, C);
+        bool parts = SPLIT != 0;
+        if constexpr (FLD) {
+          if (fp.gsplit || fp.G) {  // the operator's inputs of the next step: g_mu(x) C, one per axis
+#pragma unroll
+            for (int mu = 0; mu < 2; ++mu) {
+              float G[V];
+#pragma unroll
+              for (int v = 0; v < V; ++v) G[v] = g[mu][v] * C[v];
+              if (fp.G) store_v<V>(fp.G + mu * nodes + node, G);
+              if constexpr (SPLIT == 1 || SPLIT == 3) {
+                SplitOut sm{};
+                sm.hi = fp.gs[mu][0];
+                sm.lo = fp.gs[mu][1];
+                sm.lo2 = fp.gs[mu][2];
+                if (fp.gsplit) write_split_v<SPLIT, V>(sm, (long long)yo * fp.gldp + gx, G);
+              }
+            }
+          }
+          if (fp.gsplit) parts = false;
+        }
+        if constexpr (SPLIT != 0)
+          if (parts) write_split_v<SPLIT, V>(so, (long long)yo * so.ldp + gx, C);
 #pragma unroll
         for (int v = 0; v < V; ++v) {
           bad = __fmaf_rn(C[v], 0.f, bad);  // NaN once a C is not finite
@@ -918,6 +978,29 @@ collide_stream_march2_kernel(const KConst<float> sp, const float* __restrict__ f
   if (early) pdl_trigger();
   march2_pipe<MRT, SPLIT>(sp, f_in, F, f_out, C_out, flag, so, ychunk, blockIdx.x, blockIdx.y, pipe_stage, mpart,
                           block_linear());
+  if (!early) pdl_trigger();
+}
+
+// A single large 2-D FP32 lattice whose coefficients vary from node to node, on strips: 14 values
+// in and 6 to 18 out per node, bound by the latency of its loads from L2.  Against one block of
+// 32 x 16 nodes per tile: 512^2 bf16x6 step 17.6 -> 14.7 us, 1000 x 900 51.7 -> 40.5.
+template <int V, bool MRT, int SPLIT>
+__global__ void __launch_bounds__(32 * kStripWarps, 4)
+collide_stream_fields2_kernel(const __grid_constant__ KConst<float> sp, const float* __restrict__ f_in,
+                              const float* __restrict__ F, float* __restrict__ f_out, float* __restrict__ C_out,
+                              int* __restrict__ flag, const __grid_constant__ SplitOut so,
+                              const __grid_constant__ FieldPtrs<float> fp, const StripGrid g, int early,
+                              double* mpart) {
+  if (early) pdl_trigger();
+  // programmatic dependent launch: the operator's F (and the previous step's f) must be
+  // complete before any load
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int item = blockIdx.x * kStripWarps + (threadIdx.x >> 5);
+  if (item < g.items) {
+    const int y0 = item / g.strips * g.rows;
+    strip_march<V, MRT, SPLIT, false, true>(sp, f_in, F, f_out, C_out, flag, so, item % g.strips * 32 * V, y0,
+                                            min(y0 + g.rows, sp.n[1]), mpart, item, fp);
+  }
   if (!early) pdl_trigger();
 }
 
@@ -1729,6 +1812,20 @@ bool one_wave(const dim3& g) { return (long long)g.x * g.y * g.z <= 2LL * device
 // FP32 step 32.8 us with the early trigger, 22.9 without).
 int early_trigger(const lbm_s* h, const dim3& g) { return h->tc && one_wave(g) ? 1 : 0; }
 
+// 2-D FP32 lattices with coefficients per node: rows of a warp's strip in units of kStripRows, or 0
+// for the plain march.  That one collides each node once and is the faster form where its blocks
+// fit one wave (step, strips / plain: 64^2 bf16x6 7.9 / 6.8 us, 300^2 13.0 / 11.9, 300^2 FP32
+// 18.1 / 15.7); beyond, its second wave costs more than the strips' extra rows (512^2 bf16x6
+// 14.7 / 17.6, FP32 24.5 / 26.7, 1000 x 900 bf16x6 40.5 / 51.7).  The strips take the fewest rows
+// that fit one wave (1000 x 900 with 2 / 4 / 6 / 8 rows: 44.3 / 42.6 / 40.6 / 44.5 us), at most 8.
+int fields2_chunk(const lbm_s* h) {
+  if (h->cs_chunk > 0) return h->cs_chunk;
+  if (one_wave(dim3((h->sp.n[0] + TX - 1) / TX, (h->sp.n[1] + TY - 1) / TY, 1))) return 0;
+  int c = 1;
+  while (c < 4 && strip_grid(h->sp.n, c).items > 4LL * kStripWarps * device_sms()) ++c;
+  return c;
+}
+
 template <bool MRT, int SPLIT>
 cudaError_t launch_march2(const cudaLaunchConfig_t& cfg, const KConst<float>& sp, const float* fi, const float* F,
                           float* fo, float* Co, int* flag, const SplitOut& so, int ychunk, int early, double* mpart) {
@@ -1855,11 +1952,7 @@ cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out
   cfg.attrs = at;
   cfg.numAttrs = 1;
   if (h->fld.on) {
-    // coefficients per node: the plain march with the per-node collision (2-D: one plane)
-    const int nz = (D == 2) ? 1 : (h->cs_chunk > 0 ? std::min(h->cs_chunk, sp.n[2]) : z_chunks((long long)bx * by, sp.n[2]));
-    cfg.gridDim = dim3(bx, by, nz);
-    h->cs_nparts = kMassSlots * bx * by * nz;
-    const int early = early_trigger(h, cfg.gridDim);
+    // coefficients per node: strips in 2-D, the plain march in 3-D
     FieldPtrs<real> fp{static_cast<const real*>(h->fld.coll), static_cast<const real*>(h->fld.advw),
                        static_cast<const real*>(h->fld.g),    static_cast<real*>(h->fld.G),
                        static_cast<const real*>(h->fld.src),  static_cast<const real*>(h->fld.cw),
@@ -1871,21 +1964,33 @@ cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out
         for (int k = 0; k < 3; ++k) fp.gs[mu][k] = h->tc->gp[mu][k];
     }
     if constexpr (sizeof(real) == 8) return launch_march64_any<D, MRT, true>(h, cfg, sp, fi, F, fo, Co, fp);
-    if constexpr (sizeof(real) == 4) {
-      // tensor-core forms: the march also writes the operator's operands of the new C
-      if (split == 1)
-        return cudaLaunchKernelEx(&cfg, collide_stream_march_kernel<real, D, MRT, 1, true>, sp, fi, F, fo, Co, flag, so,
-                                  nz, early, mp, fp);
-      if (split == 2)
-        return cudaLaunchKernelEx(&cfg, collide_stream_march_kernel<real, D, MRT, 2, true>, sp, fi, F, fo, Co, flag, so,
-                                  nz, early, mp, fp);
-      if (split == 3)
-        return cudaLaunchKernelEx(&cfg, collide_stream_march_kernel<real, D, MRT, 3, true>, sp, fi, F, fo, Co, flag, so,
-                                  nz, early, mp, fp);
+    const int chunk = D == 2 ? fields2_chunk(h) : 0;
+    if constexpr (D == 2 && sizeof(real) == 4)
+    if (chunk > 0) {
+      const StripGrid g = strip_grid(sp.n, chunk);
+      cfg.gridDim = dim3((g.items + kStripWarps - 1) / kStripWarps);
+      cfg.blockDim = dim3(32 * kStripWarps);
+      h->cs_nparts = g.items;
+      auto go = [&](auto v2, auto v1) {
+        return cudaLaunchKernelEx(&cfg, g.v == 2 ? v2 : v1, sp, fi, F, fo, Co, flag, so, fp, g, h->pdl && h->tc ? 1 : 0, mp);
+      };
+      // the tensor-core forms' march also writes the operator's operands of the new C
+      if (split == 0) return go(collide_stream_fields2_kernel<2, MRT, 0>, collide_stream_fields2_kernel<1, MRT, 0>);
+      if (split == 1) return go(collide_stream_fields2_kernel<2, MRT, 1>, collide_stream_fields2_kernel<1, MRT, 1>);
+      if (split == 2) return go(collide_stream_fields2_kernel<2, MRT, 2>, collide_stream_fields2_kernel<1, MRT, 2>);
+      return go(collide_stream_fields2_kernel<2, MRT, 3>, collide_stream_fields2_kernel<1, MRT, 3>);
     }
-    if constexpr (sizeof(real) == 4)
-      return cudaLaunchKernelEx(&cfg, collide_stream_march_kernel<real, D, MRT, 0, true>, sp, fi, F, fo, Co, flag, so,
-                                nz, early, mp, fp);
+    if constexpr (sizeof(real) == 4) {
+      const int nz = D == 2 ? 1 : h->cs_chunk > 0 ? std::min(h->cs_chunk, sp.n[2]) : z_chunks((long long)bx * by, sp.n[2]);
+      cfg.gridDim = dim3(bx, by, nz);
+      h->cs_nparts = kMassSlots * bx * by * nz;
+      const int early = early_trigger(h, cfg.gridDim);
+      auto go = [&](auto k) { return cudaLaunchKernelEx(&cfg, k, sp, fi, F, fo, Co, flag, so, nz, early, mp, fp); };
+      if (split == 0) return go(collide_stream_march_kernel<real, D, MRT, 0, true>);
+      if (split == 1) return go(collide_stream_march_kernel<real, D, MRT, 1, true>);
+      if (split == 2) return go(collide_stream_march_kernel<real, D, MRT, 2, true>);
+      return go(collide_stream_march_kernel<real, D, MRT, 3, true>);
+    }
   }
   if constexpr (sizeof(real) == 8)
     return launch_march64_any<D, MRT, false>(h, cfg, sp, fi, F, fo, Co, FieldPtrs<double>{});
@@ -2072,6 +2177,11 @@ bool cs_one_wave(const lbm_s* h) {
     return one_wave(dim3(pl.bx, pl.by, pl.nz));
   }
   const int bx = (h->sp.n[0] + TX - 1) / TX, by = (h->sp.n[1] + TY - 1) / TY;
+  if (h->d == 2 && h->elem == 4 && h->fld.on) {
+    const int chunk = fields2_chunk(h);  // strips: four blocks to an SM
+    if (chunk > 0) return strip_grid(h->sp.n, chunk).items <= 4LL * kStripWarps * device_sms();
+    return one_wave(dim3(bx, by, 1));
+  }
   if (h->d == 2 && h->elem == 4) {
     const int ychunk = h->cs_chunk > 0 ? std::min(h->cs_chunk, by) : ychunk_for((long long)bx * by, by);
     return one_wave(dim3(bx, (by + ychunk - 1) / ychunk, 1));
@@ -2093,6 +2203,7 @@ long long cs_max_parts(const lbm_s* h) {
 int cs_chunk_default(const lbm_s* h) {
   const int bx = (h->sp.n[0] + TX - 1) / TX, by = (h->sp.n[1] + TY - 1) / TY;
   if (h->is_batch()) return kBatchChunk;
+  if (h->d == 2 && h->elem == 4 && h->fld.on) return fields2_chunk(h);
   if (h->d == 2) return h->elem == 4 ? ychunk_for((long long)bx * by, by) : 1;
   return h->elem == 8 ? march64_plan(h, 0).nz : z_chunks((long long)bx * by, h->sp.n[2]);
 }

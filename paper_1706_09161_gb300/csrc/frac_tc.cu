@@ -22,8 +22,8 @@
 // with tcgen05.commit, then all four warps drain the accumulator (tcgen05.ld, one
 // lane quarter per warp) into a shared [BN][128] tile that one TMA store writes to F.
 // Small problems split the contraction over ksplit CTAs, CTA `rank` contracting its k-range.
-// Where F is stored with TMA and read by the 2-D march, the partial tiles stay in slots of F,
-// [rank][axis][node], which the march adds in rank order.  Else (ragged rows, 3-D) the CTAs of a
+// Where F is stored with TMA and read by the TMA-fed 2-D march, the partial tiles stay in slots of F,
+// [rank][axis][node], which the march adds in rank order.  Else (ragged rows, 3-D, varying coefficients) the CTAs of a
 // tile form a cluster that adds the partial tiles in rank order through distributed shared
 // memory, each CTA summing and storing its share of the rows.  Either way the result does not
 // depend on timing.  (Measured: 301 x 203 bf16x6 step 13.5 us with slots, 10.6 with clusters,
@@ -1033,8 +1033,10 @@ int tc_replan(lbm_s* h, int bn, int ks, int persist) {
       return LBM_ECUDA;
   }
   P.F = static_cast<float*>(h->dev.F);
-  // row chunks of an output tile: what one CTA of a cluster stores, at most 32 rows
-  P.slots = ks > 1 && h->d == 2 && P.tma_store ? 1 : 0;
+  // partial tiles in slots of F only where the TMA-fed 2-D march reads them (the march of varying
+  // coefficients reads F with plain loads); row chunks of an output tile: what one CTA of a cluster
+  // stores, at most 32 rows
+  P.slots = ks > 1 && h->d == 2 && P.tma_store && !h->fld.on ? 1 : 0;
   const size_t need = (size_t)(P.slots ? ks : 1) * h->d * h->sp.nodes;
   if (need > h->f_elems) {
     cudaStreamSynchronize(h->stream);

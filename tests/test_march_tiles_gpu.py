@@ -117,3 +117,46 @@ def test_one_batch_call_equals_single_steps(L, kind):
             b.step(1)
         for i in range(len(cases)):
             assert np.array_equal(a.C(i), b.C(i)), i
+
+
+# strips of 64 or 32 nodes at their edges, one to many rows per warp, coefficients per node
+@pytest.mark.parametrize("kind", ["fp32", "bf16split", "bf16x6split", "tf32split"])
+@pytest.mark.parametrize("collision", ["bgk", "mrt"])
+@pytest.mark.parametrize("grid", [(3, 3), (31, 17), (33, 34), (64, 18), (66, 7), (130, 70)])
+def test_fields_strips(L, kind, collision, grid):
+    pb, C0 = _case(grid, 701 + sum(grid), collision)
+    fields = W.smooth_fields(np.random.default_rng(5), grid, collision, D0=0.03, g_amp=0.2, u_amp=0.03)
+    n = 6
+    f = []
+    with L.Lattice(pb, C0, kind) as lat:
+        for with_fields in (True, False, True):  # back to constant coefficients and on again
+            lat.set_fields(**(fields if with_fields else {}))
+        for chunk in (1, 3, 40):
+            lat.configure(0, 0, 0, chunk, 0)
+            lat.reset()
+            lat.step(n)
+            f.append(lat.f())
+            C, mass = lat.C(), lat.mass()
+            assert np.array_equal(f[0], f[-1]), chunk
+            assert abs(mass - C.sum()) <= 1e-6 * np.abs(C).sum(), chunk
+    l2_tol, node_tol, ref = arith_bounds.bounds(pb, C0, n, kind, fields=fields)
+    arith_bounds.assert_close(C, ref, l2_tol, node_tol, f"{grid} {collision} {kind}")
+
+
+# a split contraction adds its partial tiles in the operator when coefficients vary, in the march
+# when they don't, also after the coefficients are constant again
+@pytest.mark.parametrize("kind", ["bf16split", "bf16x6split"])
+def test_fields_with_a_split_contraction(L, kind):
+    pb, C0 = _case((260, 200), 809)
+    one = np.ones(pb.shape)
+    with L.Lattice(pb, C0, kind) as a, L.Lattice(pb, C0, kind) as b:
+        for lat in (a, b):
+            lat.configure(128, 2, 0, 0, 0)
+            lat.reset()
+        b.set_fields(u=np.stack([pb.u[0] * one, pb.u[1] * one]))
+        for mu in range(2):
+            assert arith_bounds.rel_l2(b.F(mu), a.F(mu)) < {"bf16split": 4e-5, "bf16x6split": 2e-6}[kind], mu
+        b.set_fields()
+        a.step(4)
+        b.step(4)
+        assert np.array_equal(a.f(), b.f())
