@@ -415,10 +415,7 @@ int init_from_C(lbm_s* h) {
   h->t_steps = 0;
   int rc = run_frac(h, h->stream);
   if (rc) return rc;
-  LBM_CUDA(lbm::launch_init_equilibrium(h, h->dev.f[h->cur], h->stream));
-  LBM_CUDA(lbm::launch_moment(h, h->dev.f[h->cur], h->dev.C, h->stream));
-  if (uses_tc(h)) LBM_CUDA(lbm::launch_split_C(h, h->stream));
-  if (h->fld.on) LBM_CUDA(lbm::launch_scale_fields(h, h->stream));
+  LBM_CUDA(lbm::launch_init_state(h, h->dev.f[h->cur], h->stream));
   return LBM_OK;
 }
 

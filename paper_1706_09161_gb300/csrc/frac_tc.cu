@@ -598,13 +598,11 @@ frac_tc_persist_batch_kernel(const TcMaps* __restrict__ maps, const TcParams* __
 template <int E>
 __global__ void split_C_kernel(const float* __restrict__ C, void* __restrict__ hi, void* __restrict__ lo,
                                void* __restrict__ lo2, int n0, int n1, int n2, int ldp) {
-  const long long total = (long long)n0 * n1 * n2;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int x = static_cast<int>(i % n0);
-    const long long row = i / n0;
-    const long long o = row * ldp + x;
-    const float c = C[i];
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, rows = n1 * n2;
+  if (x >= n0) return;
+  for (int row = blockIdx.y * blockDim.y + threadIdx.y; row < rows; row += gridDim.y * blockDim.y) {
+    const long long o = (long long)row * ldp + x;
+    const float c = C[(long long)row * n0 + x];
     if (E == 2) {
       // each part the bf16 rounding of what the previous ones left (exact FP32 residuals)
       const __nv_bfloat16 h = __float2bfloat16_rn(c);
@@ -627,10 +625,11 @@ struct GParts {
 __global__ void split_G_kernel(const float* __restrict__ C, const float* __restrict__ g, GParts gp, int d, int cparts,
                                int n0, int n1, int n2, int ldp) {
   const long long total = (long long)n0 * n1 * n2;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int x = static_cast<int>(i % n0);
-    const long long o = (i / n0) * ldp + x;
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, rows = n1 * n2;
+  if (x >= n0) return;
+  for (int row = blockIdx.y * blockDim.y + threadIdx.y; row < rows; row += gridDim.y * blockDim.y) {
+    const long long i = (long long)row * n0 + x;
+    const long long o = (long long)row * ldp + x;
     const float c = C[i];
     for (int mu = 0; mu < d; ++mu) {
       const float v = g[mu * total + i] * c;
@@ -1190,10 +1189,7 @@ cudaError_t launch_split_T(const lbm_s* h, cudaStream_t s) {
   const float* C = static_cast<const float*>(h->dev.C);
   const float* G = static_cast<const float*>(h->fld.G);
   if (p->gvar) {
-    long long b = (nodes + 255) / 256;
-    const long long cap = 16LL * device_sms();
-    if (b > cap) b = cap;
-    split_C_kernel<4><<<(int)b, 256, 0, s>>>(G, h->dev.Chi, nullptr, nullptr, n0, n1, n2, p->ldp);
+    split_C_kernel<4><<<row_grid(h), row_block(h), 0, s>>>(G, h->dev.Chi, nullptr, nullptr, n0, n1, n2, p->ldp);
   }
   for (int mu = 1; mu < h->d; ++mu)
     split_T_kernel<<<dim3((n0 + 127) / 128, p->tg[mu], mu == 1 ? n2 : n1), 128, 0, s>>>(
@@ -1236,9 +1232,6 @@ int tc_set_gfield(lbm_s* h, bool on) {
 cudaError_t launch_split_C(const lbm_s* h, cudaStream_t s) {
   const TcPlan* p = h->tc;
   if (!p) return cudaErrorNotSupported;
-  long long b = (h->sp.nodes + 255) / 256;
-  const long long cap = 16LL * device_sms();
-  if (b > cap) b = cap;
   if (p->gvar && p->elem == 4) {  // tf32 with g(x): G = g C, then the operands from G
     cudaError_t e = launch_scale_fields(h, s);
     if (e != cudaSuccess) return e;
@@ -1248,16 +1241,16 @@ cudaError_t launch_split_C(const lbm_s* h, cudaStream_t s) {
     GParts gp{};
     for (int mu = 0; mu < 3; ++mu)
       for (int k = 0; k < 3; ++k) gp.p[mu][k] = p->gp[mu][k];
-    split_G_kernel<<<(int)b, 256, 0, s>>>(static_cast<const float*>(h->dev.C), static_cast<const float*>(h->fld.g), gp,
+    split_G_kernel<<<row_grid(h), row_block(h), 0, s>>>(static_cast<const float*>(h->dev.C), static_cast<const float*>(h->fld.g), gp,
                                           h->d, p->cparts, h->sp.n[0], h->sp.n[1], h->sp.n[2], p->ldp);
     return cudaGetLastError();
   }
   if (p->elem == 2)
-    split_C_kernel<2><<<(int)b, 256, 0, s>>>(static_cast<const float*>(h->dev.C), h->dev.Chi, h->dev.Clo,
+    split_C_kernel<2><<<row_grid(h), row_block(h), 0, s>>>(static_cast<const float*>(h->dev.C), h->dev.Chi, h->dev.Clo,
                                              p->cparts == 3 ? h->dev.Cl2 : nullptr, h->sp.n[0], h->sp.n[1],
                                              h->sp.n[2], p->ldp);
   else
-    split_C_kernel<4><<<(int)b, 256, 0, s>>>(static_cast<const float*>(h->dev.C), h->dev.Chi, h->dev.Clo, nullptr,
+    split_C_kernel<4><<<row_grid(h), row_block(h), 0, s>>>(static_cast<const float*>(h->dev.C), h->dev.Chi, h->dev.Clo, nullptr,
                                              h->sp.n[0], h->sp.n[1], h->sp.n[2], p->ldp);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
