@@ -1030,7 +1030,6 @@ collide_stream_march_kernel(const KConst<real> sp, const real* __restrict__ f_in
 // planes ahead, 410 instructions per node) with its z chunks: 256^3 bf16x6 231 -> 209 us (1317 MB,
 // 93% of the measured copy rate), tf32x3 247 -> 229, 160 x 128 x 100 43 -> 33.
 constexpr int TW = TX + 8, TH = TY + 2;  // staged window: x from x0 - 4, y from y0 - 1
-constexpr int TCP = TX;  // row pitch of the tf32 C ring
 constexpr int TMA_STAGES = 3;
 constexpr uint32_t TMA_F_BYTES = 7u * TH * TW * 4;   // D3Q7 populations
 constexpr uint32_t TMA_FF_BYTES = 3u * TH * TW * 4;  // fractional terms
@@ -1361,13 +1360,9 @@ collide_stream_tma3_kernel(const __grid_constant__ KConst<float> sp, const __gri
 // ---------------------------------------------------------------------------- TMA-fed 2-D march
 // FP32 forms with n0 % 4 == 0: the block walks `ychunk` tiles up y; per tile one thread
 // loads the 40 x 18 window of the 5 populations and the 2 fractional terms with two 3-D
-// TMA box loads into a 3-stage ring, two tiles ahead.  Otherwise as march2_pipe.
+// TMA box loads into a 3-stage ring, two tiles ahead.
 constexpr uint32_t TMA2_F_BYTES = 5u * TH * TW * 4;
-constexpr uint32_t TMA2_FF_BYTES = 2u * TH * TW * 4;
-constexpr uint32_t TMA2_TX = TMA2_F_BYTES + TMA2_FF_BYTES;
 constexpr uint32_t TMA2_FF_OFF = (TMA2_F_BYTES + 127) / 128 * 128;
-constexpr uint32_t TMA2_STAGE = (TMA2_FF_OFF + TMA2_FF_BYTES + 127) / 128 * 128;
-constexpr size_t TMA2_SMEM = (size_t)TMA_STAGES * TMA2_STAGE + 128 /*align*/ + 64 /*barriers*/;
 // with ks split-K partial sums the fractional-term window holds 2 ks planes; two stages
 // then (the ring must leave room for two blocks per SM up to ks = 4)
 __host__ __device__ constexpr uint32_t tma2_ff_bytes(int ks) { return 2u * ks * TH * TW * 4; }
@@ -1387,19 +1382,14 @@ __device__ __forceinline__ void cs_tma_3d(void* dst, const CUtensorMap* map, int
       : "memory");
 }
 
-// tf32: C of the last two tile rows (slot t & 1), the source of the y-contiguous split
-__shared__ float s_c2[2 * TY * TCP];
-
-template <bool MRT, int SPLIT, bool KS = false>
+// The collide-stream phase of the fused step (blocks of 32 x 19 threads, one node per thread).
+template <bool MRT>
 __device__ __forceinline__ void march2_tma(const KConst<float>& sp, const CUtensorMap* map_f,
                                            const CUtensorMap* map_F, float* __restrict__ f_out,
                                            float* __restrict__ C_out, int* __restrict__ flag, const SplitOut& so,
                                            int ychunk, int bx, int byc, uint8_t* raw, double* mpart, int mslot) {
   constexpr int D = 2, Q = 5;
   auto& s_m = s_m2;
-  float* s_c = nullptr;
-  if constexpr (SPLIT == 2) s_c = s_c2;
-  const bool wT = SPLIT == 2 && so.thi[0] != nullptr;
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 127) & ~uintptr_t(127));
   const int ks = sp.ksum;
   const int nst = tma2_nst(ks);
@@ -1431,16 +1421,6 @@ __device__ __forceinline__ void march2_tma(const KConst<float>& sp, const CUtens
   const bool in_x = gx >= 0 && gx < n0;
   auto stage_of = [&](int t) { return (t - tr0) % nst; };
   auto parity_of = [&](int t) { return static_cast<uint32_t>(((t - tr0) / nst) & 1); };
-  // tile row t to the y copy (element (x, y) at thi[0][(y/4 tpx + x) 4 + y%4]): warp w < 4
-  // writes y group 4t + w for the tile's 32 x (512 contiguous bytes)
-  auto flush_T = [&](int t) {
-    const int xi = lane, yq = 4 * wy;
-    if (wy < 4 && x0 + xi < n0 && t * TY + yq < n1) {
-      const float* r = &s_c[((t & 1) * TY + yq) * TCP + xi];
-      const long long o = ((long long)((t * TY + yq) >> 2) * so.tpx + x0 + xi) * 4;
-      *reinterpret_cast<float4*>(so.thi[0] + o) = make_float4(r[0], r[TCP], r[2 * TCP], r[3 * TCP]);
-    }
-  };
   auto issue = [&](int t) {
     const int s = stage_of(t);
     uint8_t* st = ring + (size_t)s * stg;
@@ -1476,7 +1456,7 @@ __device__ __forceinline__ void march2_tma(const KConst<float>& sp, const CUtens
         for (int k = 1; k < ks; ++k) acc += st[TMA2_FF_OFF / 4 + ((k * D + mu) * TH + ly) * TW + lx];
         Fv[mu] = acc;
       }
-      collide_node<float, D, MRT, KS>(sp, fv, Fv, fs);
+      collide_node<float, D, MRT>(sp, fv, Fv, fs);
     }
     if (owner) {
       s_m[buf][0][sy][sx] = fs[1];
@@ -1497,9 +1477,7 @@ __device__ __forceinline__ void march2_tma(const KConst<float>& sp, const CUtens
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       issue(tr + nst);
     }
-    if (wT && tr > tr0) flush_T(tr - 1);  // its slot is rewritten only after the next barrier
     const int gy = tr * TY + dy;
-    if (SPLIT == 2 && wT && owner && !(in_x && gy < n1)) s_c[((tr & 1) * TY + dy) * TCP + dx] = 0.f;
     if (owner && in_x && gy < n1) {
       float fv[Q];
       bool known[Q];
@@ -1542,17 +1520,12 @@ __device__ __forceinline__ void march2_tma(const KConst<float>& sp, const CUtens
       const long long node = gx + (long long)n0 * gy;
 #pragma unroll
       for (int q = 0; q < Q; ++q) f_out[q * nodes + node] = fv[q];
-      if (SPLIT == 0 || C_out) C_out[node] = C;
-      if (SPLIT) write_split<SPLIT>(so, (long long)gy * so.ldp + gx, C);
-      if (SPLIT == 2 && wT) s_c[((tr & 1) * TY + dy) * TCP + dx] = C;
+      C_out[node] = C;
+      write_split<1>(so, (long long)gy * so.ldp + gx, C);
       bad |= !isfinite(C);
       macc.add(C);
     }
     buf ^= 1;
-  }
-  if (wT) {
-    __syncthreads();
-    flush_T(tr1 - 1);
   }
   // after a timeout no copy may still be landing in this block's shared memory
   if (tid == 0) {
@@ -1565,16 +1538,205 @@ __device__ __forceinline__ void march2_tma(const KConst<float>& sp, const CUtens
   block_mass(macc, mpart, mslot);
 }
 
+// The two-kernel step's form: two x-neighbours per thread, warps as in collide_stream_tma3_kernel.
+// A 512^2 lattice sits in L2: the kernel is a chain of window load, collision and stores, in which
+// the instructions per node count (one node per thread, 19 warps: 335).  512^2 bf16x6 step 12.5 ->
+// 11.2 us, FP32 23.2 -> 22.4.
 template <bool MRT, int SPLIT>
-__global__ void __launch_bounds__(TX*(TY + HALO_WARPS), 2)
-collide_stream_tma2_kernel(const KConst<float> sp, const __grid_constant__ CUtensorMap map_f,
+__global__ void __launch_bounds__(32 * T3_WARPS, 2)
+collide_stream_tma2_kernel(const __grid_constant__ KConst<float> sp, const __grid_constant__ CUtensorMap map_f,
                            const __grid_constant__ CUtensorMap map_F, float* __restrict__ f_out,
-                           float* __restrict__ C_out, int* __restrict__ flag, SplitOut so, int ychunk, int early,
-                           double* mpart) {
+                           float* __restrict__ C_out, int* __restrict__ flag, const __grid_constant__ SplitOut so,
+                           int ychunk, int early, double* mpart) {
+  constexpr int D = 2, Q = 5;
   extern __shared__ uint8_t cs_raw2[];
+  __shared__ __align__(8) float s_up[2][TY + 1][TX];  // f*_3 of row r - 1 at [r]
+  __shared__ __align__(8) float s_dn[2][TY + 1][TX];  // f*_4 of row r at [r]
+  __shared__ float s_x[2][2][TY];                     // f*_1 of the left column, f*_2 of the right one
+  // tf32: C of the last two tile rows (slot t & 1), the source of the copy regrouped along y
+  __shared__ __align__(8) float s_c[SPLIT == 2 ? 2 : 1][SPLIT == 2 ? TY : 1][TX];
   if (early) pdl_trigger();
-  march2_tma<MRT, SPLIT>(sp, &map_f, &map_F, f_out, C_out, flag, so, ychunk, blockIdx.x, blockIdx.y, cs_raw2, mpart,
-                         block_linear());
+  const bool wT = SPLIT == 2 && so.thi[0] != nullptr;
+  uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(cs_raw2) + 127) & ~uintptr_t(127));
+  const int ks = sp.ksum;
+  const int nst = tma2_nst(ks);
+  const uint32_t stg = tma2_stage(ks);
+  const uint32_t tx = TMA2_F_BYTES + tma2_ff_bytes(ks);
+  uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)nst * stg);
+  const int n0 = sp.n[0], n1 = sp.n[1];
+  const long long nodes = sp.nodes;
+  const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
+  const int x0 = blockIdx.x * TX;
+  const int tr0 = blockIdx.y * ychunk;
+  const int tr1 = min(tr0 + ychunk, (n1 + TY - 1) / TY);
+  const bool owner = warp < TX * TY / 64;
+  const int xp = 2 * (lane & 15), row = 2 * warp + (lane >> 4);  // owner's place in the tile
+  const int gx = x0 + xp;
+  // place in the staged window: owners and row ring pairs (x aligned to 8 bytes), column ring nodes
+  int lx = xp + 4, ly = row + 1;
+  if (warp == T3_WARPS - 2) ly = lane < 16 ? 0 : TY + 1;
+  if (warp == T3_WARPS - 1) {
+    lx = lane < 16 ? 3 : TX + 4;
+    ly = (lane & 15) + 1;
+  }
+  const float* win = reinterpret_cast<const float*>(ring) + ly * TW + lx;
+  auto stage_of = [&](int t) { return (t - tr0) % nst; };
+  auto parity_of = [&](int t) { return static_cast<uint32_t>(((t - tr0) / nst) & 1); };
+  auto issue = [&](int t) {
+    const int s = stage_of(t);
+    uint8_t* st = ring + (size_t)s * stg;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(cs_smem_u32(&full[s])), "r"(tx)
+                 : "memory");
+    cs_tma_3d(st, &map_f, x0 - 4, t * TY - 1, 0, &full[s]);
+    cs_tma_3d(st + TMA2_FF_OFF, &map_F, x0 - 4, t * TY - 1, 0, &full[s]);
+  };
+  // tf32: tile row t to the y copy (element (x, y) at thi[0][(y/4 tpx + x) 4 + y%4]): warp w < 4
+  // writes y group 4t + w for the tile's 32 x (512 contiguous bytes)
+  auto flush_y = [&](int t) {
+    const int yq = 4 * warp;
+    if (warp < TY / 4 && x0 + lane < n0 && t * TY + yq < n1) {
+      const float* r = &s_c[t & 1][SPLIT == 2 ? yq : 0][lane];
+      const long long o = ((long long)((t * TY + yq) >> 2) * so.tpx + x0 + lane) * 4;
+      *reinterpret_cast<float4*>(so.thi[0] + o) = make_float4(r[0], r[TX], r[2 * TX], r[3 * TX]);
+    }
+  };
+  if (tid == 0) {
+    for (int s = 0; s < nst; ++s)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cs_smem_u32(&full[s])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // f and F come from the previous kernels
+  if (tid == 0)
+    for (int t = tr0; t < tr1 && t < tr0 + nst; ++t) issue(t);
+  SumAcc<float> macc;
+  float bad = 0.f;
+  int b = 0;
+  for (int tr = tr0; tr < tr1; ++tr, b ^= 1) {
+    cs_mbar_wait(&full[stage_of(tr)], parity_of(tr), flag);
+    const float* st = win + stage_of(tr) * (stg / 4);
+    const float* sF = st + TMA2_FF_OFF / 4;  // partial k of axis mu at plane k * D + mu, added in order of k
+    float fs[2][Q];
+    if (warp < T3_WARPS - 1) {
+      float fv[2][Q], Fv[2][D];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const float2 t = *reinterpret_cast<const float2*>(st + q * (TH * TW));
+        fv[0][q] = t.x;
+        fv[1][q] = t.y;
+      }
+#pragma unroll
+      for (int mu = 0; mu < D; ++mu) {
+        float2 t = *reinterpret_cast<const float2*>(sF + mu * (TH * TW));
+        for (int k = 1; k < ks; ++k) {
+          const float2 u = *reinterpret_cast<const float2*>(sF + (k * D + mu) * (TH * TW));
+          t.x += u.x;
+          t.y += u.y;
+        }
+        Fv[0][mu] = t.x;
+        Fv[1][mu] = t.y;
+      }
+      collide_node<float, D, MRT>(sp, fv[0], Fv[0], fs[0]);
+      collide_node<float, D, MRT>(sp, fv[1], Fv[1], fs[1]);
+      if (owner || lane < 16)  // moves +y: the tile's rows, and the row below into the tile
+        *reinterpret_cast<float2*>(&s_up[b][owner ? row + 1 : 0][xp]) = make_float2(fs[0][3], fs[1][3]);
+      if (owner || lane >= 16)  // moves -y: the tile's rows, and the row above into the tile
+        *reinterpret_cast<float2*>(&s_dn[b][owner ? row : TY][xp]) = make_float2(fs[0][4], fs[1][4]);
+    } else {
+      float fv[Q], Fv[D], h[Q];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) fv[q] = st[q * (TH * TW)];
+#pragma unroll
+      for (int mu = 0; mu < D; ++mu) {
+        Fv[mu] = sF[mu * (TH * TW)];
+        for (int k = 1; k < ks; ++k) Fv[mu] += sF[(k * D + mu) * (TH * TW)];
+      }
+      collide_node<float, D, MRT>(sp, fv, Fv, h);
+      s_x[b][lane >> 4][lane & 15] = lane < 16 ? h[1] : h[2];  // moves +x, -x into the tile
+    }
+    __syncthreads();
+    // tile row tr is read by everyone: its stage takes tile row tr + nst
+    if (tid == 0 && tr + nst < tr1) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      issue(tr + nst);
+    }
+    if (SPLIT == 2 && wT && tr > tr0) flush_y(tr - 1);  // its slot is rewritten only after the next barrier
+    if (owner) {
+      const int gy = tr * TY + row;
+      const float up = __shfl_up_sync(0xffffffffu, fs[1][1], 1), dn = __shfl_down_sync(0xffffffffu, fs[0][2], 1);
+      const float2 y3 = *reinterpret_cast<const float2*>(&s_up[b][row][xp]);
+      const float2 y4 = *reinterpret_cast<const float2*>(&s_dn[b][row + 1][xp]);
+      float o[2][Q], C[2] = {0.f, 0.f};
+      o[0][0] = fs[0][0];
+      o[1][0] = fs[1][0];
+      o[0][1] = xp == 0 ? s_x[b][0][row] : up;
+      o[1][1] = fs[0][1];
+      o[0][2] = fs[1][2];
+      o[1][2] = xp == TX - 2 ? s_x[b][1][row] : dn;
+      o[0][3] = y3.x;
+      o[1][3] = y3.y;
+      o[0][4] = y4.x;
+      o[1][4] = y4.y;
+      if (x0 > 0 && x0 + TX < n0 && tr * TY > 0 && tr * TY + TY < n1) {  // no wall within reach (block-uniform)
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+#pragma unroll
+          for (int q = 0; q < Q; ++q) C[v] += o[v][q];
+      } else {
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          const bool known[Q] = {true, gx + v > 0, gx + v + 1 < n0, gy > 0, gy + 1 < n1};
+          int n_unknown = 0;
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            if (known[q]) {
+              C[v] += o[v][q];
+            } else {
+              o[v][q] = 0.f;
+              ++n_unknown;
+            }
+          }
+          if (n_unknown > 0) {
+            // Eq. (Dirichlet_BC); with k unknown populations each takes 1/k of the deficit
+            const float fill = (sp.C_wall - C[v]) / static_cast<float>(n_unknown);
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+              if (!known[q]) o[v][q] = fill;
+            C[v] = o[v][0];
+#pragma unroll
+            for (int q = 1; q < Q; ++q) C[v] += o[v][q];
+          }
+        }
+      }
+      if (gx < n0 && gy < n1) {  // (n0 is a multiple of 4)
+        const long long node = gx + (long long)n0 * gy;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) *reinterpret_cast<float2*>(f_out + q * nodes + node) = make_float2(o[0][q], o[1][q]);
+        if (SPLIT == 0 || C_out) *reinterpret_cast<float2*>(C_out + node) = make_float2(C[0], C[1]);
+        if constexpr (SPLIT != 0) write_split_v<SPLIT, 2>(so, (long long)gy * so.ldp + gx, C);
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          bad = __fmaf_rn(C[v], 0.f, bad);  // NaN once a C is not finite
+          macc.add(C[v]);
+        }
+      } else {
+        C[0] = C[1] = 0.f;  // zero outside the domain
+      }
+      if (SPLIT == 2 && wT)
+        *reinterpret_cast<float2*>(&s_c[tr & 1][SPLIT == 2 ? row : 0][xp]) = make_float2(C[0], C[1]);
+    }
+  }
+  if (SPLIT == 2 && wT) {
+    __syncthreads();
+    flush_y(tr1 - 1);
+  }
+  // every issued tile row was waited for by every warp; after a timeout no copy may still be
+  // landing in this block's shared memory
+  if (tid == 0)
+    for (int t = (tr1 - nst > tr0 ? tr1 - nst : tr0); t < tr1; ++t)
+      cs_mbar_wait(&full[stage_of(t)], parity_of(t), flag);
+  if (__any_sync(0xffffffffu, bad != 0.f) && lane == 0) atomicOr(flag, 1);
+  block_mass<T3_WARPS>(macc, mpart, block_linear());
   if (!early) pdl_trigger();
 }
 
@@ -1650,7 +1812,7 @@ lbm_fused2_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ T
     const CUtensorMap* mf = par ? &mf1 : &mf0;
     float* fo = par ? f0 : f1;
     for (int it = blockIdx.x; it < cs_items; it += G) {
-      march2_tma<MRT, 1>(sp, mf, &mF, fo, C, flag, so, ychunk, it % bxn, it / bxn, smem, mpart, it);
+      march2_tma<MRT>(sp, mf, &mF, fo, C, flag, so, ychunk, it % bxn, it / bxn, smem, mpart, it);
       __syncthreads();
     }
     target += G;
@@ -2040,6 +2202,8 @@ cudaError_t launch_cs(const lbm_s* h, const void* f_in, void* f_out, void* C_out
       const CUtensorMap& mf = slot ? *static_cast<const CUtensorMap*>(slot->map_f) : pl->f[f_in == h->dev.f[0] ? 0 : 1];
       const CUtensorMap& mF = slot ? *static_cast<const CUtensorMap*>(slot->map_F) : pl->F;
       cfg.dynamicSmemBytes = tma2_smem(h->sp.ksum);
+      cfg.blockDim = dim3(32, T3_WARPS);
+      h->cs_nparts = T3_WARPS * static_cast<int>(cfg.gridDim.x * cfg.gridDim.y);
       if (split == 0) return launch_tma2<MRT, 0>(cfg, sp, mf, mF, fo, Co, flag, so, ychunk, early, mp);
       if (split == 1) return launch_tma2<MRT, 1>(cfg, sp, mf, mF, fo, Co, flag, so, ychunk, early, mp);
       if (split == 3) return launch_tma2<MRT, 3>(cfg, sp, mf, mF, fo, Co, flag, so, ychunk, early, mp);
