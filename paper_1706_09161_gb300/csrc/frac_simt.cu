@@ -517,10 +517,11 @@ bool simt_one_wave(const lbm_s* h) {
   });
 }
 
-// The split doubles while 64 x 64 tiles leave SMs without two blocks, or while every slice
-// keeps 256 contraction steps and the tiles leave fewer than eight blocks per SM (measured:
-// 512^2 with 1/2/4/8 slices 32.8 / 27.5 / 22.9 / 26.3 us per step, 1024^2 124 / 118 / 106 /
-// 118, 96^3 with 1/2 45.4 / 53.7).
+// The split doubles while 64 x 64 tiles leave SMs without a block, or, up to four slices, while
+// every slice keeps 80 contraction steps and the tiles leave fewer than eight blocks per SM
+// (measured, us per step with 1/2/4/8 slices: 256^2 16.3 / 11.9 / 9.8 / 9.7, 384^2 22.1 / 16.7 /
+// 14.7 / 16.0, 512^2 32.4 / 26.4 / 22.8 / 26.1, 700 x 600 52 / 48 / 40 / 48, 1024^2 123 / 117 / 105 /
+// 117; 3-D with 1/2: 48^3 15.7 / 17.5, 64^3 15.8 / 18.6, 72^3 28.7 / 39.2).
 int simt_ksplit(const lbm_s* h) {
   if (h->elem != 4) return 1;
   const long long tiles = count_tiles(h, 64, 64), sms = device_sms();
@@ -529,7 +530,7 @@ int simt_ksplit(const lbm_s* h) {
   const int kbmin = (kmin + kSlice - 1) / kSlice;
   int ks = 1;
   while (ks * 2 <= 8 && ks * 2 <= kbmin &&
-         (tiles * ks < 2 * sms || (tiles * ks < 8 * sms && kmin >= 256 * 2 * ks))) ks *= 2;
+         (tiles * ks < sms - sms / 10 || (ks < 4 && tiles * ks < 8 * sms && kmin >= 160 * ks))) ks *= 2;
   return ks;
 }
 
