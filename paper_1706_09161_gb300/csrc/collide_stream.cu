@@ -1998,10 +1998,14 @@ cudaError_t launch_tma2(const cudaLaunchConfig_t& cfg, const KConst<float>& sp, 
 bool one_wave(const dim3& g) { return (long long)g.x * g.y * g.z <= 2LL * device_sms(); }
 
 // Let the next kernel (the operator) be scheduled at block start: only where this grid runs in
-// one wave and the operator takes one block per SM (the tensor-core forms).  The SIMT operator's
-// small blocks, launched early, pile up on the SMs that this grid leaves first (measured: 512^2
-// FP32 step 32.8 us with the early trigger, 22.9 without).
-int early_trigger(const lbm_s* h, const dim3& g) { return h->tc && one_wave(g) ? 1 : 0; }
+// one wave and the operator takes one block per SM (the tensor-core forms), or where both grids
+// together are small (64^2 FP32 step 6.56 us without, 6.22 with the early trigger, 100^2 7.51 and
+// 7.34).  The SIMT operator's small blocks, launched early beside a larger grid, pile up on the SMs
+// that it leaves first (512^2 FP32 32.8 us with the early trigger, 22.9 without).
+int early_trigger(const lbm_s* h, const dim3& g) {
+  if (h->tc) return one_wave(g) ? 1 : 0;
+  return one_wave(dim3(g.x * g.y * g.z + (unsigned)std::min(simt_blocks(h), 1LL << 30), 1, 1)) ? 1 : 0;
+}
 
 // 2-D FP32 lattices with coefficients per node: rows of a warp's strip in units of kStripRows, or 0
 // for the plain march.  That one collides each node once and is the faster form where its blocks

@@ -517,6 +517,11 @@ bool simt_one_wave(const lbm_s* h) {
   });
 }
 
+long long simt_blocks(const lbm_s* h) {
+  if (h->elem == 8) return count_tiles(h, tile64(h), tile64(h));
+  return with_tile32(h, h->simt_ks, [&](auto, auto G) { return count_tiles(h, G.BM, G.BN) * h->simt_ks; });
+}
+
 // The split doubles while 64 x 64 tiles leave SMs without a block, or, up to four slices, while
 // every slice keeps 80 contraction steps and the tiles leave fewer than eight blocks per SM
 // (measured, us per step with 1/2/4/8 slices: 256^2 16.3 / 11.9 / 9.8 / 9.7, 384^2 22.1 / 16.7 /

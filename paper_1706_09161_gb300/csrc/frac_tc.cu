@@ -889,9 +889,11 @@ int tc_prepare(lbm_s* h, const std::vector<std::vector<double>>& K, int force_bn
   };
   int ks = split(tc_count_tiles(h, bn));
   // 64-column tiles where they put more CTAs to work (small and ragged grids; measured:
-  // 256^2 bf16x6 step 8.7 us with 128 columns, 8.1 with 64, 301 x 203 10.6 and 9.9)
+  // 256^2 bf16x6 step 8.7 us with 128 columns, 8.1 with 64, 301 x 203 10.6 and 9.9), and where no
+  // line is longer than 64 columns (50^2 tf32x3 12.4 and 10.8, 48^2 6.9 and 6.5)
   const long long t64 = tc_count_tiles(h, 64);
-  if (bn == 128 && t64 * split(t64) <= kSMs && t64 * split(t64) > tc_count_tiles(h, 128) * ks) {
+  const long long t128 = tc_count_tiles(h, 128);
+  if (bn == 128 && t64 * split(t64) <= kSMs && (t64 == t128 || t64 * split(t64) > t128 * ks)) {
     bn = 64;
     ks = split(t64);
   }

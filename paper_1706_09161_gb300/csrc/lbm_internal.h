@@ -168,6 +168,7 @@ cudaError_t launch_frac_simt(const lbm_s* h, const void* C, void* F, cudaStream_
 int simt_ksplit(const lbm_s* h);
 // the FP32 SIMT operator's grid is resident at once (programmatic dependent launch)
 bool simt_one_wave(const lbm_s* h);
+long long simt_blocks(const lbm_s* h);  // blocks of the SIMT operator's launch
 // tensor-core split-precision fractional operator (tcgen05); returns
 // cudaErrorNotSupported when the handle's shape is not covered
 cudaError_t launch_frac_tc(const lbm_s* h, cudaStream_t s);
