@@ -935,7 +935,7 @@ int simt_replan(lbm_s* h, int ks) {
   if (!(ks == 1 || ks == 2 || ks == 4 || ks == 8)) return LBM_EINVAL;
   int kbmin = 1 << 30;
   for (int mu = 0; mu < h->d; ++mu) kbmin = std::min(kbmin, (h->sp.n[mu] + 31) / 32);
-  if (ks > kbmin) return LBM_EINVAL;
+  if (ks > kbmin && ks != lbm::simt_ksplit(h)) return LBM_EINVAL;
   h->simt_ks = ks;
   return LBM_OK;
 }
@@ -1025,7 +1025,10 @@ int lbm_configure(lbm_t h, int bn, int ks, int persist, int chunk, int fused) {
       c.persist = persist ? 1 : 0;
     }
   } else if (!h->is_batch() && h->elem == 4 && bn == 0 && !persist && !fused) {
-    c.ks = ks > 0 ? ks : h->simt_ks;  // FP32 SIMT operator: its contraction split only
+    // FP32 SIMT operator: its contraction split only; a split that is asked for leaves no slice empty
+    for (int mu = 0; ks > 0 && mu < h->d; ++mu)
+      if (ks > (h->sp.n[mu] + 31) / 32) return LBM_EINVAL;
+    c.ks = ks > 0 ? ks : h->simt_ks;
   } else if (bn > 0 || ks > 0 || persist || fused) {
     return LBM_EINVAL;  // no tensor-core operator to plan
   }
@@ -1062,7 +1065,7 @@ int lbm_autotune(lbm_t h, int nsteps, char* desc, int desc_len) {
     for (int ks : {1, 2, 4, 8}) {
       int kbmin = 1 << 30;
       for (int mu = 0; mu < h->d; ++mu) kbmin = std::min(kbmin, (h->sp.n[mu] + 31) / 32);
-      if (ks <= kbmin) ops.push_back({0, ks, 0, cur.chunk});
+      if (ks <= kbmin || ks == cur.ks) ops.push_back({0, ks, 0, cur.chunk});
     }
   if (!h->is_batch() && h->tc) {
     const int sms = lbm::device_sms();

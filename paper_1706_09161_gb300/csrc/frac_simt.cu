@@ -526,15 +526,20 @@ long long simt_blocks(const lbm_s* h) {
 // every slice keeps 80 contraction steps and the tiles leave fewer than eight blocks per SM
 // (measured, us per step with 1/2/4/8 slices: 256^2 16.3 / 11.9 / 9.8 / 9.7, 384^2 22.1 / 16.7 /
 // 14.7 / 16.0, 512^2 32.4 / 26.4 / 22.8 / 26.1, 700 x 600 52 / 48 / 40 / 48, 1024^2 123 / 117 / 105 /
-// 117; 3-D with 1/2: 48^3 15.7 / 17.5, 64^3 15.8 / 18.6, 72^3 28.7 / 39.2).
+// 117; 3-D with 1/2: 48^3 15.7 / 17.5, 64^3 15.8 / 18.6, 72^3 28.7 / 39.2).  The longer axis sets
+// the most slices in 2-D (by the shorter one: 1000 x 60 29.3 us against 14.5, 53 x 1001 35.8 and 15.2).
 int simt_ksplit(const lbm_s* h) {
   if (h->elem != 4) return 1;
   const long long tiles = count_tiles(h, 64, 64), sms = device_sms();
-  int kmin = 1 << 30;
-  for (int mu = 0; mu < h->d; ++mu) kmin = std::min(kmin, h->sp.n[mu]);
-  const int kbmin = (kmin + kSlice - 1) / kSlice;
+  int kmin = 1 << 30, kmax = 0;
+  for (int mu = 0; mu < h->d; ++mu) {
+    kmin = std::min(kmin, h->sp.n[mu]);
+    kmax = std::max(kmax, h->sp.n[mu]);
+  }
+  // 2-D: as many slices as the longer axis has, the shorter one's last slices then being empty
+  const int kbs = ((h->d == 2 ? kmax : kmin) + kSlice - 1) / kSlice;
   int ks = 1;
-  while (ks * 2 <= 8 && ks * 2 <= kbmin &&
+  while (ks * 2 <= 8 && ks * 2 <= kbs &&
          (tiles * ks < sms - sms / 10 || (ks < 4 && tiles * ks < 8 * sms && kmin >= 160 * ks))) ks *= 2;
   return ks;
 }

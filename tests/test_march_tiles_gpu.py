@@ -160,3 +160,15 @@ def test_fields_with_a_split_contraction(L, kind):
         a.step(4)
         b.step(4)
         assert np.array_equal(a.f(), b.f())
+
+
+# elongated grids: more contraction slices than the short axis has blocks of 32 (some are empty)
+@pytest.mark.parametrize("grid", [(400, 33), (35, 300), (257, 3)])
+def test_fp32_split_of_elongated_grids(L, grid):
+    pb, C0 = _case(grid, 1009 + sum(grid))
+    with L.Lattice(pb, C0, "fp32") as lat:
+        F = O.fractional_terms(O.Operators(pb), torch.tensor(lat.C()))
+        for mu, N in enumerate(grid):
+            ref = F[mu].numpy()
+            assert np.all(np.abs(lat.F(mu) - ref) <= (N + 2) * 2.0 ** -24 * np.abs(ref) + 1e-38), mu
+        lat.configure(0, 0, 0, 0, 0)  # the built-in split is accepted again
