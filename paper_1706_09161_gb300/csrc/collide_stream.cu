@@ -959,7 +959,7 @@ StripGrid strip_grid(const int* n, int chunk) {
   StripGrid g;
   g.v = n[0] % 2 == 0 ? 2 : 1;
   g.strips = (n[0] + 32 * g.v - 1) / (32 * g.v);
-  g.rows = std::min(kStripRows * chunk, n[1]);
+  g.rows = std::min(kStripRows * std::min(chunk, n[1]), n[1]);  // (chunk may be any positive int)
   g.items = g.strips * ((n[1] + g.rows - 1) / g.rows);
   return g;
 }
