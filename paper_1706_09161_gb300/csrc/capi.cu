@@ -33,7 +33,9 @@ cudaError_t dev_alloc(const lbm_s* h, void** p, size_t bytes) {
     *p = h->mem.alloc(bytes, h->stream, h->mem.ctx);
     return *p ? cudaSuccess : cudaErrorMemoryAllocation;
   }
-  return cudaMalloc(p, bytes);
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();  // the next launch's check is not to find it
+  return e;
 }
 
 void dev_free(const lbm_s* h, void* p) {
@@ -940,38 +942,44 @@ int simt_replan(lbm_s* h, int ks) {
   return LBM_OK;
 }
 
-// the handle's launch configuration set to c (operator plan for tensor-core handles, the
-// contraction split of the FP32 SIMT operator, collide-stream chunk for every handle);
-// captured graphs are dropped
-int apply_cfg(lbm_s* h, const TuneCfg& c) {
+// the parts of apply_cfg; an error may leave some of them set
+int set_cfg(lbm_s* h, const TuneCfg& c) {
   int rc = LBM_OK;
-  if (h->is_batch()) {
-    h->cs_chunk = c.chunk;
-    rc = lbm::cs_batch_prepare(h);
-  } else {
-    if (h->tc) {
-      h->fused = false;
-      if ((rc = lbm::tc_replan(h, c.bn, c.ks, c.persist))) return rc;
-      lbm::cs_release(h);
-      h->cs_chunk = c.chunk;
-      if ((rc = lbm::cs_prepare(h))) return rc;
-      h->pdl = pdl_fits(h);
-      lbm::tc_set_pdl(h, h->pdl);
-      if (c.fused) {
-        if (h->fld.on) return LBM_EINVAL;  // the fused step runs the constant-coefficient march only
-        if ((rc = lbm::fused_prepare(h))) return rc;
-        h->fused = true;
-      }
-      // every operand copy of C current: the new plan may take the regrouped tf32 copies
-      // from the collide-stream kernel, which the old one did not write
-      LBM_CUDA(lbm::launch_split_C(h, h->stream));
-    } else {
-      h->cs_chunk = c.chunk;
-      if (c.ks > 0 && h->elem == 4 && (rc = simt_replan(h, c.ks))) return rc;
-      h->pdl = pdl_fits(h);
+  h->cs_chunk = c.chunk;
+  if (h->is_batch()) return lbm::cs_batch_prepare(h);
+  if (h->tc) {
+    h->fused = false;
+    if ((rc = lbm::tc_replan(h, c.bn, c.ks, c.persist))) return rc;
+    lbm::cs_release(h);
+    if ((rc = lbm::cs_prepare(h))) return rc;
+    h->pdl = pdl_fits(h);
+    lbm::tc_set_pdl(h, h->pdl);
+    if (c.fused) {
+      if (h->fld.on) return LBM_EINVAL;  // the fused step runs the constant-coefficient march only
+      if ((rc = lbm::fused_prepare(h))) return rc;
+      h->fused = true;
     }
+    // every operand copy of C current: the new plan may take the regrouped tf32 copies
+    // from the collide-stream kernel, which the old one did not write
+    LBM_CUDA(lbm::launch_split_C(h, h->stream));
+  } else {
+    if (c.ks > 0 && h->elem == 4 && (rc = simt_replan(h, c.ks))) return rc;
+    h->pdl = pdl_fits(h);
   }
+  return LBM_OK;
+}
+
+// the handle's launch configuration set to c (operator plan for tensor-core handles, the
+// contraction split of the FP32 SIMT operator, collide-stream chunk for every handle); captured
+// graphs are dropped.  After an error the configuration is the one before the call (its buffers
+// are there: F only grows).
+int apply_cfg(lbm_s* h, const TuneCfg& c) {
+  TuneCfg old{0, h->simt_ks, 0, h->cs_chunk, h->fused ? 1 : 0};
+  if (!h->is_batch() && h->tc) lbm::tc_config(h, &old.bn, &old.ks, &old.persist);
+  const int rc = set_cfg(h, c);
   drop_graphs(h);
+  if (rc && h->is_batch()) h->cs_chunk = old.chunk;  // (its tables are still the old ones)
+  else if (rc) set_cfg(h, old);
   return rc;
 }
 
@@ -1262,7 +1270,7 @@ static int rebuild_fields(lbm_s* h) {
   if (h->tc) {  // where the partial sums of a split contraction are added depends on the march
     int bn, ks, persist;
     lbm::tc_config(h, &bn, &ks, &persist);
-    if ((rc = lbm::tc_replan(h, bn, ks, persist))) return rc;
+    if ((rc = lbm::tc_replan(h, bn, ks, persist, false))) return rc;
     lbm::cs_release(h);
     if ((rc = lbm::cs_prepare(h))) return rc;
   }

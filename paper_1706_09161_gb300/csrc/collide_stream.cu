@@ -2415,6 +2415,7 @@ int cs_batch_prepare(lbm_s* b) {
   const int P = static_cast<int>(b->subs.size());
   std::vector<BatchCS> tab(P);
   std::vector<int2> map;
+  std::vector<int> nparts(P);
   int total = 0;
   for (int i = 0; i < P; ++i) {
     lbm_s* h = b->subs[i];
@@ -2431,28 +2432,35 @@ int cs_batch_prepare(lbm_s* b) {
     e.mpart = h->cs_part;
     e.bx = (h->sp.n[0] + TX - 1) / TX;
     int blocks = e.bx * ((h->sp.n[1] + TY - 1) / TY);  // 3-D: one column each, the whole z extent
-    h->cs_nparts = kMassSlots * blocks;
+    nparts[i] = kMassSlots * blocks;
     if (h->d == 2) {
       const StripGrid g = strip_grid(h->sp.n, b->cs_chunk > 0 ? b->cs_chunk : kBatchChunk);
       e.v = g.v;
       e.strips = g.strips;
       e.rows = g.rows;
-      e.items = h->cs_nparts = g.items;
+      e.items = nparts[i] = g.items;
       blocks = (g.items + kStripWarps - 1) / kStripWarps;
     }
     for (int k = 0; k < blocks; ++k) map.push_back(make_int2(i, k));
     total += blocks;
   }
-  dev_free(b, b->batch_cs);
-  dev_free(b, b->batch_cs_start);
-  b->batch_cs = nullptr;
-  b->batch_cs_start = nullptr;
-  if (dev_alloc(b, &b->batch_cs, sizeof(BatchCS) * P) != cudaSuccess) return LBM_ENOMEM;
-  if (dev_alloc(b, (void**)&b->batch_cs_start, sizeof(int2) * total) != cudaSuccess) return LBM_ENOMEM;
-  if (cudaMemcpy(b->batch_cs, tab.data(), sizeof(BatchCS) * P, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(b->batch_cs_start, map.data(), sizeof(int2) * total, cudaMemcpyHostToDevice) != cudaSuccess)
-    return LBM_ECUDA;
+  // the tables in force stay until the new ones are whole
+  void* d_tab = nullptr;
+  void* d_map = nullptr;
+  int rc = LBM_OK;
+  if (dev_alloc(b, &d_tab, sizeof(BatchCS) * P) != cudaSuccess || dev_alloc(b, &d_map, sizeof(int2) * total) != cudaSuccess)
+    rc = LBM_ENOMEM;
+  else if (cudaMemcpy(d_tab, tab.data(), sizeof(BatchCS) * P, cudaMemcpyHostToDevice) != cudaSuccess ||
+           cudaMemcpy(d_map, map.data(), sizeof(int2) * total, cudaMemcpyHostToDevice) != cudaSuccess ||
+           cudaStreamSynchronize(b->stream) != cudaSuccess)  // no launch in flight reads the old ones
+    rc = LBM_ECUDA;
+  dev_free(b, rc ? d_tab : b->batch_cs);
+  dev_free(b, rc ? d_map : static_cast<void*>(b->batch_cs_start));
+  if (rc) return rc;
+  b->batch_cs = d_tab;
+  b->batch_cs_start = static_cast<int*>(d_map);
   b->batch_cs_blocks = total;
+  for (int i = 0; i < P; ++i) b->subs[i]->cs_nparts = nparts[i];
   return LBM_OK;
 }
 

@@ -948,10 +948,13 @@ static bool encode_F(const lbm_s* h, float* F, int slots, int rows, TcMaps* maps
 }
 
 // (Re)plan the operator: column tile width bn, contraction split ks, persistent or per
-// tile; re-encodes every tensor map.
-int tc_replan(lbm_s* h, int bn, int ks, int persist) {
-  TcPlan* p = h->tc;
-  if (!p) return LBM_EINVAL;
+// tile; re-encodes every tensor map.  The plan in force, F and the maps of it stay as they are
+// until the new plan is whole: an error leaves the handle on the old one.  With `must_grow` false a
+// larger F that is refused is no error: the partial sums then need no slots of it.
+int tc_replan(lbm_s* h, int bn, int ks, int persist, bool must_grow) {
+  if (!h->tc) return LBM_EINVAL;
+  TcPlan next = *h->tc;
+  TcPlan* const p = &next;
   if (!(bn == 64 || bn == 128 || bn == 256) || !(ks == 1 || ks == 2 || ks == 4 || ks == 8)) return LBM_EINVAL;
   if ((persist && ((bn != PBN && bn != 256) || ks != 1)) || (bn == 256 && ks != 1) || ks > tc_kbmin(h))
     return LBM_EINVAL;
@@ -973,7 +976,6 @@ int tc_replan(lbm_s* h, int bn, int ks, int persist) {
   P.n2 = n[2];
   P.naxes = h->d;
   P.nodes = h->sp.nodes;
-  P.F = static_cast<float*>(h->dev.F);
   P.flag = h->dev.flag;
   const cuuint64_t cdims[3] = {(cuuint64_t)n[0], (cuuint64_t)n[1], (cuuint64_t)n[2]};
   const cuuint64_t cstr[2] = {(cuuint64_t)ldp * E, (cuuint64_t)ldp * n[1] * E};
@@ -1035,25 +1037,33 @@ int tc_replan(lbm_s* h, int bn, int ks, int persist) {
         !encode(&p->maps.k_l2[mu], E, 2, static_cast<uint8_t*>(h->dev.Kl2) + koff[mu] * E, kdims, kstr, kbox))
       return LBM_ECUDA;
   }
-  P.F = static_cast<float*>(h->dev.F);
   // partial tiles in slots of F only where the TMA-fed 2-D march reads them (the march of varying
   // coefficients reads F with plain loads); row chunks of an output tile: what one CTA of a cluster
   // stores, at most 32 rows
   P.slots = ks > 1 && h->d == 2 && P.tma_store && !h->fld.on ? 1 : 0;
-  const size_t need = (size_t)(P.slots ? ks : 1) * h->d * h->sp.nodes;
-  if (need > h->f_elems) {
-    cudaStreamSynchronize(h->stream);
-    dev_free(h, h->dev.F);
-    h->dev.F = nullptr;
-    h->f_elems = 0;
-    if (dev_alloc(h, (void**)&h->dev.F, need * 4) != cudaSuccess) return LBM_ENOMEM;
-    h->f_elems = need;
-    P.F = static_cast<float*>(h->dev.F);
-  }
-  h->sp.ksum = P.slots ? ks : 1;
-  if (P.tma_store && !encode_F(h, P.F, h->sp.ksum, P.slots ? 32 : std::min(32, bn / ks), &p->maps)) return LBM_ECUDA;
   P.total_tiles = tiles;
   P.early_trigger = (tiles * ks <= kSMs) ? 1 : 0;
+  const size_t need = (size_t)ks * h->d * h->sp.nodes;
+  void* F = h->dev.F;
+  if (P.slots && need > h->f_elems && dev_alloc(h, &F, need * 4) != cudaSuccess) {
+    if (must_grow) return LBM_ENOMEM;
+    P.slots = 0;  // the CTAs of a tile add them
+    F = h->dev.F;
+  }
+  const int ksum = P.slots ? ks : 1;
+  P.F = static_cast<float*>(F);
+  bool ok = !P.tma_store || encode_F(h, P.F, ksum, P.slots ? 32 : std::min(32, bn / ks), &p->maps);
+  if (F != h->dev.F) {
+    ok = ok && cudaStreamSynchronize(h->stream) == cudaSuccess;  // no launch in flight uses the old F
+    dev_free(h, ok ? h->dev.F : F);
+    if (ok) {
+      h->dev.F = F;
+      h->f_elems = need;
+    }
+  }
+  if (!ok) return LBM_ECUDA;
+  h->sp.ksum = ksum;
+  *h->tc = next;
   return LBM_OK;
 }
 
@@ -1230,7 +1240,7 @@ int tc_set_gfield(lbm_s* h, bool on) {
       }
     p->gvar = true;
   }
-  return tc_replan(h, p->bn, p->prm.ksplit, p->persist ? 1 : 0);  // re-encodes the operand maps
+  return tc_replan(h, p->bn, p->prm.ksplit, p->persist ? 1 : 0, false);  // re-encodes the operand maps
 }
 
 cudaError_t launch_split_C(const lbm_s* h, cudaStream_t s) {

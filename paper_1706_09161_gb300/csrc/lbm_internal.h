@@ -234,8 +234,9 @@ int reduce_blocks_for(long long n);
 int tc_prepare(lbm_s* h, const std::vector<std::vector<double>>& K, int force_bn, int force_ks);
 // operator plan: column tile width bn (64, 128, 256), contraction split ks (1, 2, 4, 8),
 // persistent kernel or one CTA per tile; re-encodes the tensor maps (LBM_EINVAL for a
-// combination the kernels do not cover).  Captured graphs must be dropped afterwards.
-int tc_replan(lbm_s* h, int bn, int ks, int persist);
+// combination the kernels do not cover; the plan before stays after an error).  Captured graphs
+// must be dropped afterwards.
+int tc_replan(lbm_s* h, int bn, int ks, int persist, bool must_grow = true);
 long long tc_count_tiles(const lbm_s* h, int bn);  // output tiles of bn columns, all axes
 int tc_kbmin(const lbm_s* h);                      // fewest contraction blocks of any axis
 void tc_config(const lbm_s* h, int* bn, int* ks, int* persist);

@@ -1,6 +1,8 @@
 """Launch configurations that a caller sets: which values are taken, what they mean after the
 kind of march changes, and what a refused one leaves behind.  A configuration changes the schedule
 of a step, never its result: populations are equal bit for bit."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -20,7 +22,9 @@ def L():
 
 def _case(grid, seed, collision="mrt"):
     rng = np.random.default_rng(seed)
-    return W.random_problem(rng, len(grid), collision, grid, spherical=collision == "bgk"), W.random_field(rng, grid)
+    pb = W.random_problem(rng, len(grid), collision, grid, spherical=collision == "bgk")
+    pb = dataclasses.replace(pb, alpha=tuple(1.5 + 0.5 * (a - 1.2) / 0.8 for a in pb.alpha))  # stable over the runs here
+    return pb, W.random_field(rng, grid)
 
 
 # rows per warp are two per unit of the chunk: values whose double does not fit in 32 bits
@@ -49,3 +53,78 @@ def test_any_positive_chunk_is_taken(L, kind, chunk):
             lat.reset()
             lat.step(5)
             assert np.array_equal(lat.f(), ref), bool(f)
+
+
+class Hooks:
+    """Device memory from PyTorch's allocator, refused while `refuse` is set."""
+
+    def __init__(self, L):
+        self.L, self.refuse = L, False
+
+    def __enter__(self):
+        def alloc(nbytes, stream, ctx):
+            if self.refuse:
+                return None
+            return torch.cuda.caching_allocator_alloc(int(nbytes), torch.cuda.current_device(), int(stream or 0))
+
+        self.L.lbm_set_allocator(alloc, lambda ptr, ctx: torch.cuda.caching_allocator_delete(int(ptr)))
+        return self
+
+    def __exit__(self, *exc):
+        self.L.lbm_set_allocator(None, None)
+
+
+# a plan whose larger F is refused, or whose fused form is not there after F has grown: the handle
+# goes on with the plan, the buffers and the captured graph that it had
+@pytest.mark.parametrize("fused", [0, 1])
+@pytest.mark.parametrize("kind", ["bf16split", "tf32split"])
+def test_a_refused_plan_leaves_the_old_one(L, kind, fused):
+    pb, C0 = _case((520, 520), 1409)
+    with Hooks(L) as mem, L.Lattice(pb, C0, kind) as a, L.Lattice(pb, C0, kind) as b:
+        a.step(130)  # a captured graph of 128 steps and two single ones
+        mem.refuse = not fused
+        with pytest.raises(L.LBMError):
+            a.configure(128, 8, 0, 3, fused)
+        mem.refuse = False
+        a.step(130)
+        b.step(260)
+        assert np.array_equal(a.f(), b.f())
+        a.configure(128, 8, 0, 3, 0)
+        b.configure(128, 8, 0, 3, 0)
+        a.step(3)
+        b.step(3)
+        assert np.array_equal(a.f(), b.f())
+
+
+def test_a_refused_batch_configuration_leaves_the_old_one(L):
+    cases = [_case(g, 1511 + sum(g)) for g in [(37, 20), (64, 64)]]
+    args = ([p for p, _ in cases], [c for _, c in cases], "bf16split")
+    with Hooks(L) as mem, L.Batch(*args) as a, L.Batch(*args) as b:
+        a.step(40)
+        mem.refuse = True
+        with pytest.raises(L.LBMError):
+            L.lbm_configure(a.h, 0, 0, 0, 16, 0)
+        mem.refuse = False
+        a.step(40)
+        b.step(80)
+        for i in range(len(cases)):
+            assert np.array_equal(a.C(i), b.C(i)), i
+            assert a.mass(i) == b.mass(i), i
+
+
+# with varying coefficients a split needs no larger F; constant ones again would take slots of it
+# and go without where they are refused
+def test_constant_coefficients_again_without_memory(L):
+    pb, C0 = _case((520, 520), 1409)
+    one = np.ones(pb.shape)
+    with Hooks(L) as mem, L.Lattice(pb, C0, "bf16split") as a, L.Lattice(pb, C0, "bf16split") as b:
+        a.set_fields(u=np.stack([pb.u[0] * one, pb.u[1] * one]), g=np.stack([pb.g[0] * one, pb.g[1] * one]))
+        for lat in (a, b):
+            lat.configure(128, 8, 0, 0, 0)
+        mem.refuse = True
+        a.set_fields()
+        mem.refuse = False
+        b.reset()
+        a.step(130)
+        b.step(130)
+        assert np.array_equal(a.f(), b.f())
