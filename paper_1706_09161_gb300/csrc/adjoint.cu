@@ -383,12 +383,6 @@ adj_G_gemm64(const GLayout L, const real* __restrict__ A, const real* __restrict
 // 256^2, 15 steps, both axes, single cold-cache launches: 570 us before, 105 us now.
 constexpr int GM = 64, GN = 32;
 
-__device__ __forceinline__ unsigned long long fadd2(unsigned long long a, unsigned long long b) {
-  unsigned long long d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
 template <bool NCONTIG>
 __global__ void __launch_bounds__(64)
 adj_G_gemm32(const GLayout L, const float* __restrict__ A, const float* __restrict__ B, float2* __restrict__ part) {

@@ -527,6 +527,7 @@ static int create_problem(const lbm_params* prm, const double* C0_host, void* st
   if (prm->precision == LBM_FP32 && !batched) {
     h->simt_ks = lbm::simt_ksplit(h);  // small FP32 problems: the SIMT operator's contraction split
   }
+  h->simt_sub = lbm::simt_sub(h);
   long long ksz = 0;
   for (int mu = 0; mu < h->d; ++mu) ksz += (long long)prm->grid[mu] * prm->grid[mu];
   h->reduce_blocks = lbm::reduce_blocks_for(nodes);
@@ -939,6 +940,7 @@ int simt_replan(lbm_s* h, int ks) {
   for (int mu = 0; mu < h->d; ++mu) kbmin = std::min(kbmin, (h->sp.n[mu] + 31) / 32);
   if (ks > kbmin && ks != lbm::simt_ksplit(h)) return LBM_EINVAL;
   h->simt_ks = ks;
+  h->simt_sub = lbm::simt_sub(h);
   return LBM_OK;
 }
 

@@ -13,6 +13,7 @@
 // FP32: small problems split the contraction over the ks blocks of a thread-block cluster,
 // which add their partial tiles in slice order through distributed shared memory.
 #include <algorithm>
+#include <climits>
 
 #include "lbm_internal.h"
 #include "simt_dev.cuh"
@@ -36,6 +37,7 @@ struct GemmPlan {
   GemmAxis ax[3];
   int naxes;
   int ks;              // contraction slices per tile (FP32: the blocks of one cluster)
+  int sub;             // FP32: parts of a slice with an accumulation chain of their own, added in order
   long long total;
   int early;           // one-wave grid: let the next kernel be scheduled at block start
 };
@@ -67,12 +69,12 @@ __device__ __forceinline__ BlockAt locate_block(const GemmPlan& P, long long b, 
 // and columns, so that all shared and global accesses are 128-bit; the staged A is swizzled
 // so that transposing C's rows into it is free of bank conflicts.  Slices of SBK contraction
 // steps, double buffered through registers.  Each output's products are added in contraction
-// order within its slice, whichever tile serves it.
+// order within its part of a slice, whichever tile serves it.
 // Measured with the rules below, before (64 x 64 or 32 x 32 tiles of scalar FMAs, partial sums
 // added by the consumer) and after: step of 512^2 32.2 -> 22.9 us, 256^2 13.8 -> 9.6 us,
 // operator of 256^3 845 -> 484 us (66% of the FP32 pipe's rate), of 1024^2 98 us.
 constexpr int SBK = 16;
-constexpr int kSlice = 32;  // contraction slices of a split start at multiples of this
+constexpr int kSlice = 32;  // contraction slices of a split, and their parts, start at multiples of this
 
 __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr, uint32_t rank) {
   uint32_t r;
@@ -130,8 +132,10 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
   const int M = X.M, N = X.N, amode = X.amode;
   const bool va = X.vec & 1, vb = X.vec & 2, vc = X.vec & 4;
   const int nkb = (X.K + kSlice - 1) / kSlice;
-  const int kbeg = (rank * nkb / ks) * kSlice;
-  const int K = min(X.K, ((rank + 1) * nkb / ks) * kSlice);
+  // part j of the contraction (sub parts to a slice) starts here
+  auto part = [&](int j) { return (int)((long long)j * nkb / (ks * P.sub)) * kSlice; };
+  const int kbeg = part(rank * P.sub);
+  const int K = min(X.K, part((rank + 1) * P.sub));
   const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
 
   float4 ra[LA], rb[LB];
@@ -186,11 +190,29 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
 #pragma unroll
     for (int j = 0; j < 2 * CG; ++j) acc[i][j] = 0ull;
 
+  // the finished parts (SUB: only the 32 x 32 tiles have more than one)
+  constexpr bool SUB = RG == 1;
+  unsigned long long sum[SUB ? R : 1][SUB ? 2 * CG : 1] = {};
+  int j = 1, kpart = SUB && P.sub > 1 ? part(rank * P.sub + 1) : INT_MAX;
+  auto close_part = [&]() {  // acc joins the finished parts
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+      for (int h = 0; h < 2 * CG; ++h) {
+        sum[SUB ? i : 0][SUB ? h : 0] = fadd2(sum[SUB ? i : 0][SUB ? h : 0], acc[i][h]);
+        acc[i][h] = 0ull;
+      }
+  };
+
   fetch(kbeg);
   stash(0);
   __syncthreads();
   int buf = 0;
   for (int k0 = kbeg; k0 < K; k0 += SBK) {
+    if (SUB && k0 >= kpart) {
+      close_part();
+      while (k0 >= kpart) kpart = ++j < P.sub ? part(rank * P.sub + j) : INT_MAX;
+    }
     const bool more = k0 + SBK < K;
     if (more) fetch(k0 + SBK);
     const float* as = As + buf * SBK * BM;
@@ -218,6 +240,13 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
     if (more) stash(buf ^ 1);
     __syncthreads();
     buf ^= 1;
+  }
+  if (SUB && P.sub > 1) {
+    close_part();
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+      for (int h = 0; h < 2 * CG; ++h) acc[i][h] = sum[SUB ? i : 0][SUB ? h : 0];
   }
   auto row_of = [&](int i) { return 4 * TY * (i / 4) + 4 * ty + (i & 3); };
   auto quad = [&](int i, int h) {
@@ -406,6 +435,7 @@ GemmPlan make_plan(const lbm_s* h, const real* C, real* F, bool transpose, long 
   const real* KA = am ? KT : K;
   GemmPlan P{};
   P.ks = ks;
+  P.sub = 1;
   long long koff = 0;
   // axis x: F_0 = C (rows x n0) * K_0^T
   add_axis(P, BM, BN, (int)(nodes / n0), n0, n0, 1, 0, C, n0, 0, KT + koff, n0, 0, F, n0, 0);
@@ -496,6 +526,7 @@ cudaError_t frac_all_axes(const lbm_s* h, const real* C, real* F, cudaStream_t s
       // 2-D only: the 3-D marches' long blocks, launched early, would pile up two to an SM on
       // the SMs this grid leaves first (measured: 48^3 step 24 -> 37 us)
       P.early = !transpose && pdl && h->d == 2 && blocks_fit(kernel, G.THREADS, P.total);
+      P.sub = h->simt_sub;
       cfg.gridDim = dim3(static_cast<unsigned>(P.total), 1, 1);
       cfg.blockDim = dim3(G.THREADS, 1, 1);
       return cudaLaunchKernelEx(&cfg, kernel, P);
@@ -542,6 +573,24 @@ int simt_ksplit(const lbm_s* h) {
   while (ks * 2 <= 8 && ks * 2 <= kbs &&
          (tiles * ks < sms - sms / 10 || (ks < 4 && tiles * ks < 8 * sms && kmin >= 160 * ks))) ks *= 2;
   return ks;
+}
+
+// Parts of a slice that are summed on their own (the built-in split only: a split that is asked for
+// is taken as it is).  An FP32 chain of additions rounds at the scale of its running sum, so the
+// contraction is cut in as many chains as fill the GPU with two 64 x 64 tiles per SM, at least 32
+// steps each; where the built-in split has fewer slices than that (300^2 four of eight, 64^3 one of
+// two), a block sums its part of them one after the other.  Error of C against 64 bits, one chain
+// per slice / so: 64^3, 8 steps, 1.6e-7 / 1.4e-7.  The registers for it are there in the 32 x 32 tiles,
+// which serve every such grid.
+int simt_sub(const lbm_s* h) {
+  if (h->elem != 4 || h->simt_ks != simt_ksplit(h)) return 1;
+  const long long tiles = count_tiles(h, 64, 64);
+  int kmin = 1 << 30;
+  for (int mu = 0; mu < h->d; ++mu) kmin = std::min(kmin, h->sp.n[mu]);
+  const int kbs = (kmin + kSlice - 1) / kSlice;
+  int chains = 1;
+  while (chains * 2 <= 8 && chains * 2 <= kbs && tiles * chains < 2LL * device_sms()) chains *= 2;
+  return tiles * h->simt_ks < 2LL * device_sms() ? std::max(1, chains / h->simt_ks) : 1;
 }
 
 cudaError_t launch_frac_simt_T(const lbm_s* h, const void* in, long long in_stride, void* out, cudaStream_t s) {

@@ -12,6 +12,12 @@ __device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsign
   return d;
 }
 
+__device__ __forceinline__ unsigned long long fadd2(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
 __device__ __forceinline__ unsigned long long twice(float a) {
   unsigned long long d;
   asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(a));
