@@ -289,9 +289,12 @@ frac_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams P) {
 // and warps 2-5 drain the other accumulator (tcgen05.ld, 32 columns at a time, through a
 // double-buffered shared chunk and a TMA store), so a tile's epilogue overlaps the next
 // tile's loads and MMAs.  With 128-column tiles each accumulator buffer has two regions:
-// consecutive k-blocks alternate between them and the epilogue adds the two in FP32 (as
+// consecutive k-steps alternate between them and the epilogue adds the two in FP32 (as
 // the per-tile kernel's regions: shorter accumulation chains, smaller rounding error of
-// the split forms).  Every wait is bounded as in the per-tile kernel; on a timeout
+// the split forms).  The deep form (NBUF = 1, grids of one to two tiles per SM) has one buffer of
+// four regions, the chains of the per-tile kernel: a tile's MMAs then wait for the drain of the one
+// before, its loads don't (error of C against 64 bits after 8 steps, two regions / four: 100^3
+// bf16x6 1.8e-7 / 1.6e-7).  Every wait is bounded as in the per-tile kernel; on a timeout
 // the CTA stops issuing, waits (bounded) for its copies and MMAs in flight, releases
 // TMEM and returns with bit 2 of the error flag set.
 constexpr int PBN = 128;
@@ -303,13 +306,13 @@ __host__ __device__ constexpr int persist_threads(int E) { return E == 4 ? kPers
 // BN = 128 (three ring stages; two with the weights in three parts) or 256 (two; the
 // double accumulator then fills TMEM); KP = weight parts (2, or 3 for the five-product
 // bf16 form, BN = 128 only)
-template <int E, int BN = PBN, int KP = 2>
+template <int E, int BN = PBN, int KP = 2, int NBUF = 2>
 struct PCfg {
   using G = Cfg<E, BN, 1, KP>;
   static constexpr int STAGES = (BN == 128 && KP == 2) ? 3 : 2;
-  static constexpr int NREG = (2 * 2 * BN <= 512) ? 2 : 1;  // accumulator regions per buffer
+  static constexpr int NREG = NBUF == 1 ? 512 / BN : (2 * 2 * BN <= 512) ? 2 : 1;  // accumulator regions per buffer
   static_assert(NREG <= ksteps<E>(), "every region is written by a tile's first k-block");
-  static constexpr int TMEM_COLS = 2 * NREG * BN;
+  static constexpr int TMEM_COLS = NBUF * NREG * BN;
   static constexpr uint32_t CHUNK = 32 * BM * 4;  // 32 output rows x 128 x (FP32)
   static constexpr size_t RING = (size_t)STAGES * G::STAGE;
   static constexpr size_t SMEM = RING + 2 * CHUNK + 1024 /*align*/ + 256 /*barriers*/;
@@ -324,9 +327,9 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
 // Locate(t, maps, prm, cid): the problem and local tile index of global tile t
-template <int E, int BN, int KP, class Locate>
+template <int E, int BN, int KP, int NBUF, class Locate>
 __device__ __forceinline__ void persist_body(const Locate& locate, int ntiles, int* flag, uint8_t* smem_raw) {
-  using C = PCfg<E, BN, KP>;
+  using C = PCfg<E, BN, KP, NBUF>;
   using G = typename C::G;
   constexpr int STAGES = C::STAGES;
   constexpr int NREG = C::NREG;
@@ -404,8 +407,8 @@ __device__ __forceinline__ void persist_body(const Locate& locate, int ntiles, i
       locate(t, maps, P, cid);
       const TileAt tl = decode_tile(*P, cid, BN);
       const int nkb = P->ax[tl.mu].kblocks;
-      const int b = i & 1;
-      if (i >= 2 && !mbar_wait(&tempty[b], ((i >> 1) - 1) & 1, flag)) break;
+      const int b = i % NBUF;
+      if (i >= NBUF && !mbar_wait(&tempty[b], (i / NBUF - 1) & 1, flag)) break;
       tc_fence_after();
       const uint32_t d = tmem + b * NREG * BN;
       const int amode = a_mode<E>(tl.mu);
@@ -462,8 +465,8 @@ __device__ __forceinline__ void persist_body(const Locate& locate, int ntiles, i
       int cid;
       locate(t, maps, P, cid);
       const TileAt tl = decode_tile(*P, cid, BN);
-      const int b = i & 1;
-      if (et == 0) *s_ok = mbar_wait(&tfull[b], (i >> 1) & 1, flag) ? 1 : 0;
+      const int b = i % NBUF;
+      if (et == 0) *s_ok = mbar_wait(&tfull[b], (i / NBUF) & 1, flag) ? 1 : 0;
       epi_sync();
       if (!*s_ok) break;
       tc_fence_after();
@@ -578,11 +581,11 @@ struct LocateBatch {
   }
 };
 
-template <int E, int BN, int KP>
+template <int E, int BN, int KP, int NBUF>
 __global__ void __launch_bounds__(persist_threads(E), 1)
 frac_tc_persist_kernel(const __grid_constant__ TcMaps maps, const __grid_constant__ TcParams P) {
   extern __shared__ uint8_t smem_raw[];
-  persist_body<E, BN, KP>(LocateOne{&maps, &P}, P.total_tiles, P.flag, smem_raw);
+  persist_body<E, BN, KP, NBUF>(LocateOne{&maps, &P}, P.total_tiles, P.flag, smem_raw);
 }
 
 template <int E, int KP>
@@ -590,7 +593,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
 frac_tc_persist_batch_kernel(const TcMaps* __restrict__ maps, const TcParams* __restrict__ prm,
                              const int* __restrict__ start, int nprob, int ntiles, int* flag) {
   extern __shared__ uint8_t smem_raw[];
-  persist_body<E, PBN, KP>(LocateBatch{maps, prm, start, nprob}, ntiles, flag, smem_raw);
+  persist_body<E, PBN, KP, 2>(LocateBatch{maps, prm, start, nprob}, ntiles, flag, smem_raw);
 }
 
 // ---------------------------------------------------------------------------- splits
@@ -746,23 +749,30 @@ cudaError_t launch_bn(const TcPlan* p, cudaStream_t s) {
 }
 
 
-template <int E, int BN, int KP = 2>
-cudaError_t launch_persist(const TcPlan* p, cudaStream_t s) {
+template <int E, int BN, int KP, int NBUF>
+cudaError_t launch_persist_n(const TcPlan* p, cudaStream_t s) {
   static std::atomic<unsigned long long> attr{0};
-  if (const cudaError_t e = smem_attr_once(attr, frac_tc_persist_kernel<E, BN, KP>, (int)PCfg<E, BN, KP>::SMEM);
+  if (const cudaError_t e = smem_attr_once(attr, frac_tc_persist_kernel<E, BN, KP, NBUF>, (int)PCfg<E, BN, KP, NBUF>::SMEM);
       e != cudaSuccess)
     return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(std::min(p->prm.total_tiles, device_sms()), 1, 1);  // one CTA per SM
   cfg.blockDim = dim3(persist_threads(E), 1, 1);
-  cfg.dynamicSmemBytes = PCfg<E, BN, KP>::SMEM;
+  cfg.dynamicSmemBytes = PCfg<E, BN, KP, NBUF>::SMEM;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = p->pdl ? 1 : 0;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, frac_tc_persist_kernel<E, BN, KP>, p->maps, p->prm);
+  return cudaLaunchKernelEx(&cfg, frac_tc_persist_kernel<E, BN, KP, NBUF>, p->maps, p->prm);
+}
+
+template <int E, int BN, int KP = 2>
+cudaError_t launch_persist(const TcPlan* p, cudaStream_t s) {
+  if constexpr (BN == PBN)
+    if (p->deep) return launch_persist_n<E, BN, KP, 1>(p, s);
+  return launch_persist_n<E, BN, KP, 2>(p, s);
 }
 
 }  // namespace
@@ -878,7 +888,8 @@ int tc_prepare(lbm_s* h, const std::vector<std::vector<double>>& K, int force_bn
   // to 8 CTAs per tile so that about one CTA per SM is busy; more tiles than SMs: the persistent
   // kernel (128-column tiles, no split; step, per tile / persistent: 64^3 bf16x6 23.5 / 20.4 us,
   // 64 x 64 x 90 30.2 / 22.7, tf32x3 32.4 / 24.7, 1100^2 bf16x6 63.6 / 63.2; 130 x 40 x 50, where
-  // half the lines are padding, 36.1 / 36.9); batched handles always use it
+  // half the lines are padding, 36.1 / 36.9), the deep form of it where the per-tile plan would have
+  // 128-column tiles with four accumulator regions; batched handles always use it
   const int kSMs = device_sms();
   int bn = (p->kparts == 2 && tc_count_tiles(h, 256) >= kSMs) ? 256 : 128;
   const int kbmin = tc_kbmin(h);
@@ -897,17 +908,17 @@ int tc_prepare(lbm_s* h, const std::vector<std::vector<double>>& K, int force_bn
     bn = 64;
     ks = split(t64);
   }
-  bool persist = false;
+  int persist = 0;
   if (force_bn > 0) {
     bn = force_bn;
     ks = std::max(1, force_ks);
-    persist = (force_bn == PBN && ks == 1);
+    persist = force_bn == PBN && ks == 1 ? 1 : 0;
   } else if (tc_count_tiles(h, PBN) > kSMs) {
-    persist = true;
+    persist = bn == PBN && tc_count_tiles(h, PBN) < 2 * kSMs ? 2 : 1;
     bn = PBN;
     ks = 1;
   }
-  return tc_replan(h, bn, ks, persist ? 1 : 0);
+  return tc_replan(h, bn, ks, persist);
 }
 
 long long tc_count_tiles(const lbm_s* h, int bn) {
@@ -956,6 +967,7 @@ int tc_replan(lbm_s* h, int bn, int ks, int persist, bool must_grow) {
   TcPlan next = *h->tc;
   TcPlan* const p = &next;
   if (!(bn == 64 || bn == 128 || bn == 256) || !(ks == 1 || ks == 2 || ks == 4 || ks == 8)) return LBM_EINVAL;
+  if (persist == 2 && bn != PBN) return LBM_EINVAL;
   if ((persist && ((bn != PBN && bn != 256) || ks != 1)) || (bn == 256 && ks != 1) || ks > tc_kbmin(h))
     return LBM_EINVAL;
   // the five- and six-product forms keep third parts per stage: 64 or 128 columns
@@ -967,6 +979,7 @@ int tc_replan(lbm_s* h, int bn, int ks, int persist, bool must_grow) {
   const size_t* koff = p->koff;
   p->bn = bn;
   p->persist = persist != 0;
+  p->deep = persist == 2;
   // tensor maps
   const int BK = 128 / E;
   const int MNW = 128 / E;  // MN-major box width (elements)
@@ -1155,7 +1168,7 @@ void tc_config(const lbm_s* h, int* bn, int* ks, int* persist) {
   const TcPlan* p = h->tc;
   *bn = p ? p->bn : 0;
   *ks = p ? p->prm.ksplit : 0;
-  *persist = (p && p->persist) ? 1 : 0;
+  *persist = (p && p->persist) ? (p->deep ? 2 : 1) : 0;
 }
 
 bool tc_one_wave(const lbm_s* h) {
@@ -1240,7 +1253,7 @@ int tc_set_gfield(lbm_s* h, bool on) {
       }
     p->gvar = true;
   }
-  return tc_replan(h, p->bn, p->prm.ksplit, p->persist ? 1 : 0, false);  // re-encodes the operand maps
+  return tc_replan(h, p->bn, p->prm.ksplit, p->persist ? (p->deep ? 2 : 1) : 0, false);  // re-encodes the operand maps
 }
 
 cudaError_t launch_split_C(const lbm_s* h, cudaStream_t s) {

@@ -235,7 +235,7 @@ int reduce_blocks_for(long long n);
 // force_bn / force_ks (> 0) fix the column-tile width and k-split (grouped batches use 128 / 1)
 int tc_prepare(lbm_s* h, const std::vector<std::vector<double>>& K, int force_bn, int force_ks);
 // operator plan: column tile width bn (64, 128, 256), contraction split ks (1, 2, 4, 8),
-// persistent kernel or one CTA per tile; re-encodes the tensor maps (LBM_EINVAL for a
+// persistent kernel (1: two accumulator buffers, 2: one deep one) or one CTA per tile; re-encodes the tensor maps (LBM_EINVAL for a
 // combination the kernels do not cover; the plan before stays after an error).  Captured graphs
 // must be dropped afterwards.
 int tc_replan(lbm_s* h, int bn, int ks, int persist, bool must_grow = true);

@@ -54,6 +54,7 @@ struct TcPlan {
   int cparts = 2;    // parts of C: 2, or 3 (bf16, six products)
   int bn = 64;
   bool persist = false;  // one CTA per SM walking the tile list (frac_tc_persist_kernel)
+  bool deep = false;     // persistent kernel with one accumulator buffer of four regions
   bool pdl = false;      // launch with programmatic stream serialization (the handle's choice)
   int ldk[3] = {0, 0, 0};     // padded row pitch of K_mu's split parts (elements)
   size_t koff[3] = {0, 0, 0}; // offset of K_mu's split parts (elements)
