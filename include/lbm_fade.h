@@ -431,7 +431,9 @@ int lbm_wait_check(int complete, int limit_us, void* stream);
  * parameter derivatives of K_mu (lbm_frac_matrix_grad), of Omega (Eqs. MatrixS, D_ab)
  * and of the advective equilibrium term (Eq. Feq), including the initial populations
  * feq(C0, K C0).  Forward states are recomputed from checkpoints taken every
- * ckpt_every steps (memory: ckpt_every + T/ckpt_every states); sums are FP64.
+ * ckpt_every steps (memory: ckpt_every + T/ckpt_every states).  Sums over nodes and steps are
+ * FP64; in FP32 forms the ones inside a node or a block are unevaluated pairs of floats (some
+ * 48 bits), and 16 products at a time of dL/dK_mu are added in FP32.
  *   snap_steps : nsnap strictly increasing step indices >= 0 (the last one is T)
  *   obs        : nsnap x nodes host doubles (field layout as lbm_create)
  * BGK and MRT single-problem handles with constant coefficients (LBM_ENOTSUP for batches and

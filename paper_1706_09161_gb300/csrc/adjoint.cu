@@ -19,9 +19,10 @@
 // plus the initial condition f(0) = feq(C0, K C0).  Forward states are recomputed from
 // checkpoints taken every `ckpt` steps, each kernel writing its slot of the segment; the last
 // segment's states come from the forward pass itself.  A backward step is two launches: the
-// step's adjoint and the operator's transpose.  Gradient sums are FP64; G_mu is one GEMM per
-// checkpoint segment (FP32 forms: products summed in FP32 over 16 terms, then as pairs of
-// floats).  256^2, 300 steps, 10 snapshots, checkpoints every 100, through the Python call:
+// step's adjoint and the operator's transpose.  Gradient sums are FP64, in FP32 forms those over a
+// node's populations as pairs of floats; G_mu is one GEMM per checkpoint segment (FP32 forms:
+// products summed in FP32 over 16 terms, then as pairs of floats in a block, which keep about 48
+// bits, and in FP64 over blocks).  256^2, 300 steps, 10 snapshots, checkpoints every 100, through the Python call:
 // 25.2 ms when slots were copied, the sums formed by passes of their own and G accumulated in
 // FP64; 12.8 ms now.
 #include <cuda.h>
@@ -32,6 +33,7 @@
 
 #include "lbm_internal.h"
 #include "simt_dev.cuh"
+#include "two_float.cuh"
 
 namespace lbm {
 namespace {
@@ -121,6 +123,31 @@ __device__ __forceinline__ void block_accumulate(const double* v, double* __rest
     for (int i = 0; i < kThreads / 32; ++i) acc += s[threadIdx.x][i];
     part[blockIdx.x * K + threadIdx.x] += acc;
   }
+}
+
+// (sum of x[q] y[q]) z to FP64's precision: FP32 terms as an unevaluated pair of floats, products by
+// FMA and sums by TwoSum (Ogita, Rump, Oishi 2005), which leaves the FP64 pipe one addition and two
+// conversions
+template <int Q>
+__device__ __forceinline__ double wide_dot(const double* x, const double* y, double z) {
+  double s = x[0] * y[0];
+#pragma unroll
+  for (int q = 1; q < Q; ++q) s += x[q] * y[q];
+  return s * z;
+}
+template <int Q>
+__device__ __forceinline__ double wide_dot(const float* x, const float* y, float z) {
+  float hi = __fmul_rn(x[0], y[0]), lo = __fmaf_rn(x[0], y[0], -hi);
+#pragma unroll
+  for (int q = 1; q < Q; ++q) {
+    const float p = __fmul_rn(x[q], y[q]), pe = __fmaf_rn(x[q], y[q], -p);
+    float s, e;
+    two_sum(hi, p, s, e);
+    hi = s;
+    lo = __fadd_rn(lo, __fadd_rn(e, pe));
+  }
+  const float p = __fmul_rn(hi, z), e = __fmaf_rn(lo, z, __fmaf_rn(hi, z, -p));
+  return static_cast<double>(p) + (isfinite(p) ? static_cast<double>(e) : 0.0);
 }
 
 // Adds the warp's FP64 sums of v[0..K) to part[warp * K + k] (fixed order; the same grid
@@ -237,13 +264,10 @@ adj_step_kernel(const __grid_constant__ AdjConst<real> c, const real* __restrict
     } else {
 #pragma unroll
       for (int mu = 0; mu < D; ++mu) {
-        real a = c.da[mu][0] * ls[0], b = c.db[mu][0] * dl[0];
+        real b = c.db[mu][0] * dl[0];
 #pragma unroll
-        for (int q = 1; q < Q; ++q) {
-          a += c.da[mu][q] * ls[q];
-          b += c.db[mu][q] * dl[q];
-        }
-        g[D + mu] = static_cast<double>(a) * static_cast<double>(b);
+        for (int q = 1; q < Q; ++q) b += c.db[mu][q] * dl[q];
+        g[D + mu] = wide_dot<Q>(c.da[mu], ls, b);
       }
     }
   }
@@ -528,17 +552,15 @@ __global__ void adj_G_reduce64(long long count, int nslab, const double* __restr
   }
 }
 
-// the slabs' pairs added as pairs, the result to FP64 (a non-finite sum has no meaningful lo)
+// the slabs' pairs added in FP64, in slab order (a non-finite sum has no meaningful lo)
 __global__ void adj_G_reduce32(long long count, int nslab, const float2* __restrict__ part, double* __restrict__ G) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x) {
-    float hi = 0.0f, lo = 0.0f;
+    double acc = 0.0;
     for (int z = 0; z < nslab; ++z) {
       const float2 v = part[(size_t)z * count + i];
-      const float s = __fadd_rn(hi, v.x), bp = __fsub_rn(s, hi);
-      lo = __fadd_rn(lo, __fadd_rn(v.y, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(v.x, bp))));
-      hi = s;
+      acc += isfinite(v.x) ? static_cast<double>(v.x) + static_cast<double>(v.y) : static_cast<double>(v.x);
     }
-    G[i] += isfinite(hi) ? static_cast<double>(hi) + static_cast<double>(lo) : static_cast<double>(hi);
+    G[i] += acc;
   }
 }
 
