@@ -526,8 +526,9 @@ static int create_problem(const lbm_params* prm, const double* C0_host, void* st
   const size_t E = h->elem;
   if (prm->precision == LBM_FP32 && !batched) {
     h->simt_ks = lbm::simt_ksplit(h);  // small FP32 problems: the SIMT operator's contraction split
+    h->simt_sub = lbm::simt_sub(h);
+    h->simt_built_in = true;
   }
-  h->simt_sub = lbm::simt_sub(h);
   long long ksz = 0;
   for (int mu = 0; mu < h->d; ++mu) ksz += (long long)prm->grid[mu] * prm->grid[mu];
   h->reduce_blocks = lbm::reduce_blocks_for(nodes);
@@ -928,19 +929,27 @@ int lbm_load(lbm_t h, const void* src_host, long long bytes) {
 namespace {
 
 struct TuneCfg {
-  int bn, ks, persist, chunk;
+  int bn, ks, persist, chunk;  // (ks: 0 is the built-in split of the FP32 SIMT operator)
   int fused = 0;
 };
 
-// FP32 SIMT operator of a single problem: contraction split ks (1, 2, 4 or 8, at most
-// the contraction blocks of 32 of the shortest axis)
+// FP32 SIMT operator of a single problem: contraction split ks (1, 2, 4 or 8, at most the
+// contraction blocks of 32 of the shortest axis: no slice is empty), one accumulation chain to a
+// slice, or the built-in split (ks = 0)
 int simt_replan(lbm_s* h, int ks) {
+  if (ks == 0) {
+    h->simt_ks = lbm::simt_ksplit(h);
+    h->simt_sub = lbm::simt_sub(h);
+    h->simt_built_in = true;
+    return LBM_OK;
+  }
   if (!(ks == 1 || ks == 2 || ks == 4 || ks == 8)) return LBM_EINVAL;
   int kbmin = 1 << 30;
   for (int mu = 0; mu < h->d; ++mu) kbmin = std::min(kbmin, (h->sp.n[mu] + 31) / 32);
-  if (ks > kbmin && ks != lbm::simt_ksplit(h)) return LBM_EINVAL;
+  if (ks > kbmin) return LBM_EINVAL;
   h->simt_ks = ks;
-  h->simt_sub = lbm::simt_sub(h);
+  h->simt_sub = 1;
+  h->simt_built_in = false;
   return LBM_OK;
 }
 
@@ -965,7 +974,7 @@ int set_cfg(lbm_s* h, const TuneCfg& c) {
     // from the collide-stream kernel, which the old one did not write
     LBM_CUDA(lbm::launch_split_C(h, h->stream));
   } else {
-    if (c.ks > 0 && h->elem == 4 && (rc = simt_replan(h, c.ks))) return rc;
+    if (h->elem == 4 && (rc = simt_replan(h, c.ks))) return rc;
     h->pdl = pdl_fits(h);
   }
   return LBM_OK;
@@ -976,7 +985,7 @@ int set_cfg(lbm_s* h, const TuneCfg& c) {
 // graphs are dropped.  After an error the configuration is the one before the call (its buffers
 // are there: F only grows).
 int apply_cfg(lbm_s* h, const TuneCfg& c) {
-  TuneCfg old{0, h->simt_ks, 0, h->cs_chunk, h->fused ? 1 : 0};
+  TuneCfg old{0, h->simt_built_in ? 0 : h->simt_ks, 0, h->cs_chunk, h->fused ? 1 : 0};
   if (!h->is_batch() && h->tc) lbm::tc_config(h, &old.bn, &old.ks, &old.persist);
   const int rc = set_cfg(h, c);
   drop_graphs(h);
@@ -1035,10 +1044,8 @@ int lbm_configure(lbm_t h, int bn, int ks, int persist, int chunk, int fused) {
       c.persist = persist ? 1 : 0;
     }
   } else if (!h->is_batch() && h->elem == 4 && bn == 0 && !persist && !fused) {
-    // FP32 SIMT operator: its contraction split only; a split that is asked for leaves no slice empty
-    for (int mu = 0; ks > 0 && mu < h->d; ++mu)
-      if (ks > (h->sp.n[mu] + 31) / 32) return LBM_EINVAL;
-    c.ks = ks > 0 ? ks : h->simt_ks;
+    // FP32 SIMT operator: its contraction split only
+    c.ks = ks > 0 ? ks : h->simt_built_in ? 0 : h->simt_ks;
   } else if (bn > 0 || ks > 0 || persist || fused) {
     return LBM_EINVAL;  // no tensor-core operator to plan
   }
@@ -1056,7 +1063,7 @@ int lbm_autotune(lbm_t h, int nsteps, char* desc, int desc_len) {
   TuneCfg cur{0, 0, 0, h->cs_chunk > 0 ? h->cs_chunk : lbm::cs_chunk_default(h), h->fused ? 1 : 0};
   if (!h->is_batch() && h->tc) lbm::tc_config(h, &cur.bn, &cur.ks, &cur.persist);
   const bool simt32 = !h->is_batch() && !h->tc && h->elem == 4;  // FP32 SIMT operator
-  if (simt32) cur.ks = h->simt_ks;
+  if (simt32) cur.ks = h->simt_built_in ? 0 : h->simt_ks;
   // candidate chunks
   std::vector<int> chunks;
   if (h->is_batch()) {
@@ -1075,7 +1082,7 @@ int lbm_autotune(lbm_t h, int nsteps, char* desc, int desc_len) {
     for (int ks : {1, 2, 4, 8}) {
       int kbmin = 1 << 30;
       for (int mu = 0; mu < h->d; ++mu) kbmin = std::min(kbmin, (h->sp.n[mu] + 31) / 32);
-      if (ks <= kbmin || ks == cur.ks) ops.push_back({0, ks, 0, cur.chunk});
+      if (ks <= kbmin && !(h->simt_built_in && h->simt_sub == 1 && ks == h->simt_ks)) ops.push_back({0, ks, 0, cur.chunk});
     }
   if (!h->is_batch() && h->tc) {
     const int sms = lbm::device_sms();

@@ -13,6 +13,7 @@
 // FP32: small problems split the contraction over the ks blocks of a thread-block cluster,
 // which add their partial tiles in slice order through distributed shared memory.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 
 #include "lbm_internal.h"
@@ -67,13 +68,12 @@ __device__ __forceinline__ BlockAt locate_block(const GemmPlan& P, long long b, 
 // shared memory instead made the loop shared-memory bound: 16 wavefronts per 16 clocks of
 // FMAs; 256^3 operator 584 us against 484.)  A thread's outputs come in groups of four rows
 // and columns, so that all shared and global accesses are 128-bit; the staged A is swizzled
-// so that transposing C's rows into it is free of bank conflicts.  Slices of SBK contraction
-// steps, double buffered through registers.  Each output's products are added in contraction
+// so that transposing C's rows into it is free of bank conflicts.  Rounds of SBK contraction
+// steps (groups of 16), double buffered through registers.  Each output's products are added in contraction
 // order within its part of a slice, whichever tile serves it.
 // Measured with the rules below, before (64 x 64 or 32 x 32 tiles of scalar FMAs, partial sums
 // added by the consumer) and after: step of 512^2 32.2 -> 22.9 us, 256^2 13.8 -> 9.6 us,
 // operator of 256^3 845 -> 484 us (66% of the FP32 pipe's rate), of 1024^2 98 us.
-constexpr int SBK = 16;
 constexpr int kSlice = 32;  // contraction slices of a split, and their parts, start at multiples of this
 
 __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr, uint32_t rank) {
@@ -103,16 +103,20 @@ __device__ __forceinline__ void store4(float* p, float4 v, int left, bool vec) {
   if (left > 3) p[3] = v.w;
 }
 
-template <int RG, int CG, int TY>
+template <int RG, int CG, int TY, int SBK, bool SUB>
+__global__ void __launch_bounds__(8 * TY) frac_simt32_kernel(const __grid_constant__ GemmPlan P);
+
+template <int RG, int CG, int TY, int SBK, bool SUB = false>
 struct F32Cfg {
-  static constexpr int THREADS = 8 * TY;
+  static constexpr int THREADS = 8 * TY, AMODE = 1;
   static constexpr int BM = 4 * RG * TY, BN = 32 * CG;
+  static auto kernel() { return frac_simt32_kernel<RG, CG, TY, SBK, SUB>; }
 };
 
-template <int RG, int CG, int TY>
+template <int RG, int CG, int TY, int SBK, bool SUB>
 __global__ void __launch_bounds__(8 * TY)
 frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
-  using G = F32Cfg<RG, CG, TY>;
+  using G = F32Cfg<RG, CG, TY, SBK, SUB>;
   constexpr int THREADS = G::THREADS, BM = G::BM, BN = G::BN, R = 4 * RG;
   constexpr int LA = BM * SBK / 4 / THREADS;       // float4 loads per thread
   constexpr int LB = BN * SBK / 4 / THREADS;
@@ -133,9 +137,10 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
   const bool va = X.vec & 1, vb = X.vec & 2, vc = X.vec & 4;
   const int nkb = (X.K + kSlice - 1) / kSlice;
   // part j of the contraction (sub parts to a slice) starts here
-  auto part = [&](int j) { return (int)((long long)j * nkb / (ks * P.sub)) * kSlice; };
-  const int kbeg = part(rank * P.sub);
-  const int K = min(X.K, part((rank + 1) * P.sub));
+  const int sub = SUB ? P.sub : 1;
+  auto part = [&](int j) { return j * nkb / (ks * sub) * kSlice; };
+  const int kbeg = part(rank * sub);
+  const int K = min(X.K, part((rank + 1) * sub));
   const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
 
   float4 ra[LA], rb[LB];
@@ -144,7 +149,7 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
     for (int i = 0; i < LA; ++i) {
       const int e = tid + i * THREADS;
       if (amode == 0) {  // four k of one row
-        const int m = m0 + e / (SBK / 4), k = k0 + 4 * (e % (SBK / 4));
+        const int m = m0 + e / 4 % BM, k = k0 + 16 * (e / (4 * BM)) + 4 * (e % 4);
         ra[i] = load4(A + m * X.lda + k, m < M ? K - k : 0, va);
       } else {           // four rows at one k
         const int k = k0 + e / (BM / 4), m = m0 + 4 * (e % (BM / 4));
@@ -166,15 +171,15 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
       const int e = tid + i * THREADS;
       const float4 v = ra[i];
       if (amode == 0) {
-        const int kq = e % (SBK / 4);
-        float* p = as + 4 * kq * BM + ((e / (SBK / 4)) ^ (8 * kq));
+        const int kq = 4 * (e / (4 * BM)) + e % 4;
+        float* p = as + 4 * kq * BM + ((e / 4 % BM) ^ (8 * (kq % 4)));
         p[0] = v.x;
         p[BM] = v.y;
         p[2 * BM] = v.z;
         p[3 * BM] = v.w;
       } else {
         const int k = e / (BM / 4);
-        *reinterpret_cast<float4*>(as + k * BM + ((4 * (e % (BM / 4))) ^ (8 * (k / 4)))) = v;
+        *reinterpret_cast<float4*>(as + k * BM + ((4 * (e % (BM / 4))) ^ (8 * (k / 4 % 4)))) = v;
       }
     }
 #pragma unroll
@@ -190,10 +195,9 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
 #pragma unroll
     for (int j = 0; j < 2 * CG; ++j) acc[i][j] = 0ull;
 
-  // the finished parts (SUB: only the 32 x 32 tiles have more than one)
-  constexpr bool SUB = RG == 1;
+  // the finished parts of the slice (SUB: it may have more than one)
   unsigned long long sum[SUB ? R : 1][SUB ? 2 * CG : 1] = {};
-  int j = 1, kpart = SUB && P.sub > 1 ? part(rank * P.sub + 1) : INT_MAX;
+  int j = 1, kpart = SUB ? part(rank * sub + 1) : INT_MAX;
   auto close_part = [&]() {  // acc joins the finished parts
 #pragma unroll
     for (int i = 0; i < R; ++i)
@@ -211,7 +215,7 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
   for (int k0 = kbeg; k0 < K; k0 += SBK) {
     if (SUB && k0 >= kpart) {
       close_part();
-      while (k0 >= kpart) kpart = ++j < P.sub ? part(rank * P.sub + j) : INT_MAX;
+      while (k0 >= kpart) kpart = ++j < sub ? part(rank * sub + j) : INT_MAX;
     }
     const bool more = k0 + SBK < K;
     if (more) fetch(k0 + SBK);
@@ -219,11 +223,12 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
     const float* bs = Bs + buf * SBK * BN + 4 * tx;
 #pragma unroll
     for (int kk = 0; kk < SBK; ++kk) {
+      if (kk > 0 && kk % 16 == 0 && k0 + kk >= K) break;  // the rest of the round is past the end
       float4 a[RG];
       ulonglong2 b[CG];
 #pragma unroll
       for (int g = 0; g < RG; ++g)
-        a[g] = *reinterpret_cast<const float4*>(as + kk * BM + 4 * TY * g + ((4 * ty) ^ (8 * (kk / 4))));
+        a[g] = *reinterpret_cast<const float4*>(as + kk * BM + 4 * TY * g + ((4 * ty) ^ (8 * (kk / 4 % 4))));
 #pragma unroll
       for (int h = 0; h < CG; ++h) b[h] = *reinterpret_cast<const ulonglong2*>(bs + kk * BN + 32 * h);
 #pragma unroll
@@ -241,7 +246,7 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
     __syncthreads();
     buf ^= 1;
   }
-  if (SUB && P.sub > 1) {
+  if (SUB) {
     close_part();
 #pragma unroll
     for (int i = 0; i < R; ++i)
@@ -296,51 +301,62 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
   if (!P.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// ---------------------------------------------------------------------------- FP64
-// Bound by the FP64 pipe (2 FMA per clock and SM: a warp instruction holds it for 16
+// ---------------------------------------------------------------------------- FP64, small FP32
+// FP64 is bound by the FP64 pipe (2 FMA per clock and SM: a warp instruction holds it for 16
 // clocks), so what counts is that every SM gets the same share of the tiles and that no
 // tile is padding; shared-memory and issue costs hide behind the pipe.  256 threads per
 // block; tiles of T x T outputs, T = 32 (2 x 2 per thread), 16 (1 each) or 8 (1 each, four
 // thread groups taking a quarter of each contraction slice).  Measured against tiles of 64 and
 // 32 alone: operator of 64^2 (8 blocks of 32 x 32 before, 128 of 8 x 8 now) 23 -> 7 us with the
 // launch, of 80^3 (each side of 80 padded to 128 before) 409 -> 246 us, 79% of the FP64 pipe.
-template <int T>
-struct F64Cfg {
+// FP32 (T = 32): the unsplit operator of small grids, batch members above all, is a chain of load
+// latencies in too few blocks to hide them; the 256 threads here have four times the loads in
+// flight of the packed kernel's 64 (operator and march of 3 problems of 224^2: 65 us per step with
+// the packed kernel, 45 so; 8 of 128^2 110 and 75).
+template <typename real, int T, bool SUB>
+__global__ void __launch_bounds__(256) frac_plain_kernel(const __grid_constant__ GemmPlan P);
+
+template <typename real, int T, bool SUB = false>
+struct PlainCfg {
+  static constexpr int THREADS = 256;
+  static constexpr int BM = T, BN = T, AMODE = 0;
+  static auto kernel() { return frac_plain_kernel<real, T, SUB>; }
   static constexpr int BK = 32;
   static constexpr int KSL = T == 8 ? 4 : 1;     // in-block contraction groups
   static constexpr int TR = T == 32 ? 2 : 1;     // outputs per thread along either side
   static constexpr int L = (T * BK + 255) / 256; // elements per thread and operand
 };
 
-template <int T>
+template <typename real, int T, bool SUB>
 __global__ void __launch_bounds__(256)
-frac_simt64_kernel(const __grid_constant__ GemmPlan P) {
-  using G = F64Cfg<T>;
+frac_plain_kernel(const __grid_constant__ GemmPlan P) {
+  using G = PlainCfg<real, T, SUB>;
   constexpr int BK = G::BK, TR = G::TR, KSL = G::KSL, PK = BK / KSL;
-  __shared__ double As[2][T][BK + 1];
-  __shared__ double Bs[2][BK][T];
+  static_assert(G::AMODE == 0, "A is read with k contiguous");
+  __shared__ real As[2][T][BK + 1];
+  __shared__ real Bs[2][BK][T];
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (P.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const BlockAt at = locate_block(P, blockIdx.x, T, T);
+  const BlockAt at = locate_block(P, blockIdx.x, G::BM, G::BN);
   const GemmAxis& X = P.ax[at.a];
   const int m0 = at.m0, n0 = at.n0;
-  const double* __restrict__ A = static_cast<const double*>(X.A) + at.bz * X.sA;
-  const double* __restrict__ B = static_cast<const double*>(X.B) + at.bz * X.sB;
-  double* __restrict__ Cm = static_cast<double*>(X.C) + at.bz * X.sC;
+  const real* __restrict__ A = static_cast<const real*>(X.A) + at.bz * X.sA;
+  const real* __restrict__ B = static_cast<const real*>(X.B) + at.bz * X.sB;
+  real* __restrict__ Cm = static_cast<real*>(X.C) + at.bz * X.sC;
   const int M = X.M, N = X.N, K = X.K;
   const int tid = threadIdx.x;
   const int grp = tid / (256 / KSL), t = tid % (256 / KSL);
   const int ty = t / (T / TR), tx = t % (T / TR);
 
-  double ra[G::L], rb[G::L];
+  real ra[G::L], rb[G::L];
   auto fetch = [&](int k0) {
 #pragma unroll
     for (int i = 0; i < G::L; ++i) {
       const int e = tid + i * 256;
       const int m = m0 + e / BK, ka = k0 + e % BK;
-      ra[i] = (m < M && ka < K) ? A[m * X.lda + ka] : 0.0;
+      ra[i] = (m < M && ka < K) ? A[m * X.lda + ka] : static_cast<real>(0);
       const int kb = k0 + e / T, n = n0 + e % T;
-      rb[i] = (kb < K && n < N) ? B[kb * X.ldb + n] : 0.0;
+      rb[i] = (kb < K && n < N) ? B[kb * X.ldb + n] : static_cast<real>(0);
     }
   };
   auto stash = [&](int buf) {
@@ -351,22 +367,39 @@ frac_simt64_kernel(const __grid_constant__ GemmPlan P) {
       Bs[buf][e / T][e % T] = rb[i];
     }
   };
-  double acc[TR][TR];
+  real acc[TR][TR];
 #pragma unroll
   for (int i = 0; i < TR; ++i)
 #pragma unroll
-    for (int j = 0; j < TR; ++j) acc[i][j] = 0.0;
+    for (int j = 0; j < TR; ++j) acc[i][j] = static_cast<real>(0);
+  // the finished parts of the contraction (SUB, as in the packed kernel)
+  real sum[TR][TR] = {};
+  const int nkb = (K + kSlice - 1) / kSlice;
+  int part = 1, kpart = SUB ? nkb / P.sub * kSlice : INT_MAX;
+  auto close_part = [&]() {
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+      for (int j = 0; j < TR; ++j) {
+        sum[i][j] += acc[i][j];
+        acc[i][j] = static_cast<real>(0);
+      }
+  };
   fetch(0);
   stash(0);
   __syncthreads();
   int buf = 0;
   for (int k0 = 0; k0 < K; k0 += BK) {
+    if (SUB && k0 >= kpart) {
+      close_part();
+      while (k0 >= kpart) kpart = ++part < P.sub ? part * nkb / P.sub * kSlice : INT_MAX;
+    }
     const bool more = k0 + BK < K;
     if (more) fetch(k0 + BK);
 #pragma unroll
     for (int q = 0; q < PK; ++q) {
       const int kk = grp * PK + q;
-      double av[TR], bv[TR];
+      real av[TR], bv[TR];
 #pragma unroll
       for (int i = 0; i < TR; ++i) av[i] = As[buf][ty * TR + i][kk];
 #pragma unroll
@@ -380,8 +413,15 @@ frac_simt64_kernel(const __grid_constant__ GemmPlan P) {
     __syncthreads();
     buf ^= 1;
   }
+  if (SUB) {
+    close_part();
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+      for (int j = 0; j < TR; ++j) acc[i][j] = sum[i][j];
+  }
   if (KSL > 1) {  // the groups' sums, in contraction order (the operand buffers are idle)
-    double* red = &As[0][0][0];
+    real* red = &As[0][0][0];
     red[grp * T * T + t] = acc[0][0];
     __syncthreads();
     if (grp == 0)
@@ -423,15 +463,14 @@ void add_axis(GemmPlan& P, int BM, int BN, int M, int N, int K, int batch, int a
 
 // transpose = false: F_mu = K_mu applied along mu to C_mu, transpose = true: K_mu^T; the
 // input of axis mu is the field at C + mu * cstride (cstride = 0: one input for every axis);
-// T x T output tiles.  FP32 reads the y and z axes' A (K_mu) from the other stored
-// orientation, with the output index contiguous.
+// BM x BN output tiles.  am = 1 (the packed kernel) reads the y and z axes' A (K_mu) from the other
+// stored orientation, with the output index contiguous.
 template <typename real>
-GemmPlan make_plan(const lbm_s* h, const real* C, real* F, bool transpose, long long cstride, int BM, int BN, int ks) {
+GemmPlan make_plan(const lbm_s* h, const real* C, real* F, bool transpose, long long cstride, int BM, int BN, int ks, int am) {
   const int n0 = h->sp.n[0], n1 = h->sp.n[1], n2 = h->sp.n[2];
   const long long nodes = h->sp.nodes;
   const real* K = static_cast<const real*>(transpose ? h->dev.KT : h->dev.K);
   const real* KT = static_cast<const real*>(transpose ? h->dev.K : h->dev.KT);
-  const int am = sizeof(real) == 4 ? 1 : 0;
   const real* KA = am ? KT : K;
   GemmPlan P{};
   P.ks = ks;
@@ -462,12 +501,22 @@ long long count_tiles(const lbm_s* h, int BM, int BN) {
 
 // FP32 block tiles: 32 x 32 where 64 x 64 tiles (times the contraction split) leave SMs
 // without two blocks; else 128 x 64 unless its padding exceeds that of 64 x 64 tiles by 2%.
+// The 32 x 32 tiles of a split run in rounds of 32 steps (a chain may end there); unsplit (batch
+// members, short lines), up to two tiles per SM, on the plain kernel, and beyond in rounds of 64 (3 problems side by side, us
+// per step, packed with rounds of 32 / 64 / plain: 224^2 65 / 58 / 45, 320^2 76 / 62 / 63, 416^2
+// 94 / 84 / 97, 512^2 110 / 101 / 140).
 template <class F>
 auto with_tile32(const lbm_s* h, int ks, const F& f) {
   const long long t64 = count_tiles(h, 64, 64);
-  if (t64 * ks < 2LL * device_sms()) return f(frac_simt32_kernel<1, 1, 8>, F32Cfg<1, 1, 8>{});
-  if (200 * count_tiles(h, 128, 64) > 102 * t64) return f(frac_simt32_kernel<2, 2, 8>, F32Cfg<2, 2, 8>{});
-  return f(frac_simt32_kernel<2, 2, 16>, F32Cfg<2, 2, 16>{});
+  if (t64 * ks < 2LL * device_sms()) {
+    const bool sub = h->simt_sub > 1;
+    if (ks == 1 && count_tiles(h, 32, 32) <= 2LL * device_sms())
+      return sub ? f(PlainCfg<float, 32, true>{}) : f(PlainCfg<float, 32>{});
+    if (sub) return f(F32Cfg<1, 1, 8, 32, true>{});
+    return ks > 1 ? f(F32Cfg<1, 1, 8, 32>{}) : f(F32Cfg<1, 1, 8, 64>{});
+  }
+  if (200 * count_tiles(h, 128, 64) > 102 * t64) return f(F32Cfg<2, 2, 8, 16>{});
+  return f(F32Cfg<2, 2, 16, 16>{});
 }
 
 // FP64 tile side: the smallest share of the busiest SM, ceil(tiles / SMs) T^2 outputs, with
@@ -486,12 +535,21 @@ int tile64(const lbm_s* h) {
   return best;
 }
 
-// the grid of `blocks` blocks is resident at once (one wave)
-template <typename Kernel>
-bool blocks_fit(Kernel k, int threads, long long blocks) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, 0) != cudaSuccess) return false;
-  return blocks <= (long long)per_sm * device_sms();
+// the grid of `blocks` blocks is resident at once (one wave).  Asked of the driver once per kernel
+// and device: every launch needs the answer.
+template <class Cfg>
+bool blocks_fit(long long blocks) {
+  static std::atomic<int> known[64];  // blocks per SM + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  int v = known[dev & 63].load(std::memory_order_relaxed);
+  if (v == 0) {
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Cfg::kernel(), Cfg::THREADS, 0) != cudaSuccess)
+      return false;
+    known[dev & 63].store(v = per_sm + 1, std::memory_order_relaxed);
+  }
+  return blocks <= (long long)(v - 1) * device_sms();
 }
 
 template <typename real>
@@ -509,27 +567,27 @@ cudaError_t frac_all_axes(const lbm_s* h, const real* C, real* F, cudaStream_t s
   cfg.numAttrs = 1;
   if constexpr (sizeof(real) == 8) {
     const int T = tile64(h);
-    const GemmPlan P = make_plan<real>(h, C, F, transpose, cstride, T, T, 1);
+    const GemmPlan P = make_plan<real>(h, C, F, transpose, cstride, T, T, 1, 0);
     cfg.gridDim = dim3(static_cast<unsigned>(P.total), 1, 1);
     cfg.blockDim = dim3(256, 1, 1);
-    if (T == 32) return cudaLaunchKernelEx(&cfg, frac_simt64_kernel<32>, P);
-    if (T == 16) return cudaLaunchKernelEx(&cfg, frac_simt64_kernel<16>, P);
-    return cudaLaunchKernelEx(&cfg, frac_simt64_kernel<8>, P);
+    if (T == 32) return cudaLaunchKernelEx(&cfg, frac_plain_kernel<double, 32, false>, P);
+    if (T == 16) return cudaLaunchKernelEx(&cfg, frac_plain_kernel<double, 16, false>, P);
+    return cudaLaunchKernelEx(&cfg, frac_plain_kernel<double, 8, false>, P);
   } else {
     const int ks = h->simt_ks;
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = ks;
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     if (ks > 1) cfg.numAttrs = 2;
-    return with_tile32(h, ks, [&](auto kernel, auto G) {
-      GemmPlan P = make_plan<real>(h, C, F, transpose, cstride, G.BM, G.BN, ks);
+    return with_tile32(h, ks, [&](auto G) {
+      GemmPlan P = make_plan<real>(h, C, F, transpose, cstride, G.BM, G.BN, ks, G.AMODE);
       // 2-D only: the 3-D marches' long blocks, launched early, would pile up two to an SM on
       // the SMs this grid leaves first (measured: 48^3 step 24 -> 37 us)
-      P.early = !transpose && pdl && h->d == 2 && blocks_fit(kernel, G.THREADS, P.total);
+      P.early = !transpose && pdl && h->d == 2 && blocks_fit<decltype(G)>(P.total);
       P.sub = h->simt_sub;
       cfg.gridDim = dim3(static_cast<unsigned>(P.total), 1, 1);
       cfg.blockDim = dim3(G.THREADS, 1, 1);
-      return cudaLaunchKernelEx(&cfg, kernel, P);
+      return cudaLaunchKernelEx(&cfg, G.kernel(), P);
     });
   }
 }
@@ -540,17 +598,17 @@ bool simt_one_wave(const lbm_s* h) {
   if (h->elem == 8) {
     const int T = tile64(h);
     const long long b = count_tiles(h, T, T);
-    return T == 32 ? blocks_fit(frac_simt64_kernel<32>, 256, b) : T == 16 ? blocks_fit(frac_simt64_kernel<16>, 256, b)
-                                                                          : blocks_fit(frac_simt64_kernel<8>, 256, b);
+    return T == 32 ? blocks_fit<PlainCfg<double, 32>>(b)
+                   : T == 16 ? blocks_fit<PlainCfg<double, 16>>(b) : blocks_fit<PlainCfg<double, 8>>(b);
   }
-  return with_tile32(h, h->simt_ks, [&](auto kernel, auto G) {
-    return blocks_fit(kernel, G.THREADS, count_tiles(h, G.BM, G.BN) * h->simt_ks);
+  return with_tile32(h, h->simt_ks, [&](auto G) {
+    return blocks_fit<decltype(G)>(count_tiles(h, G.BM, G.BN) * h->simt_ks);
   });
 }
 
 long long simt_blocks(const lbm_s* h) {
   if (h->elem == 8) return count_tiles(h, tile64(h), tile64(h));
-  return with_tile32(h, h->simt_ks, [&](auto, auto G) { return count_tiles(h, G.BM, G.BN) * h->simt_ks; });
+  return with_tile32(h, h->simt_ks, [&](auto G) { return count_tiles(h, G.BM, G.BN) * h->simt_ks; });
 }
 
 // The split doubles while 64 x 64 tiles leave SMs without a block, or, up to four slices, while
@@ -559,6 +617,8 @@ long long simt_blocks(const lbm_s* h) {
 // 14.7 / 16.0, 512^2 32.4 / 26.4 / 22.8 / 26.1, 700 x 600 52 / 48 / 40 / 48, 1024^2 123 / 117 / 105 /
 // 117; 3-D with 1/2: 48^3 15.7 / 17.5, 64^3 15.8 / 18.6, 72^3 28.7 / 39.2).  The longer axis sets
 // the most slices in 2-D (by the shorter one: 1000 x 60 29.3 us against 14.5, 53 x 1001 35.8 and 15.2).
+// 2-D lines of at most 64 stay whole: the cluster costs more than the half of the contraction that it
+// takes off a block (32 steps from a reset, two slices / plain unsplit: 48^2 331 / 276 us, 64^2 322 / 267).
 int simt_ksplit(const lbm_s* h) {
   if (h->elem != 4) return 1;
   const long long tiles = count_tiles(h, 64, 64), sms = device_sms();
@@ -570,20 +630,20 @@ int simt_ksplit(const lbm_s* h) {
   // 2-D: as many slices as the longer axis has, the shorter one's last slices then being empty
   const int kbs = ((h->d == 2 ? kmax : kmin) + kSlice - 1) / kSlice;
   int ks = 1;
-  while (ks * 2 <= 8 && ks * 2 <= kbs &&
+  while (kmax > (h->d == 2 ? 64 : 0) && ks * 2 <= 8 && ks * 2 <= kbs &&
          (tiles * ks < sms - sms / 10 || (ks < 4 && tiles * ks < 8 * sms && kmin >= 160 * ks))) ks *= 2;
   return ks;
 }
 
-// Parts of a slice that are summed on their own (the built-in split only: a split that is asked for
-// is taken as it is).  An FP32 chain of additions rounds at the scale of its running sum, so the
+// Parts of a slice that are summed on their own with the built-in split (one that is asked for is taken
+// as it is, and a batch's members are unsplit).  An FP32 chain of additions rounds at the scale of its running sum, so the
 // contraction is cut in as many chains as fill the GPU with two 64 x 64 tiles per SM, at least 32
 // steps each; where the built-in split has fewer slices than that (300^2 four of eight, 64^3 one of
 // two), a block sums its part of them one after the other.  Error of C against 64 bits, one chain
 // per slice / so: 64^3, 8 steps, 1.6e-7 / 1.4e-7.  The registers for it are there in the 32 x 32 tiles,
 // which serve every such grid.
 int simt_sub(const lbm_s* h) {
-  if (h->elem != 4 || h->simt_ks != simt_ksplit(h)) return 1;
+  if (h->elem != 4) return 1;
   const long long tiles = count_tiles(h, 64, 64);
   int kmin = 1 << 30;
   for (int mu = 0; mu < h->d; ++mu) kmin = std::min(kmin, h->sp.n[mu]);

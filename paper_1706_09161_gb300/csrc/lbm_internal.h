@@ -104,6 +104,7 @@ struct lbm_s {
   size_t f_elems = 0;                  // capacity of dev.F (elements)
   int simt_ks = 1;                     // contraction split of the FP32 SIMT operator (blocks per cluster)
   int simt_sub = 1;                    // accumulation chains per slice of that split (simt_sub())
+  bool simt_built_in = false;          // the split is the built-in one, not one that was asked for
   // programmatic dependent launch between the operator and collide-stream: only when both
   // grids run in a single wave (measured: with multi-wave 3-D grids it costs ~30%)
   bool pdl = false;
@@ -167,7 +168,7 @@ cudaError_t launch_frac_simt(const lbm_s* h, const void* C, void* F, cudaStream_
 // contraction split of the FP32 SIMT operator for a single problem (a cluster of that many
 // blocks adds its partial tiles), 1 for FP64
 int simt_ksplit(const lbm_s* h);
-int simt_sub(const lbm_s* h);  // accumulation chains per slice of the handle's split
+int simt_sub(const lbm_s* h);  // accumulation chains per slice of the built-in split
 // the FP32 SIMT operator's grid is resident at once (programmatic dependent launch)
 bool simt_one_wave(const lbm_s* h);
 long long simt_blocks(const lbm_s* h);  // blocks of the SIMT operator's launch
