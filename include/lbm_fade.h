@@ -213,8 +213,8 @@ int lbm_write_f(lbm_t h, const double* f_host);
  *   tensor-core forms, single problem: the operator's column tile width (64, 128, 256),
  *     its contraction split (1, 2, 4, 8 partial sums) or the persistent kernel;
  *   FP32 form, single problem: the SIMT operator's contraction split (1, 2, 4, 8);
- *   every handle: collide-stream tile rows per block (2-D) or z chunks (3-D);
- *   batches: tile rows per block of every 2-D member.
+ *   every single problem: the collide-stream chunk (lbm_configure);
+ *   batches: that of every 2-D member.
  * The operator plan is searched first with the current collide-stream setting, then the
  * collide-stream setting with the best plan; 2-D bf16 plans are also tried as a fused
  * step (operator and collide-stream phases of many steps in one cooperative launch,
@@ -228,8 +228,11 @@ int lbm_autotune(lbm_t h, int nsteps, char* desc, int desc_len);
 /* Apply a launch configuration directly (for example one lbm_autotune found before):
  * bn > 0 sets the tensor-core operator plan (bn in {64, 128, 256}, ks in {1, 2, 4, 8},
  * persist 0/1; combinations the kernels do not cover give LBM_EINVAL), bn = 0 keeps it;
- * chunk > 0 sets the collide-stream tile rows (2-D) or z chunks (3-D), 0 the built-in
- * choice; fused = 1 runs whole steps in one cooperative kernel (2-D bf16 split with a
+ * chunk > 0 sets the collide-stream chunk, 0 the built-in choice: z chunks (3-D), tile rows
+ * of 16 node rows per block (2-D), pairs of node rows per warp (2-D members of a batch, and 2-D
+ * FP32-based handles with coefficients, a source or wall values per node, which then march in
+ * strips on every grid).  Such a handle keeps two chunks, one for constant coefficients and
+ * one for these: a call sets that of the march in force.  The result does not depend on it; fused = 1 runs whole steps in one cooperative kernel (2-D bf16 split with a
  * per-tile plan of 64/128 columns split 2 or 4, rows TMA can address; LBM_ENOTSUP
  * otherwise).  FP32 single problems take ks > 0 as the SIMT operator's contraction split
  * (1, 2, 4, 8, at most the 32-wide contraction blocks of the shortest axis) with

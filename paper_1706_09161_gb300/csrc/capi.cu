@@ -956,7 +956,7 @@ int simt_replan(lbm_s* h, int ks) {
 // the parts of apply_cfg; an error may leave some of them set
 int set_cfg(lbm_s* h, const TuneCfg& c) {
   int rc = LBM_OK;
-  h->cs_chunk = c.chunk;
+  lbm::cs_chunk_of(h) = c.chunk;
   if (h->is_batch()) return lbm::cs_batch_prepare(h);
   if (h->tc) {
     h->fused = false;
@@ -985,7 +985,7 @@ int set_cfg(lbm_s* h, const TuneCfg& c) {
 // graphs are dropped.  After an error the configuration is the one before the call (its buffers
 // are there: F only grows).
 int apply_cfg(lbm_s* h, const TuneCfg& c) {
-  TuneCfg old{0, h->simt_built_in ? 0 : h->simt_ks, 0, h->cs_chunk, h->fused ? 1 : 0};
+  TuneCfg old{0, h->simt_built_in ? 0 : h->simt_ks, 0, lbm::cs_chunk_of(h), h->fused ? 1 : 0};
   if (!h->is_batch() && h->tc) lbm::tc_config(h, &old.bn, &old.ks, &old.persist);
   const int rc = set_cfg(h, c);
   drop_graphs(h);
@@ -1035,7 +1035,7 @@ int time_steps(lbm_s* h, int nsteps, float* ms) {
 
 int lbm_configure(lbm_t h, int bn, int ks, int persist, int chunk, int fused) {
   if (!h || chunk < 0) return LBM_EINVAL;
-  TuneCfg c{0, 0, 0, chunk > 0 ? chunk : lbm::cs_chunk_default(h), fused ? 1 : 0};
+  TuneCfg c{0, 0, 0, chunk, fused ? 1 : 0};  // (chunk 0 is the built-in choice to every launch)
   if (!h->is_batch() && h->tc) {
     lbm::tc_config(h, &c.bn, &c.ks, &c.persist);
     if (bn > 0) {
@@ -1060,7 +1060,8 @@ int lbm_autotune(lbm_t h, int nsteps, char* desc, int desc_len) {
   std::vector<char> state((size_t)state_bytes(h));
   int rc = lbm_save(h, state.data(), (long long)state.size());
   if (rc) return rc;
-  TuneCfg cur{0, 0, 0, h->cs_chunk > 0 ? h->cs_chunk : lbm::cs_chunk_default(h), h->fused ? 1 : 0};
+  const int set = lbm::cs_chunk_of(h);
+  TuneCfg cur{0, 0, 0, set > 0 ? set : lbm::cs_chunk_default(h), h->fused ? 1 : 0};
   if (!h->is_batch() && h->tc) lbm::tc_config(h, &cur.bn, &cur.ks, &cur.persist);
   const bool simt32 = !h->is_batch() && !h->tc && h->elem == 4;  // FP32 SIMT operator
   if (simt32) cur.ks = h->simt_built_in ? 0 : h->simt_ks;

@@ -2013,13 +2013,13 @@ int early_trigger(const lbm_s* h, const dim3& g) {
 // 18.1 / 15.7); beyond, its second wave costs more than the strips' extra rows (512^2 bf16x6
 // 14.7 / 17.6, FP32 24.5 / 26.7, 1000 x 900 bf16x6 40.5 / 51.7).  The strips take the fewest rows
 // that fit one wave (1000 x 900 with 2 / 4 / 6 / 8 rows: 44.3 / 42.6 / 40.6 / 44.5 us), at most 8.
-int fields2_chunk(const lbm_s* h) {
-  if (h->cs_chunk > 0) return h->cs_chunk;
+int fields2_built_in(const lbm_s* h) {
   if (one_wave(dim3((h->sp.n[0] + TX - 1) / TX, (h->sp.n[1] + TY - 1) / TY, 1))) return 0;
   int c = 1;
   while (c < 4 && strip_grid(h->sp.n, c).items > 4LL * kStripWarps * device_sms()) ++c;
   return c;
 }
+int fields2_chunk(const lbm_s* h) { return h->fld_chunk > 0 ? h->fld_chunk : fields2_built_in(h); }
 
 template <bool MRT, int SPLIT>
 cudaError_t launch_march2(const cudaLaunchConfig_t& cfg, const KConst<float>& sp, const float* fi, const float* F,
@@ -2406,7 +2406,7 @@ long long cs_max_parts(const lbm_s* h) {
 int cs_chunk_default(const lbm_s* h) {
   const int bx = (h->sp.n[0] + TX - 1) / TX, by = (h->sp.n[1] + TY - 1) / TY;
   if (h->is_batch()) return kBatchChunk;
-  if (h->d == 2 && h->elem == 4 && h->fld.on) return fields2_chunk(h);
+  if (h->d == 2 && h->elem == 4 && h->fld.on) return fields2_built_in(h);
   if (h->d == 2) return h->elem == 4 ? ychunk_for((long long)bx * by, by) : 1;
   return h->elem == 8 ? march64_plan(h, 0).nz : z_chunks((long long)bx * by, h->sp.n[2]);
 }

@@ -108,8 +108,11 @@ struct lbm_s {
   // programmatic dependent launch between the operator and collide-stream: only when both
   // grids run in a single wave (measured: with multi-wave 3-D grids it costs ~30%)
   bool pdl = false;
-  // collide-stream work per block: 2-D tile rows, 3-D z chunks (0: the built-in choice)
+  // collide-stream work per block: 2-D tile rows, 3-D z chunks, batches: strip rows in units of
+  // kStripRows (0: the built-in choice).  The 2-D FP32 march of varying coefficients has its own
+  // setting (strip rows), so that one kind of march never takes what was chosen for the other.
   int cs_chunk = 0;
+  int fld_chunk = 0;
   // fused small-problem step (one cooperative launch runs many steps), if selected
   bool fused = false;
   int fused_grid = 0;
@@ -255,7 +258,9 @@ void cs_release(lbm_s* h);
 bool encode_f32_map(void* map, int rank, void* base, const unsigned long long* dims,
                     const unsigned long long* strides_bytes, const unsigned int* box);
 bool cs_one_wave(const lbm_s* h);  // the collide-stream grid fits in one wave
-int cs_chunk_default(const lbm_s* h);  // the built-in tile rows (2-D) / z chunks (3-D)
+int cs_chunk_default(const lbm_s* h);  // the built-in choice of the march in force, whatever is set
+// the chunk setting of the march in force
+inline int& cs_chunk_of(lbm_s* h) { return h->fld.on && h->d == 2 && h->elem == 4 ? h->fld_chunk : h->cs_chunk; }
 long long cs_max_parts(const lbm_s* h);  // the most mass partials any collide-stream launch of h writes
 // fused 2-D step (bf16 split, per-tile plan with 64/128-column tiles and a split of 2 or
 // 4): LBM_OK if this handle can run it (sets fused_grid), LBM_ENOTSUP otherwise

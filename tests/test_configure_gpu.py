@@ -128,3 +128,55 @@ def test_constant_coefficients_again_without_memory(L):
         a.step(130)
         b.step(130)
         assert np.array_equal(a.f(), b.f())
+
+
+# the mass is added up in the order of the march's blocks, so that its last bits tell the marches
+# and their chunks apart; the populations don't depend on them
+def test_the_built_in_chunk_comes_back(L):
+    pb, C0 = _case((300, 300), 1703)
+    fields = W.smooth_fields(np.random.default_rng(5), pb.grid, "mrt", D0=0.03, g_amp=0.2, u_amp=0.03)
+
+    def mass(lat):
+        lat.reset()
+        lat.step(5)
+        return lat.mass()
+
+    with L.Lattice(pb, C0, "bf16x6split") as a, L.Lattice(pb, C0, "bf16x6split") as b:
+        a.set_fields(**fields)
+        b.set_fields(**fields)
+        built_in = mass(a)
+        b.configure(0, 0, 0, 40, 0)
+        assert mass(b) != built_in  # (what this test can tell apart)
+        b.configure(0, 0, 0, 0, 0)
+        assert mass(b) == built_in
+
+
+@pytest.mark.parametrize("kind", ["fp32", "bf16x6split"])
+def test_a_chunk_belongs_to_its_march(L, kind):
+    pb, C0 = _case((300, 300), 1703)
+    fields = W.smooth_fields(np.random.default_rng(5), pb.grid, "mrt", D0=0.03, g_amp=0.2, u_amp=0.03)
+
+    def run(lat):
+        lat.reset()
+        lat.step(5)
+        return lat.f(), lat.mass()
+
+    def same(x, y):
+        return np.array_equal(x[0], y[0]) and x[1] == y[1]
+
+    with L.Lattice(pb, C0, kind) as a, L.Lattice(pb, C0, kind) as b:
+        b.configure(0, 0, 0, 3, 0)  # tile rows of the march of constant coefficients
+        const = run(b)
+        for lat in (a, b):
+            lat.set_fields(**fields)
+        assert same(run(a), run(b))
+        a.configure(0, 0, 0, 7, 0)  # strip rows of the march of varying ones
+        varying = run(a)
+        a.set_fields()
+        b.set_fields()
+        assert same(run(b), const)
+        a.set_fields(**fields)
+        assert same(run(a), varying)
+        a.set_fields()
+        with L.Lattice(pb, C0, kind) as fresh:
+            assert same(run(a), run(fresh))
