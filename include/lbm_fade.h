@@ -227,17 +227,22 @@ int lbm_autotune(lbm_t h, int nsteps, char* desc, int desc_len);
 
 /* Apply a launch configuration directly (for example one lbm_autotune found before):
  * bn > 0 sets the tensor-core operator plan (bn in {64, 128, 256}, ks in {1, 2, 4, 8},
- * persist 0/1; combinations the kernels do not cover give LBM_EINVAL), bn = 0 keeps it;
+ * persist 0/1; combinations the kernels do not cover give LBM_EINVAL), bn = 0 keeps it (a new
+ * handle of one to two 128-column tiles per SM has a persistent plan with the accumulator
+ * regions of the per-tile one, which no bn > 0 names);
  * chunk > 0 sets the collide-stream chunk, 0 the built-in choice: z chunks (3-D), tile rows
  * of 16 node rows per block (2-D), pairs of node rows per warp (2-D members of a batch, and 2-D
  * FP32-based handles with coefficients, a source or wall values per node, which then march in
  * strips on every grid).  Such a handle keeps two chunks, one for constant coefficients and
- * one for these: a call sets that of the march in force.  The result does not depend on it; fused = 1 runs whole steps in one cooperative kernel (2-D bf16 split with a
+ * one for these: a call sets that of the march in force.  The result does not depend on it;
+ * fused = 1 runs whole steps in one cooperative kernel (2-D bf16 split with a
  * per-tile plan of 64/128 columns split 2 or 4, rows TMA can address; LBM_ENOTSUP
  * otherwise).  FP32 single problems take ks > 0 as the SIMT operator's contraction split
  * (1, 2, 4, 8, at most the 32-wide contraction blocks of the shortest axis) with
- * bn = persist = fused = 0; other non-tensor-core handles accept only
- * bn = ks = persist = fused = 0.  Synchronises when the split needs a larger F. */
+ * bn = persist = fused = 0; ks = 0 keeps the split, on a new handle the built-in one (which
+ * on elongated 2-D grids may be above that limit); other non-tensor-core handles accept only
+ * bn = ks = persist = fused = 0.  After an error the configuration is the one before the
+ * call.  Synchronises for batches, and when a tensor-core split needs a larger F. */
 int lbm_configure(lbm_t h, int bn, int ks, int persist, int chunk, int fused);
 
 long long lbm_state_size(lbm_t h);

@@ -1151,7 +1151,13 @@ int lbm_autotune(lbm_t h, int nsteps, char* desc, int desc_len) {
     if (h->tc && !h->is_batch())
       std::snprintf(desc, (size_t)desc_len,
                     "%soperator %s bn=%d ks=%d, collide chunk=%d: %.2f us/step (default %.2f)",
-                    best.fused ? "fused step, " : "", best.persist ? "persistent" : "per-tile", best.bn, best.ks,
+                    best.fused ? "fused step, " : "",
+                    best.persist == 2 ? "persistent (built-in, four regions)" : best.persist ? "persistent" : "per-tile",
+                    best.persist == 2 ? 0 : best.bn, best.ks,  // (bn = 0 keeps the plan of a new handle)
+                    best.chunk, 1e3 * best_ms / nsteps, 1e3 * base_ms / nsteps);
+    else if (simt32 && best.ks == 0)  // (as lbm_configure takes it: the split of a new handle is kept)
+      std::snprintf(desc, (size_t)desc_len,
+                    "operator SIMT ks=0 (built-in: %d), collide chunk=%d: %.2f us/step (default %.2f)", h->simt_ks,
                     best.chunk, 1e3 * best_ms / nsteps, 1e3 * base_ms / nsteps);
     else if (simt32)
       std::snprintf(desc, (size_t)desc_len, "operator SIMT ks=%d, collide chunk=%d: %.2f us/step (default %.2f)",

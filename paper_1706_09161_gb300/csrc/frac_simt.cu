@@ -618,7 +618,7 @@ long long simt_blocks(const lbm_s* h) {
 // 117; 3-D with 1/2: 48^3 15.7 / 17.5, 64^3 15.8 / 18.6, 72^3 28.7 / 39.2).  The longer axis sets
 // the most slices in 2-D (by the shorter one: 1000 x 60 29.3 us against 14.5, 53 x 1001 35.8 and 15.2).
 // 2-D lines of at most 64 stay whole: the cluster costs more than the half of the contraction that it
-// takes off a block (32 steps from a reset, two slices / plain unsplit: 48^2 331 / 276 us, 64^2 322 / 267).
+// takes off a block (32 steps from a reset, two slices / plain unsplit in two chains: 48^2 331 / 291 us, 64^2 322 / 284).
 int simt_ksplit(const lbm_s* h) {
   if (h->elem != 4) return 1;
   const long long tiles = count_tiles(h, 64, 64), sms = device_sms();

@@ -2,6 +2,7 @@
 kind of march changes, and what a refused one leaves behind.  A configuration changes the schedule
 of a step, never its result: populations are equal bit for bit."""
 import dataclasses
+import re
 
 import numpy as np
 import pytest
@@ -180,3 +181,20 @@ def test_a_chunk_belongs_to_its_march(L, kind):
         a.set_fields()
         with L.Lattice(pb, C0, kind) as fresh:
             assert same(run(a), run(fresh))
+
+
+# what lbm_autotune reports can be passed back: also the built-in split of an elongated grid, above what
+# lbm_configure takes as a number, and the built-in persistent plan of one to two tiles per SM
+@pytest.mark.parametrize("kind,grid", [("fp32", (400, 33)), ("fp32", (300, 300)), ("bf16x6split", (75, 75, 75)),
+                                       ("tf32split", (260, 130))])
+def test_a_tuned_configuration_can_be_set_again(L, kind, grid):
+    pb, C0 = _case(grid, 1801)
+    with L.Lattice(pb, C0, kind) as a, L.Lattice(pb, C0, kind) as b:
+        desc = a.autotune(128)
+        ks, chunk = (int(re.search(key + r"=(\d+)", desc).group(1)) for key in ("ks", "chunk"))
+        bn = int(re.search(r"bn=(\d+)", desc).group(1)) if "bn=" in desc else 0
+        b.configure(bn, ks, int("persistent" in desc), chunk, 0)
+        for lat in (a, b):
+            lat.reset()
+            lat.step(5)
+        assert np.array_equal(a.f(), b.f()), desc
