@@ -151,20 +151,14 @@ __device__ __forceinline__ void collide_node(const KConst<real>& sp, const real*
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       real acc;
-      if constexpr (KS && sizeof(real) == 4) {
+      if constexpr (KS) {
+        static_assert(Q == 5 && sizeof(real) == 4, "rows of the 2-D FP32 matrix");
         const float4 a = s_om_rows[i][0];
         acc = a.x * dl[0];
         acc += a.y * dl[1];
         acc += a.z * dl[2];
         acc += a.w * dl[3];
-        if constexpr (Q == 5) {
-          acc += s_om_rows[i][1].x * dl[4];
-        } else {
-          const float4 b = s_om_rows[i][1];
-          acc += b.x * dl[4];
-          acc += b.y * dl[5];
-          acc += b.z * dl[6];
-        }
+        acc += s_om_rows[i][1].x * dl[4];
       } else {
         acc = sp.omega[i][0] * dl[0];
 #pragma unroll
@@ -338,7 +332,7 @@ __device__ __forceinline__ void block_mass(SumAcc<real>& macc, double* part, int
 constexpr int TX = 32, TY = 16, HALO_WARPS = 3;
 static_assert(kMassSlots * 32 == TX * (TY + HALO_WARPS), "one mass partial per warp of a block");
 
-template <typename real, int D, bool MRT, bool FLD = false, bool KS = false>
+template <typename real, int D, bool MRT, bool FLD = false>
 __device__ __forceinline__ void collide_at(const KConst<real>& sp, const real* __restrict__ f_in,
                                            const real* __restrict__ F, bool inside, long long node, real* fs,
                                            const FieldPtrs<real>& fp) {
@@ -362,7 +356,7 @@ __device__ __forceinline__ void collide_at(const KConst<real>& sp, const real* _
     for (int mu = 0; mu < D; ++mu) c.adv[mu] = fp.advw[mu * nodes + node];
     c.src = fp.src ? fp.src[node] : static_cast<real>(0);
     collide_node_field<real, D, MRT>(sp, fp, c, f, Fv, fs);
-  } else collide_node<real, D, MRT, KS>(sp, f, Fv, fs);
+  } else collide_node<real, D, MRT>(sp, f, Fv, fs);
 }
 
 // Asynchronous prefetch of the 2-D march (FP32): every thread copies the populations and
@@ -397,7 +391,7 @@ __host__ __device__ constexpr int march_warps(int txx, int tyy) { return (txx * 
 static_assert(march_warps(TX, TY) == TY + HALO_WARPS, "32 x 16 tiles: 16 owner and 3 ring warps");
 
 // One block's column (TXX x TYY tile bx, by; planes z0 .. z1-1) of one problem.
-template <typename real, int D, bool MRT, int SPLIT, bool FLD = false, bool KS = false, int TXX = TX, int TYY = TY>
+template <typename real, int D, bool MRT, int SPLIT, bool FLD = false, int TXX = TX, int TYY = TY>
 __device__ __forceinline__ void march_body(const KConst<real>& sp, const real* __restrict__ f_in,
                                            const real* __restrict__ F, real* __restrict__ f_out,
                                            real* __restrict__ C_out, int* __restrict__ flag, const SplitOut& so,
@@ -444,22 +438,22 @@ __device__ __forceinline__ void march_body(const KConst<real>& sp, const real* _
   if (owner) {
     if (D == 3) {
       real t[Q];
-      collide_at<real, D, MRT, FLD, KS>(sp, f_in, F, in_xy && z0 > 0, col + (z0 - 1) * plane, t, fp);
+      collide_at<real, D, MRT, FLD>(sp, f_in, F, in_xy && z0 > 0, col + (z0 - 1) * plane, t, fp);
       prev5 = t[5];
     }
-    collide_at<real, D, MRT, FLD, KS>(sp, f_in, F, in_xy, col + z0 * plane, cur, fp);
+    collide_at<real, D, MRT, FLD>(sp, f_in, F, in_xy, col + z0 * plane, cur, fp);
   }
   int buf = 0;
   for (int z = z0; z < z1; ++z) {
     if (owner) {
-      if (D == 3) collide_at<real, D, MRT, FLD, KS>(sp, f_in, F, in_xy && z + 1 < n2, col + (z + 1) * plane, nxt, fp);
+      if (D == 3) collide_at<real, D, MRT, FLD>(sp, f_in, F, in_xy && z + 1 < n2, col + (z + 1) * plane, nxt, fp);
       s_m[buf][0][sy][sx] = cur[1];
       s_m[buf][1][sy][sx] = cur[2];
       s_m[buf][2][sy][sx] = cur[3];
       s_m[buf][3][sy][sx] = cur[4];
     } else {
       real h[Q];
-      collide_at<real, D, MRT, FLD, KS>(sp, f_in, F, in_xy, col + z * plane, h, fp);
+      collide_at<real, D, MRT, FLD>(sp, f_in, F, in_xy, col + z * plane, h, fp);
       if (side == 0) s_m[buf][0][sy][sx] = h[1];       // moves +x into the tile
       else if (side == 1) s_m[buf][1][sy][sx] = h[2];  // moves -x into the tile
       else if (side == 2) s_m[buf][2][sy][sx] = h[3];  // moves +y into the tile
@@ -553,7 +547,7 @@ __shared__ float s_m2[2][4][TY + 2][TX + 2];
 // rows tr0 .. tr0 + ychunk - 1 of column bx), each thread prefetching its node of the
 // next two tiles through the cp.async ring while the current tile is collided.  The
 // per-tile work is that of march_body with one plane.
-template <bool MRT, int SPLIT, bool KS = false>
+template <bool MRT, int SPLIT>
 __device__ __forceinline__ void march2_pipe(const KConst<float>& sp, const float* __restrict__ f_in,
                                             const float* __restrict__ F, float* __restrict__ f_out,
                                             float* __restrict__ C_out, int* __restrict__ flag, const SplitOut& so,
@@ -621,7 +615,7 @@ __device__ __forceinline__ void march2_pipe(const KConst<float>& sp, const float
 #pragma unroll
         for (int mu = 0; mu < D; ++mu) Fv[mu] = frac_term(sp, F, mu, gx + (long long)n0 * gy);
       }
-      collide_node<float, D, MRT, KS>(sp, fv, Fv, fs);
+      collide_node<float, D, MRT>(sp, fv, Fv, fs);
     } else {
 #pragma unroll
       for (int q = 0; q < Q; ++q) fs[q] = 0.f;
@@ -1015,8 +1009,8 @@ collide_stream_march_kernel(const KConst<real> sp, const real* __restrict__ f_in
   const int bz = blockIdx.z;
   const int z0 = static_cast<int>((long long)bz * n2 / nz), z1 = static_cast<int>((long long)(bz + 1) * n2 / nz);
   if (early) pdl_trigger();
-  march_body<real, D, MRT, SPLIT, FLD, false, TXX, TYY>(sp, f_in, F, f_out, C_out, flag, so, blockIdx.x, blockIdx.y, z0, z1, mpart,
-                                       block_linear(), fp);
+  march_body<real, D, MRT, SPLIT, FLD, TXX, TYY>(sp, f_in, F, f_out, C_out, flag, so, blockIdx.x, blockIdx.y, z0, z1,
+                                                 mpart, block_linear(), fp);
   if (!early) pdl_trigger();
 }
 
@@ -2389,7 +2383,6 @@ bool cs_one_wave(const lbm_s* h) {
     const int ychunk = h->cs_chunk > 0 ? std::min(h->cs_chunk, by) : ychunk_for((long long)bx * by, by);
     return one_wave(dim3(bx, (by + ychunk - 1) / ychunk, 1));
   }
-  if (h->d == 2) return one_wave(dim3(bx, by, 1));
   const int nz = h->cs_chunk > 0 ? std::min(h->cs_chunk, h->sp.n[2]) : z_chunks((long long)bx * by, h->sp.n[2]);
   return one_wave(dim3(bx, by, nz));
 }

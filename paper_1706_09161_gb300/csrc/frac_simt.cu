@@ -16,6 +16,7 @@
 #include <atomic>
 #include <climits>
 
+#include "cluster_dev.cuh"
 #include "lbm_internal.h"
 #include "simt_dev.cuh"
 
@@ -75,22 +76,6 @@ __device__ __forceinline__ BlockAt locate_block(const GemmPlan& P, long long b, 
 // added by the consumer) and after: step of 512^2 32.2 -> 22.9 us, 256^2 13.8 -> 9.6 us,
 // operator of 256^3 845 -> 484 us (66% of the FP32 pipe's rate), of 1024^2 98 us.
 constexpr int kSlice = 32;  // contraction slices of a split, and their parts, start at multiples of this
-
-__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  float4 v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(r)
-               : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 
 __device__ __forceinline__ void store4(float* p, float4 v, int left, bool vec) {
   if (left >= 4 && vec) {
@@ -280,7 +265,8 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
     for (int i = 0; i < R; ++i)
 #pragma unroll
       for (int h = 0; h < CG; ++h) *reinterpret_cast<float4*>(s_mem + row_of(i) * BN + 32 * h + 4 * tx) = quad(i, h);
-    cluster_sync_all();
+    cluster_arrive();
+    cluster_wait();
     const int rows = BM / ks;
     const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(s_mem));
     for (int e = tid; e < rows * (BN / 4); e += THREADS) {
@@ -296,7 +282,8 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
       }
       if (m0 + m < M) store4(Cm + (m0 + m) * X.ldc + n0 + n, v, N - (n0 + n), vc);
     }
-    cluster_sync_all();  // peers have read this block's tile before it leaves
+    cluster_arrive();
+    cluster_wait();  // peers have read this block's tile before it leaves
   }
   if (!P.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

@@ -19,8 +19,9 @@
 // Per CTA: warp 0 / lane 0 issues TMA loads (128B-swizzled tiles, no multicast)
 // into a STAGES-deep ring guarded by mbarriers (the first loads leave before the
 // accumulator is allocated), warp 1 / lane 0 issues the MMAs and releases ring slots
-// with tcgen05.commit, then all four warps drain the accumulator (tcgen05.ld, one
-// lane quarter per warp) into a shared [BN][128] tile that one TMA store writes to F.
+// with tcgen05.commit, then all eight warps drain the accumulator (tcgen05.ld, two warps to
+// a lane quarter, alternate 32-column chunks) into a shared [BN][128] tile, each chunk of
+// which one TMA store writes to F.
 // Small problems split the contraction over ksplit CTAs, CTA `rank` contracting its k-range.
 // Where F is stored with TMA and read by the TMA-fed 2-D march, the partial tiles stay in slots of F,
 // [rank][axis][node], which the march adds in rank order.  Else (ragged rows, 3-D, varying coefficients) the CTAs of a
@@ -41,6 +42,7 @@
 #include <cstring>
 #include <vector>
 
+#include "cluster_dev.cuh"
 #include "lbm_internal.h"
 #include "tc_dev.cuh"
 
@@ -54,21 +56,6 @@ namespace {
 // into hi + lo
 constexpr int kTileSplitWarps = 6;
 constexpr int kTileThreads = 256;
-
-// four floats of the shared memory of cluster rank `rank` at this block's address `addr`
-__device__ __forceinline__ float4 ld_peer_f4(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  float4 v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(r)
-               : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void peers_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void peers_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 template <int E, int BN, int KS, int KP = 2>
 __device__ __forceinline__ void frac_tc_tile(const TcMaps& maps, const TcParams& P, int block, uint8_t* smem_raw) {
@@ -221,15 +208,15 @@ __device__ __forceinline__ void frac_tc_tile(const TcMaps& maps, const TcParams&
     constexpr int RP = BN / KS;
     r0 = rank * RP;
     r1 = r0 + RP;
-    peers_arrive();
-    peers_wait();
+    cluster_arrive();
+    cluster_wait();
     const uint32_t base = smem_u32(tile);
 #pragma unroll
     for (int e = threadIdx.x; e < RP * (BM / 4); e += kTileThreads) {
       const uint32_t off = 4u * (r0 * BM + 4 * e);
       float4 v[KS];
 #pragma unroll
-      for (int q = 0; q < KS; ++q) v[q] = ld_peer_f4(base + off, q);
+      for (int q = 0; q < KS; ++q) v[q] = ld_cluster_f4(base + off, q);
 #pragma unroll
       for (int q = 1; q < KS; ++q) {
         v[0].x += v[q].x;
@@ -239,7 +226,7 @@ __device__ __forceinline__ void frac_tc_tile(const TcMaps& maps, const TcParams&
       }
       *reinterpret_cast<float4*>(reinterpret_cast<uint8_t*>(tile) + off) = v[0];  // only this CTA reads its own rows
     }
-    peers_arrive();  // this thread is done with the peers' tiles
+    cluster_arrive();  // this thread is done with the peers' tiles
     if (P.tma_store) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncthreads();
@@ -264,7 +251,7 @@ __device__ __forceinline__ void frac_tc_tile(const TcMaps& maps, const TcParams&
       }
     }
   }
-  if (KS > 1 && !slots) peers_wait();  // the peers have read this CTA's tile
+  if (KS > 1 && !slots) cluster_wait();  // the peers have read this CTA's tile
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {

@@ -191,7 +191,6 @@ struct CsSlot {
 cudaError_t launch_collide_stream(const lbm_s* h, const void* f_in, void* f_out, void* C_out,
                                   cudaStream_t s, int tk = 0, const CsSlot* slot = nullptr);
 bool cs_encode_slot(const lbm_s* h, const void* f, const void* F, void* map_f, void* map_F);
-// f = feq(C, F) (with u(x) when the coefficients vary)
 // launch shape of the kernels that take nodes row by row (no 64-bit division per node): blocks of
 // 128 threads, as many rows of short lines as fit
 inline dim3 row_block(const lbm_s* h) {
@@ -204,7 +203,8 @@ inline dim3 row_grid(const lbm_s* h) {
   const long long rows = (long long)h->sp.n[1] * h->sp.n[2];
   return dim3((h->sp.n[0] + b.x - 1) / b.x, (unsigned)std::min<long long>((rows + b.y - 1) / b.y, 65535));
 }
-// f = feq(C, F) into f, C = <1|f>, and the operator's operands of that C
+// f = feq(C, F) into f (with u(x) when the coefficients vary), C = <1|f>, and the operator's operands
+// of that C
 cudaError_t launch_init_state(const lbm_s* h, void* f, cudaStream_t s);
 // G_mu = g_mu(x) C (spatially varying coefficients only)
 cudaError_t launch_scale_fields(const lbm_s* h, cudaStream_t s);
