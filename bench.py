@@ -17,7 +17,8 @@ of the same workload are reported beside it (``forms``), and at N = 1 the other
 named workloads (3-D 256^3, the 64-problem batch, the FP64 64^2 case and the
 inverse problem's loss + gradient) each get an entry in ``workloads`` with their
 own MLUPS, end-to-end MLUPS, rooflines of both kernels and accuracy against an
-oracle sample.
+oracle sample.  The whole record, tens of KB, goes to stderr; stdout has the one line of the
+headline with the rates, times and errors of the rest (``result_line``).
 
 N > 1 runs under torchrun.  The batch workload is partitioned: each rank takes a
 cost-balanced subset of the problems (no collective on the data path).  A single
@@ -635,6 +636,33 @@ def run_reference(args):
     return 0
 
 
+def result_line(line):
+    """The benchmark's one line on stdout, a few KB: the whole record without what belongs to a form or a
+    workload beside the headline (their rates, times and errors stay).  The whole record goes to
+    stderr."""
+    out = dict(line)
+    if line.get("accuracy"):
+        out["accuracy"] = {k: v for k, v in line["accuracy"].items() if k != "by_horizon"}
+
+    def short(ent):
+        keys = ("value", "unit", "ms_per_step", "us_per_lattice_step", "status", "error")
+        row = {k: ent[k] for k in keys if k in ent}
+        if "e2e" in ent:
+            row["e2e"] = ent["e2e"]["value"]
+        err = ent.get("accuracy", {}).get("rel_l2_vs_fp64_oracle")
+        if err is not None:
+            row["rel_l2_vs_fp64_oracle"] = err
+        return row
+
+    if line.get("forms"):
+        out["forms"] = {k: short(v) for k, v in line["forms"].items()}
+    if line.get("workloads"):
+        out["workloads"] = {k: short(v) if "fp32" not in v else
+                            {p: {"value": v[p]["value"], "unit": v["unit"]} for p in ("fp32", "fp64")}
+                            for k, v in line["workloads"].items()}
+    return out
+
+
 def measure_walk(lbm, torch, steps=3, warmup=1):
     """The killed stable-Levy walk (Section 3.1), the paper's Monte-Carlo counterpart: 2^24
     FP32 paths x 200 increments on the [0,1]^2 case of the oracle's walk pin (alpha = (1.5,
@@ -889,7 +917,8 @@ def main():
                         "d2h_bytes_per_step": d2h_bytes},
                 "gpu_launches": gpu_launches, "clocks": clk,
                 "status": lbm.lbm_strerror(rc if rc else warm_status)}
-        print(json.dumps(line))
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(result_line(line)))
     if dist is not None:
         dist.barrier()
         dist.destroy_process_group()
