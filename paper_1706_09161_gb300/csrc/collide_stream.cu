@@ -406,29 +406,28 @@ __device__ __forceinline__ void march_body(const KConst<real>& sp, const real* _
   const int tid = threadIdx.x + 32 * threadIdx.y, lane = threadIdx.x;
   const int x0 = bx * TXX, y0 = by * TYY;
 
-  // the node this thread collides every plane, and where its movers go
-  int gx, gy, sx, sy;
-  const bool owner = tid < TXX * TYY;
-  int side = -1;  // ring: which of the tile's sides this node borders (left, right, below, above)
+  // the node this thread collides every plane, and where its movers go.  (The 3-D FP32 marches have 48
+  // registers: a variable for the ring's side, kept through the planes, made the grouped one spill, 4
+  // problems of 48^3 65 -> 80 us.)
+  int gx, gy;
+  const bool owner = TXX == 32 ? threadIdx.y < TYY : tid < TXX * TYY;
+  const int ring = tid - TXX * TYY;
   if (owner) {
-    gx = x0 + tid % TXX;
-    gy = y0 + tid / TXX;
-  } else if (const int ring = tid - TXX * TYY; ring < 2 * TYY) {
-    side = ring / TYY;
-    gx = side ? x0 + TXX : x0 - 1;
+    gx = x0 + (TXX == 32 ? lane : tid % TXX);
+    gy = y0 + (TXX == 32 ? (int)threadIdx.y : tid / TXX);
+  } else if (ring < 2 * TYY) {
+    gx = ring / TYY ? x0 + TXX : x0 - 1;
     gy = y0 + ring % TYY;
   } else {
-    const int row = ring - 2 * TYY;
-    side = 2 + row / TXX;  // 4 and beyond: threads past the ring, idle
-    gx = x0 + row % TXX;
-    gy = side == 2 ? y0 - 1 : y0 + TYY;
+    gx = x0 + (ring - 2 * TYY) % TXX;
+    gy = ring < 2 * TYY + TXX ? y0 - 1 : y0 + TYY;
   }
-  sx = gx - x0 + 1;
-  sy = gy - y0 + 1;
+  const int sx = gx - x0 + 1, sy = gy - y0 + 1;
   // programmatic dependent launch: the operator's F (and the previous step's f) must be
   // complete before any load
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const bool in_xy = side < 4 && gx >= 0 && gx < n0 && gy >= 0 && gy < n1;
+  constexpr bool spare = march_warps(TXX, TYY) * 32 > TXX * TYY + 2 * (TXX + TYY);  // threads past the ring, idle
+  const bool in_xy = (!spare || ring < 2 * (TXX + TYY)) && gx >= 0 && gx < n0 && gy >= 0 && gy < n1;
   const long long col = gx + (long long)n0 * gy;
   bool bad = false;
   SumAcc<real> macc;
@@ -454,10 +453,15 @@ __device__ __forceinline__ void march_body(const KConst<real>& sp, const real* _
     } else {
       real h[Q];
       collide_at<real, D, MRT, FLD>(sp, f_in, F, in_xy, col + z * plane, h, fp);
-      if (side == 0) s_m[buf][0][sy][sx] = h[1];       // moves +x into the tile
-      else if (side == 1) s_m[buf][1][sy][sx] = h[2];  // moves -x into the tile
-      else if (side == 2) s_m[buf][2][sy][sx] = h[3];  // moves +y into the tile
-      else if (side == 3) s_m[buf][3][sy][sx] = h[4];  // moves -y into the tile
+      // the ring: left and right columns, rows below and above, each moving into the tile
+      if (ring < 2 * TYY) {
+        if (ring < TYY) s_m[buf][0][sy][sx] = h[1];
+        else s_m[buf][1][sy][sx] = h[2];
+      } else if (ring < 2 * TYY + TXX) {
+        s_m[buf][2][sy][sx] = h[3];
+      } else if (!spare || ring < 2 * (TXX + TYY)) {
+        s_m[buf][3][sy][sx] = h[4];
+      }
     }
     __syncthreads();
     if (owner && in_xy) {
@@ -1880,7 +1884,7 @@ collide_stream_batch_kernel(const BatchCS* __restrict__ tab, const int2* __restr
   }
   __syncthreads();
   float* fo = const_cast<float*>(e.f[parity ^ 1]);
-  float* Co = keep_C ? e.C : nullptr;
+  float* Co = SPLIT == 0 || keep_C ? e.C : nullptr;
   if constexpr (D == 2) {
     const int item = pb.y * kStripWarps + (tid >> 5);
     if (item < e.items) {
