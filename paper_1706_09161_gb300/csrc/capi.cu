@@ -320,7 +320,7 @@ void free_all(lbm_s* h) {
 // from the collide-stream kernel itself)
 bool pdl_fits(const lbm_s* h) {
   if (h->is_batch()) return false;
-  if (!h->tc) return lbm::cs_one_wave(h) && lbm::simt_one_wave(h);  // SIMT operator
+  if (!h->tc) return (h->elem == 4 || lbm::simt64_short(h)) && lbm::cs_one_wave(h) && lbm::simt_one_wave(h);  // SIMT operator
   const bool adjacent = lbm::bf16_parts(h->prm.precision) || lbm::cs_writes_T(h);
   return adjacent && !(h->fld.on && h->d == 3) && lbm::cs_one_wave(h) && lbm::tc_one_wave(h);
 }

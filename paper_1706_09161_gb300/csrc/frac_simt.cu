@@ -593,6 +593,18 @@ bool simt_one_wave(const lbm_s* h) {
   });
 }
 
+// Blocks that are launched early go to the SMs that the kernel before leaves first, several to an SM.
+// Where an SM's share of the FP64 operator (two FMAs per clock) is some 4 us, the launch gap that this
+// hides is worth more; beyond, the pile is the longer (step in us, launched early / not; runs of
+// captured graphs, then of single launches: 24^3 7,700 FMAs per SM 21.9 / 22.4 and 22.4 / 27.9, 96^2
+// 12,300 10.7 / 10.1 and 10.0 / 14.6, 32^3 24,600 33.0 / 27.4 and 33.5 / 32.0, 175^2 45.8 / 34.8 and
+// 37.8 / 39.1, 256^2 330 / 83 and 144 / 88).
+bool simt64_short(const lbm_s* h) {
+  const int T = tile64(h);
+  const long long per_sm = (count_tiles(h, T, T) + device_sms() - 1) / device_sms();
+  return per_sm * T * T * std::max(h->sp.n[0], std::max(h->sp.n[1], h->sp.n[2])) <= 16384;
+}
+
 long long simt_blocks(const lbm_s* h) {
   if (h->elem == 8) return count_tiles(h, tile64(h), tile64(h));
   return with_tile32(h, h->simt_ks, [&](auto G) { return count_tiles(h, G.BM, G.BN) * h->simt_ks; });

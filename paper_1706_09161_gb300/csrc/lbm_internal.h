@@ -174,6 +174,7 @@ int simt_ksplit(const lbm_s* h);
 int simt_sub(const lbm_s* h);  // accumulation chains per slice of the built-in split
 // the FP32 SIMT operator's grid is resident at once (programmatic dependent launch)
 bool simt_one_wave(const lbm_s* h);
+bool simt64_short(const lbm_s* h);  // an FP64 operator short enough to be launched early
 long long simt_blocks(const lbm_s* h);  // blocks of the SIMT operator's launch
 // tensor-core split-precision fractional operator (tcgen05); returns
 // cudaErrorNotSupported when the handle's shape is not covered
