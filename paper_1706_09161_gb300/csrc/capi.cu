@@ -553,6 +553,7 @@ static int create_problem(const lbm_params* prm, const double* C0_host, void* st
   if ((rc = upload_weights(h, dv.h, &Kall))) return fail(rc);
   if (lbm::bf16_parts(prm->precision) || prm->precision == LBM_FP32_TF32SPLIT) {
     if ((rc = lbm::tc_prepare(h, Kall, batched ? 128 : 0, batched ? 1 : 0))) return fail(rc);
+    h->tc_built_in = !batched;
     h->launches_per_step = 2;  // (lbm_launches_per_step counts the tf32 regrouping launches)
   } else {
     h->launches_per_step = 2;  // one SIMT operator launch over every axis, one collide-stream
@@ -931,6 +932,7 @@ namespace {
 struct TuneCfg {
   int bn, ks, persist, chunk;  // (ks: 0 is the built-in split of the FP32 SIMT operator)
   int fused = 0;
+  bool built_in = false;       // the tensor-core plan is the built-in one
 };
 
 // FP32 SIMT operator of a single problem: contraction split ks (1, 2, 4 or 8, at most the
@@ -961,6 +963,7 @@ int set_cfg(lbm_s* h, const TuneCfg& c) {
   if (h->tc) {
     h->fused = false;
     if ((rc = lbm::tc_replan(h, c.bn, c.ks, c.persist))) return rc;
+    h->tc_built_in = c.built_in;
     lbm::cs_release(h);
     if ((rc = lbm::cs_prepare(h))) return rc;
     h->pdl = pdl_fits(h);
@@ -987,6 +990,7 @@ int set_cfg(lbm_s* h, const TuneCfg& c) {
 int apply_cfg(lbm_s* h, const TuneCfg& c) {
   TuneCfg old{0, h->simt_built_in ? 0 : h->simt_ks, 0, lbm::cs_chunk_of(h), h->fused ? 1 : 0};
   if (!h->is_batch() && h->tc) lbm::tc_config(h, &old.bn, &old.ks, &old.persist);
+  old.built_in = h->tc_built_in;
   const int rc = set_cfg(h, c);
   drop_graphs(h);
   if (rc && h->is_batch()) h->cs_chunk = old.chunk;  // (its tables are still the old ones)
@@ -1038,6 +1042,7 @@ int lbm_configure(lbm_t h, int bn, int ks, int persist, int chunk, int fused) {
   TuneCfg c{0, 0, 0, chunk, fused ? 1 : 0};  // (chunk 0 is the built-in choice to every launch)
   if (!h->is_batch() && h->tc) {
     lbm::tc_config(h, &c.bn, &c.ks, &c.persist);
+    c.built_in = h->tc_built_in && bn <= 0;
     if (bn > 0) {
       c.bn = bn;
       c.ks = ks > 0 ? ks : 1;
@@ -1063,6 +1068,7 @@ int lbm_autotune(lbm_t h, int nsteps, char* desc, int desc_len) {
   const int set = lbm::cs_chunk_of(h);
   TuneCfg cur{0, 0, 0, set > 0 ? set : lbm::cs_chunk_default(h), h->fused ? 1 : 0};
   if (!h->is_batch() && h->tc) lbm::tc_config(h, &cur.bn, &cur.ks, &cur.persist);
+  cur.built_in = h->tc_built_in;
   const bool simt32 = !h->is_batch() && !h->tc && h->elem == 4;  // FP32 SIMT operator
   if (simt32) cur.ks = h->simt_built_in ? 0 : h->simt_ks;
   // candidate chunks
@@ -1285,7 +1291,8 @@ static int rebuild_fields(lbm_s* h) {
   }
   if (h->tc) {  // where the partial sums of a split contraction are added depends on the march
     int bn, ks, persist;
-    lbm::tc_config(h, &bn, &ks, &persist);
+    if (h->tc_built_in) lbm::tc_built_in_plan(h, &bn, &ks, &persist);
+    else lbm::tc_config(h, &bn, &ks, &persist);
     if ((rc = lbm::tc_replan(h, bn, ks, persist, false))) return rc;
     lbm::cs_release(h);
     if ((rc = lbm::cs_prepare(h))) return rc;

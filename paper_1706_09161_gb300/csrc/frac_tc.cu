@@ -808,6 +808,82 @@ int tc_set_weights(lbm_s* h, const std::vector<std::vector<double>>& K) {
   return LBM_OK;
 }
 
+namespace {
+
+// Clusters of KS CTAs of the per-tile operator, one CTA to an SM, that are resident at once: a cluster
+// lies within one GPC, whose SMs are not a multiple of it, so fewer than SMs / KS.  Asked of the
+// driver once per device.
+template <int KS>
+int clusters_resident() {
+  static std::atomic<int> known[64];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if ((n = known[dev & 63].load(std::memory_order_relaxed)) > 0) return n - 1;
+  auto kernel = frac_tc_kernel<2, 128, KS, 2>;
+  const int smem = (int)Cfg<2, 128, KS, 2>::SMEM;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(KS * device_sms(), 1, 1);
+  cfg.blockDim = dim3(kTileThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = KS;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) return 0;
+  known[dev & 63].store(n + 1, std::memory_order_relaxed);
+  return n;
+}
+
+}  // namespace
+
+// The built-in plan: column tiles of 128 (an M = 128 MMA costs the same for any N <= 128)
+// or 256 when that still fills the GPU; small problems split the contraction over up
+// to 8 CTAs per tile so that about one CTA per SM is busy, where the CTAs of a tile are a cluster
+// no more than leaves every cluster resident (18 tiles of 300^2 with coefficients per node, tf32x3:
+// eight CTAs to a cluster take two waves, operator 17.1 us; 30 tiles of 64 columns split four ways 9);
+// more tiles than SMs: the persistent
+// kernel (128-column tiles, no split; step, per tile / persistent: 64^3 bf16x6 23.5 / 20.4 us,
+// 64 x 64 x 90 30.2 / 22.7, tf32x3 32.4 / 24.7, 1100^2 bf16x6 63.6 / 63.2; 130 x 40 x 50, where
+// half the lines are padding, 36.1 / 36.9), the deep form of it where the per-tile plan would have
+// 128-column tiles with four accumulator regions; batched handles always use it
+void tc_built_in_plan(const lbm_s* h, int* bn_out, int* ks_out, int* persist_out) {
+  const int kSMs = device_sms();
+  const TcPlan* p = h->tc;
+  const bool clusters = !(h->d == 2 && h->sp.n[0] % 4 == 0 && !h->fld.on);  // as tc_replan
+  int bn = (p->kparts == 2 && tc_count_tiles(h, 256) >= kSMs) ? 256 : 128;
+  const int kbmin = tc_kbmin(h);
+  auto split = [&](long long tiles) {
+    int k = 1;
+    auto fits = [&](int ks) {
+      return !clusters || tiles <= (ks == 2 ? clusters_resident<2>() : ks == 4 ? clusters_resident<4>() : clusters_resident<8>());
+    };
+    while (k * 2 <= 8 && k * 2 <= kbmin && tiles * k * 2 <= kSMs && fits(k * 2)) k *= 2;
+    return k;
+  };
+  int ks = split(tc_count_tiles(h, bn));
+  // 64-column tiles where they put more CTAs to work (small and ragged grids; measured:
+  // 256^2 bf16x6 step 8.7 us with 128 columns, 8.1 with 64, 301 x 203 10.6 and 9.9), and where no
+  // line is longer than 64 columns (50^2 tf32x3 12.4 and 10.8, 48^2 6.9 and 6.5)
+  const long long t64 = tc_count_tiles(h, 64);
+  const long long t128 = tc_count_tiles(h, 128);
+  if (bn == 128 && t64 * split(t64) <= kSMs && (t64 == t128 || t64 * split(t64) > t128 * ks)) {
+    bn = 64;
+    ks = split(t64);
+  }
+  int persist = 0;
+  if (tc_count_tiles(h, PBN) > kSMs) {
+    persist = bn == PBN && tc_count_tiles(h, PBN) < 2 * kSMs ? 2 : 1;
+    bn = PBN;
+    ks = 1;
+  }
+  *bn_out = bn;
+  *ks_out = ks;
+  *persist_out = persist;
+}
+
 // Allocate the split operands, split K_mu on the host, encode the tensor maps.
 int tc_prepare(lbm_s* h, const std::vector<std::vector<double>>& K, int force_bn, int force_ks) {
   TcPlan* p = new (std::nothrow) TcPlan();
@@ -870,40 +946,13 @@ int tc_prepare(lbm_s* h, const std::vector<std::vector<double>>& K, int force_bn
   }
   if (int rc = tc_set_weights(h, K)) return rc;
 
-  // default plan: column tiles of 128 (an M = 128 MMA costs the same for any N <= 128)
-  // or 256 when that still fills the GPU; small problems split the contraction over up
-  // to 8 CTAs per tile so that about one CTA per SM is busy; more tiles than SMs: the persistent
-  // kernel (128-column tiles, no split; step, per tile / persistent: 64^3 bf16x6 23.5 / 20.4 us,
-  // 64 x 64 x 90 30.2 / 22.7, tf32x3 32.4 / 24.7, 1100^2 bf16x6 63.6 / 63.2; 130 x 40 x 50, where
-  // half the lines are padding, 36.1 / 36.9), the deep form of it where the per-tile plan would have
-  // 128-column tiles with four accumulator regions; batched handles always use it
-  const int kSMs = device_sms();
-  int bn = (p->kparts == 2 && tc_count_tiles(h, 256) >= kSMs) ? 256 : 128;
-  const int kbmin = tc_kbmin(h);
-  auto split = [&](long long tiles) {
-    int k = 1;
-    while (k * 2 <= 8 && k * 2 <= kbmin && tiles * k * 2 <= kSMs) k *= 2;
-    return k;
-  };
-  int ks = split(tc_count_tiles(h, bn));
-  // 64-column tiles where they put more CTAs to work (small and ragged grids; measured:
-  // 256^2 bf16x6 step 8.7 us with 128 columns, 8.1 with 64, 301 x 203 10.6 and 9.9), and where no
-  // line is longer than 64 columns (50^2 tf32x3 12.4 and 10.8, 48^2 6.9 and 6.5)
-  const long long t64 = tc_count_tiles(h, 64);
-  const long long t128 = tc_count_tiles(h, 128);
-  if (bn == 128 && t64 * split(t64) <= kSMs && (t64 == t128 || t64 * split(t64) > t128 * ks)) {
-    bn = 64;
-    ks = split(t64);
-  }
-  int persist = 0;
+  int bn, ks, persist;
   if (force_bn > 0) {
     bn = force_bn;
     ks = std::max(1, force_ks);
     persist = force_bn == PBN && ks == 1 ? 1 : 0;
-  } else if (tc_count_tiles(h, PBN) > kSMs) {
-    persist = bn == PBN && tc_count_tiles(h, PBN) < 2 * kSMs ? 2 : 1;
-    bn = PBN;
-    ks = 1;
+  } else {
+    tc_built_in_plan(h, &bn, &ks, &persist);
   }
   return tc_replan(h, bn, ks, persist);
 }

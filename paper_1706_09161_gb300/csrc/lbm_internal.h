@@ -128,6 +128,7 @@ struct lbm_s {
   bool mass_valid = false;
   double mass_limit = 0.0;
   lbm::TcPlan* tc = nullptr;           // split-precision tensor-core operator, if used
+  bool tc_built_in = false;            // its plan is the built-in one, not one that was asked for
   void* cs_plan = nullptr;             // TMA-fed 3-D collide-stream (tensor maps), if used
   // batch of independent problems: one sub-handle per problem (each owns its buffers)
   std::vector<lbm_s*> subs;
@@ -244,6 +245,8 @@ int tc_prepare(lbm_s* h, const std::vector<std::vector<double>>& K, int force_bn
 // combination the kernels do not cover; the plan before stays after an error).  Captured graphs
 // must be dropped afterwards.
 int tc_replan(lbm_s* h, int bn, int ks, int persist, bool must_grow = true);
+// the operator plan of a new handle, or of one whose march reads F as this one's does now
+void tc_built_in_plan(const lbm_s* h, int* bn, int* ks, int* persist);
 long long tc_count_tiles(const lbm_s* h, int bn);  // output tiles of bn columns, all axes
 int tc_kbmin(const lbm_s* h);                      // fewest contraction blocks of any axis
 void tc_config(const lbm_s* h, int* bn, int* ks, int* persist);

@@ -39,3 +39,24 @@ def test_persistent_plan_sums_as_the_per_tile_plan(L, grid, kinds):
             a.step(3)
             b.step(3)
             assert np.array_equal(a.f(), b.f()), kind
+
+
+# clusters of eight CTAs fill fewer SMs than there are, and 18 tiles would take two waves of them: the
+# built-in plan of ragged rows, and of varying coefficients on aligned ones, is 64 columns split four ways
+@pytest.mark.parametrize("grid,fields", [((301, 300), False), ((300, 301), True)])
+def test_built_in_clusters_are_resident(L, grid, fields):
+    rng = np.random.default_rng(2201)
+    pb = W.random_problem(rng, 2, "mrt", grid)
+    C0 = W.random_field(rng, grid)
+    coeff = W.smooth_fields(np.random.default_rng(5), grid, "mrt", D0=0.03, g_amp=0.2, u_amp=0.03)
+    with L.Lattice(pb, C0, "tf32split") as a, L.Lattice(pb, C0, "tf32split") as b:
+        b.configure(64, 4, 0, 0, 0)
+        for lat in (a, b):
+            if fields:
+                lat.set_fields(**coeff)
+            lat.reset()
+        for mu in range(2):
+            assert np.array_equal(a.F(mu), b.F(mu)), mu
+        a.set_fields()  # (constant coefficients again: the plan of a new handle)
+        with L.Lattice(pb, C0, "tf32split") as new:
+            assert np.array_equal(a.F(0), new.F(0))
