@@ -295,7 +295,8 @@ frac_simt32_kernel(const __grid_constant__ GemmPlan P) {
 // block; tiles of T x T outputs, T = 32 (2 x 2 per thread), 16 (1 each) or 8 (1 each, four
 // thread groups taking a quarter of each contraction slice).  Measured against tiles of 64 and
 // 32 alone: operator of 64^2 (8 blocks of 32 x 32 before, 128 of 8 x 8 now) 23 -> 7 us with the
-// launch, of 80^3 (each side of 80 padded to 128 before) 409 -> 246 us, 79% of the FP64 pipe.
+// launch, of 80^3 (each side of 80 padded to 128 before) 409 -> 207 us, 95% of the FP64 pipe
+// (246 while whole rounds of 32 contraction steps were multiplied, 450^2 369 for 357).
 // FP32 (T = 32): the unsplit operator of small grids, batch members above all, is a chain of load
 // latencies in too few blocks to hide them; the 256 threads here have four times the loads in
 // flight of the packed kernel's 64 (operator and march of 3 problems of 224^2: 65 us per step with
@@ -383,9 +384,11 @@ frac_plain_kernel(const __grid_constant__ GemmPlan P) {
     }
     const bool more = k0 + BK < K;
     if (more) fetch(k0 + BK);
+    // (nothing past the end is multiplied: half a round, or a group's share of it)
 #pragma unroll
     for (int q = 0; q < PK; ++q) {
       const int kk = grp * PK + q;
+      if (q % 16 == 0 && k0 + kk >= K) break;
       real av[TR], bv[TR];
 #pragma unroll
       for (int i = 0; i < TR; ++i) av[i] = As[buf][ty * TR + i][kk];
