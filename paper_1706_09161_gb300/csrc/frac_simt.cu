@@ -502,6 +502,10 @@ auto with_tile32(const lbm_s* h, int ks, const F& f) {
     const bool sub = h->simt_sub > 1;
     if (ks == 1 && count_tiles(h, 32, 32) <= 2LL * device_sms())
       return sub ? f(PlainCfg<float, 32, true>{}) : f(PlainCfg<float, 32>{});
+    // (several chains take 127 registers in rounds of 32: beyond six blocks per SM they no longer spread
+    // evenly, 320^2 with 5.3 of them 11.8 us per step against 12.5 in rounds of 16, 352^2 with 6.4 19.6
+    // against 13.2)
+    if (sub && count_tiles(h, 32, 32) * ks > 6LL * device_sms()) return f(F32Cfg<1, 1, 8, 16, true>{});
     if (sub) return f(F32Cfg<1, 1, 8, 32, true>{});
     return ks > 1 ? f(F32Cfg<1, 1, 8, 32>{}) : f(F32Cfg<1, 1, 8, 64>{});
   }
