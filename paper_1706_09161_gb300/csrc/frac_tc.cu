@@ -853,12 +853,16 @@ void tc_built_in_plan(const lbm_s* h, int* bn_out, int* ks_out, int* persist_out
   const int kSMs = device_sms();
   const TcPlan* p = h->tc;
   const bool clusters = !(h->d == 2 && h->sp.n[0] % 4 == 0 && !h->fld.on);  // as tc_replan
+  // a cluster's launch and barriers cost more than the split of a line of at most 64 saves (48^2 tf32x3
+  // with coefficients per node 10.9 us per step split in two, 10.4 whole), and its k-steps have a
+  // region each as it is
+  const int longest = std::max(h->sp.n[0], std::max(h->sp.n[1], h->sp.n[2]));
   int bn = (p->kparts == 2 && tc_count_tiles(h, 256) >= kSMs) ? 256 : 128;
   const int kbmin = tc_kbmin(h);
   auto split = [&](long long tiles) {
     int k = 1;
     auto fits = [&](int ks) {
-      return !clusters || tiles <= (ks == 2 ? clusters_resident<2>() : ks == 4 ? clusters_resident<4>() : clusters_resident<8>());
+      return !clusters || (longest > 64 && tiles <= (ks == 2 ? clusters_resident<2>() : ks == 4 ? clusters_resident<4>() : clusters_resident<8>()));
     };
     while (k * 2 <= 8 && k * 2 <= kbmin && tiles * k * 2 <= kSMs && fits(k * 2)) k *= 2;
     return k;
