@@ -554,8 +554,10 @@ TRAFFIC_CAPTURES = {
 }
 KERNEL_SOURCES = {
     "fractional_operator": ["paper_1706_09161_gb300/csrc/frac_tc.cu", "paper_1706_09161_gb300/csrc/tc_dev.cuh",
+                            "paper_1706_09161_gb300/csrc/cluster_dev.cuh",
                             "paper_1706_09161_gb300/csrc/lbm_internal.h"],
     "collide_stream": ["paper_1706_09161_gb300/csrc/collide_stream.cu", "paper_1706_09161_gb300/csrc/tc_dev.cuh",
+                       "paper_1706_09161_gb300/csrc/two_float.cuh",
                        "paper_1706_09161_gb300/csrc/lbm_internal.h"],
 }
 

@@ -377,6 +377,8 @@ int lbm_get_stream(lbm_t h, void** stream);
  *   ms[1] = fused collide/stream/walls/moment.
  * All steps are queued before one synchronisation, so the intervals exclude the host's
  * submission of each launch.  Divide by nsteps for the mean duration per launch.
+ * Every step stores C, as the last step of an lbm_step call does (the ones before it need not
+ * on the tensor-core forms).
  * LBM_EINVAL for nsteps outside that range.  Synchronises. */
 int lbm_profile(lbm_t h, int nsteps, double* ms);
 

@@ -24,13 +24,14 @@
 // which one TMA store writes to F.
 // Small problems split the contraction over ksplit CTAs, CTA `rank` contracting its k-range.
 // Where F is stored with TMA and read by the TMA-fed 2-D march, the partial tiles stay in slots of F,
-// [rank][axis][node], which the march adds in rank order.  Else (ragged rows, 3-D, varying coefficients) the CTAs of a
-// tile form a cluster that adds the partial tiles in rank order through distributed shared
-// memory, each CTA summing and storing its share of the rows.  Either way the result does not
-// depend on timing.  (Measured: 301 x 203 bf16x6 step 13.5 us with slots, 10.6 with clusters,
+// [rank][axis][node], which the march adds in rank order.  Else (ragged rows, 3-D, varying
+// coefficients) the CTAs of a tile form a cluster that adds the partial tiles in rank order
+// through distributed shared memory, each CTA summing and storing its share of the rows.
+// Either way the result does not depend on timing.  (Measured: 301 x 203 bf16x6 step 13.5 us with slots, 10.6 with clusters,
 // whose plain stores and reads of F are a quarter; 512^2 12.4 and 13.2: a cluster's four CTAs
-// cannot start on the SMs that the previous kernel leaves one by one.)  Problems with many tiles use the persistent kernel further
-// down (two TMEM accumulators, epilogue overlapping the next tile).  Every mbarrier wait is
+// cannot start on the SMs that the previous kernel leaves one by one.)  Problems with many
+// tiles use the persistent kernel further down (two TMEM accumulators, the epilogue
+// overlapping the next tile, or one of four regions).  Every mbarrier wait is
 // bounded by a 2 s %globaltimer budget; a wait that gives up sets bit 2 of the
 // handle's error flag and the CTA skips the rest of its work and releases TMEM.
 #include <cuda.h>
@@ -862,7 +863,9 @@ void tc_built_in_plan(const lbm_s* h, int* bn_out, int* ks_out, int* persist_out
   auto split = [&](long long tiles) {
     int k = 1;
     auto fits = [&](int ks) {
-      return !clusters || (longest > 64 && tiles <= (ks == 2 ? clusters_resident<2>() : ks == 4 ? clusters_resident<4>() : clusters_resident<8>()));
+      if (!clusters) return true;
+      return longest > 64 && tiles <= (ks == 2 ? clusters_resident<2>() : ks == 4 ? clusters_resident<4>()
+                                                                                   : clusters_resident<8>());
     };
     while (k * 2 <= 8 && k * 2 <= kbmin && tiles * k * 2 <= kSMs && fits(k * 2)) k *= 2;
     return k;

@@ -622,7 +622,7 @@ class Batch:
         return lbm_mass(self.h, prob)
 
     def autotune(self, nsteps: int = 64) -> str:
-        """Time the candidate tile rows per collide-stream block and keep the fastest."""
+        """Time the candidate collide-stream chunks (row pairs per warp) and keep the fastest."""
         return lbm_autotune(self.h, nsteps)
 
     def save(self) -> np.ndarray:
