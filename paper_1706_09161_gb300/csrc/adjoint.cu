@@ -183,7 +183,7 @@ __device__ __forceinline__ void warp_accumulate(const double* val, double* __res
 // gradients.  Bound by memory latency and the FP64 pipe; the sum lambda_f + lambda_C of the
 // later step is formed on the fly for the node and its neighbours (cached reads), which saves
 // a pass over the populations, and the FP64 work is three operations per summed value.
-// 256^2, single cold-cache launches: 14.5 us and 3.4 us for the pass, now 8.4 us.
+// 256^2, single cold-cache launches: 14.5 us and 3.4 us for the pass, now 9.9 us.
 constexpr int kStepThreads = 128;
 
 template <typename real, int D>

@@ -1025,8 +1025,8 @@ collide_stream_march_kernel(const KConst<real> sp, const real* __restrict__ f_in
 // three planes ahead of the plane being collided.  Nodes outside the domain arrive as zeros
 // (TMA out-of-bounds fill), which the collision maps to zero movers, exactly as the plain march
 // treats them.  Measured against one node per thread (608 threads, two barriers per plane, two
-// planes ahead, 410 instructions per node) with its z chunks: 256^3 bf16x6 231 -> 209 us (1317 MB,
-// 93% of the measured copy rate), tf32x3 247 -> 229, 160 x 128 x 100 43 -> 33.
+// planes ahead, 410 instructions per node) with its z chunks: 256^3 bf16x6 231 -> 209 us (1315 MB
+// with C, which a call's last step stores: 93% of the measured copy rate), tf32x3 247 -> 227, 160 x 128 x 100 43 -> 33.
 constexpr int TW = TX + 8, TH = TY + 2;  // staged window: x from x0 - 4, y from y0 - 1
 constexpr int TMA_STAGES = 3;
 constexpr uint32_t TMA_F_BYTES = 7u * TH * TW * 4;   // D3Q7 populations

@@ -833,7 +833,10 @@ int clusters_resident() {
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();  // (no split then)
+    return 0;
+  }
   known[dev & 63].store(n + 1, std::memory_order_relaxed);
   return n;
 }
